@@ -1,0 +1,40 @@
+"""Kernels at the edges of their tiles, on the GPU: lengths around the pieces a CTA or a warp takes, remainders of their
+unrolled loops, the smallest and largest sizes, against NumPy arithmetic on the same values."""
+import numpy as np
+import pytest
+
+from tests.gpu_common import dev_vec, need_gpu
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Solver():
+    need_gpu()
+    from paper_2506_18408_gb300 import Solver
+
+    return Solver
+
+
+def _unit(n, seed):
+    v = np.random.default_rng(seed).standard_normal(n)
+    return dev_vec(v / np.linalg.norm(v))
+
+
+# z = B y: pieces of 512 (FP64) or 1024 (FP32, BF16) rows of a block, four columns at a time
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "bf16"])
+@pytest.mark.parametrize("n,m,block_rows", [(33, 1, 0), (511, 3, 512), (512, 4, 512), (513, 5, 512), (1025, 7, 8192),
+                                            (3 * 1024 + 1, 9, 1056), (8191, 34, 8192)])
+def test_correction_is_the_basis_times_y(Solver, precision, n, m, block_rows):
+    A = workloads.convdiff(n, (30.0,))
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, precision=precision, block_rows=block_rows)
+    z, k, _, B, y = sv.inner_cycle(_unit(n, n), m=m, s=max(32, 4 * m) if n > 256 else 32, k=2)
+    B, y, z = B[:k].cpu().numpy(), y.cpu().numpy(), z.cpu().numpy()
+    size = np.abs(y) @ np.abs(B)
+    # FP64: k products and sums, the coefficients' and the exported basis's own roundings.  FP32 pairs: two-term
+    # coefficients (2^-47 each) and a low part whose k sums each round to 2^-24 of at most k 2^-23 of the whole.
+    bound = (2 * k + 8) * 2.0 ** -53 if precision == "fp64" else (k + 8) ** 2 * 2.0 ** -46
+    assert np.all(np.abs(z - y @ B) <= bound * size + 1e-300)
+    sv.close()

@@ -132,7 +132,7 @@ struct sfgmres_ctx {
     uint16_t* ent = nullptr;
 
     // workspaces
-    DevBuf U, W, sigma, normpart, hpart, cpart, C, Q, Qt, R, d, e, c0, rho, y, coef, hco, cyc;
+    DevBuf U, W, sigma, normpart, hpart, cpart, C, Q, R, d, e, c0, rho, y, coef, hco, cyc;
     DevBuf Vb, Z, nu, Wo, opart, npart, npart2, h1, h2, H, cs, sn, g, yo, est_hist, ffom_hist, ires_hist, rho_hist,
         k_hist, reason_hist,
         ost;
@@ -251,7 +251,7 @@ int choose_vec(int64_t, int, int maxlen) { return maxlen <= 16 ? 1 : 0; }
 // on those stragglers (measured on 128^3: 137 us per step with 304 blocks, 112 us with 288).  The FP32 and BF16
 // inner kernels are short enough that the QR does not slow them, and all SMs serve them best.
 int single_block_rows(int n, int sms, int prec) {
-    if (prec == 0 && sms > 2 * kQrCluster) sms -= kQrCluster;
+    if (prec == 0 && sms > 2 * kQrSms) sms -= kQrSms;
     int q = 1, b = 32;
     for (;;) {
         const int64_t per = ((int64_t)n + (int64_t)sms * q - 1) / ((int64_t)sms * q);
@@ -288,19 +288,12 @@ void set_list_geometry(sfgmres_ctx* h) {
     ++h->geo_ver;
 }
 
-// CTAs per problem of the sketched-QR update.  Small sketches of few problems whose inner step leaves an SM with at
-// most one of its CTAs (nblk <= sms): 0, the single-CTA kernel (512 threads; its reductions cost shared-memory
-// barriers instead of cluster barriers and distributed-shared-memory exchanges).  It needs a large share of an SM's
-// registers and shared memory, so beside an inner step that fills every SM it would wait for the step to end (the
-// random Zipf workload, s = 240: 335 -> 361 ms per FP64 solve).  Otherwise a cluster of small CTAs (they fit beside
-// the step's) with as many CTAs as the batch leaves room for: the update is bound by the latency of its reads, which
-// more SMs hide better.
-int qr_cluster_for(int P, int s, int m, int nblk, int sms) {
-    if (P <= kQrSmallProblems && qr_small_fits(s, m) && nblk <= sms) return 0;  // one CTA per problem
-    if (P <= 16) return kQrCluster;
-    if (P <= 32) return 4;
-    if (P <= 64) return 2;
-    return 1;
+// Shared memory left on an SM beside the inner step's CTAs (one or two of them, by the number of row blocks; 8 KB each
+// for their static shared memory and the reserve), for a sketched-QR CTA to run there at the same time.
+size_t qr_smem_left(int nblk, int sms, size_t step_smem) {
+    const size_t per_sm = (nblk > sms) ? 2 : 1;
+    const size_t used = per_sm * (step_smem + 8 * 1024), all = 226 * 1024;
+    return used < all ? all - used : 0;
 }
 
 // ---- CSR validation on the device ----
@@ -861,8 +854,8 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->hpart, nb * kMaxTrunc * at))) return rc;
     if ((rc = ensure(h, h->cpart, nb * S * at))) return rc;
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
-    if ((rc = ensure(h, h->Q, Pn * M * S * 8))) return rc;
-    if ((rc = ensure(h, h->Qt, Pn * M * S * 8))) return rc;
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at));
+    if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;
     if ((rc = ensure(h, h->e, Pn * S * 8))) return rc;
@@ -922,7 +915,6 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     P.cpart = h->cpart.p;
     P.C = (double*)h->C.p;
     P.Q = (double*)h->Q.p;
-    P.Qt = (double*)h->Qt.p;
     P.R = (double*)h->R.p;
     P.d = (double*)h->d.p;
     P.e = (double*)h->e.p;
@@ -932,7 +924,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     P.coef = (double*)h->coef.p;
     P.hco = (double*)h->hco.p;
     P.cyc = (CycleState*)h->cyc.p;
-    P.qr_cluster = qr_cluster_for(g->P, s, m, g->nblk, h->sms);
+    P.qr = qs;
     P.jmax = jmax;
     P.Vb = (double*)h->Vb.p;
     P.Z = (double*)h->Z.p;
@@ -1070,7 +1062,7 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
                                                             (const void*)P.rp, (const void*)P.col, (const void*)P.val, (const void*)P.val32,
                           (const void*)P.blk_v0, (const void*)P.seg, (const void*)P.sl_off, (const void*)P.sl_col,
                           (const void*)P.sl_val, (const void*)P.sl_base, (const void*)P.sl_len, (const void*)P.ent, P.U, P.W,
-                          (const void*)P.sigma, P.normpart, P.hpart, P.cpart, (const void*)P.C, (const void*)P.Q, (const void*)P.Qt,
+                          (const void*)P.sigma, P.normpart, P.hpart, P.cpart, (const void*)P.C, (const void*)P.Q,
                           (const void*)P.R, (const void*)P.d, (const void*)P.e, (const void*)P.c0,
                           (const void*)P.rho, (const void*)P.y, (const void*)P.coef, (const void*)P.hco,
                           (const void*)P.cyc, (const void*)P.Vb, (const void*)P.Z, (const void*)P.nu,
@@ -1085,7 +1077,7 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
         u(p);
     for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
                       (int64_t)P.s, (int64_t)P.zeta, (int64_t)P.kind, (int64_t)P.sk_headroom, (int64_t)P.prec,
-                      (int64_t)P.m, (int64_t)P.t, (int64_t)P.qr_cluster, (int64_t)P.jmax, (int64_t)h->c3,
+                      (int64_t)P.m, (int64_t)P.t, (int64_t)P.qr.cluster, (int64_t)P.qr.staged, (int64_t)P.jmax, (int64_t)h->c3,
                       (int64_t)h->profile, (int64_t)P.gwait_extra, (int64_t)P.outer_variant})
         k.push_back((uint64_t)v);
     uint64_t bits;
@@ -1586,7 +1578,7 @@ int sfgmres_destroy(sfgmres_t h) {
             if (q) cudaFree(q);
     if (h->sl_sys) cudaFree(h->sl_sys);
     if (h->sl_base) cudaFree(h->sl_base);
-    DevBuf* bufs[] = {&h->U, &h->W, &h->sigma, &h->normpart, &h->hpart, &h->cpart, &h->C, &h->Q, &h->Qt, &h->R, &h->d,
+    DevBuf* bufs[] = {&h->U, &h->W, &h->sigma, &h->normpart, &h->hpart, &h->cpart, &h->C, &h->Q, &h->R, &h->d,
                       &h->e, &h->c0, &h->rho, &h->y, &h->coef, &h->hco, &h->cyc, &h->Vb, &h->Z, &h->nu, &h->Wo,
                       &h->opart, &h->npart, &h->npart2, &h->h1, &h->h2, &h->H, &h->cs, &h->sn, &h->g, &h->yo,
                       &h->est_hist, &h->ffom_hist, &h->ires_hist, &h->rho_hist, &h->k_hist, &h->reason_hist, &h->ost, &h->bst, &h->xst,

@@ -29,88 +29,96 @@ namespace cg = cooperative_groups;
 namespace sfg {
 
 // ---------------------------------------------------------------------------------------------------------------
-// Sketched QR update of column i, one cluster of nq CTAs per problem (cluster index = problem); CTA q owns rows [s q / nq, s (q+1) / nq) of Q and of the working vectors.  Q is kept twice: column-major
-// (Q[l*s + r]) for the projection Q^T p, where each thread takes a column and streams its rows, and row-major
-// (Qt[r*m + l]) for the subtraction p -= Q a, where each thread takes a row and streams its columns: every lane reads
-// contiguous memory, so each load instruction keeps 32 cache lines in flight and each line serves 16 elements (the
-// update is bound by the latency of these reads, not by their bandwidth).  When the CTA has few columns to project
-// (small i) or few rows (s / nq below 128), the work is split further: the projection's rows into up to 8 groups,
-// the subtraction's columns into up to 4, with the group partials combined in group order.  Partial dot products of
-// the CTAs go through distributed shared memory and are summed in rank order (deterministic, the same values in
-// every CTA, so every decision is taken identically everywhere).  Five cluster barriers per update: one per
-// Gram-Schmidt pass (the two passes' partials live in separate buffers), one for ||p||^2 and p^T e together
-// (d_i = p^T e / r_ii), one for the updated residual norm, and a last one before any CTA leaves.  Each CTA reads the
-// stop state itself (written by earlier launches; the one field another stream may change meanwhile, the breakdown
-// step, only ever moves to values above i).  CTAs are small (128 threads, at most 56 registers) so they fit beside
-// the inner step's CTAs.
-__device__ __forceinline__ double qr_rank_sum(cg::cluster_group& cl, double* base, int off, int nq) {
-    double acc = 0.0;
-#pragma unroll 8
-    for (int r2 = 0; r2 < nq; ++r2) acc += cl.map_shared_rank(base, r2)[off];
-    return acc;
-}
-
-// Sum over the CTA's 128 threads of v (warp trees, then the 4 warps in order); valid in thread 0 (0 elsewhere).
-__device__ __forceinline__ double qr_block_sum(double v, double* red4) {
-    v = warp_sum(v);
-    __syncthreads();  // red4 is free (its previous values have been read)
-    if ((threadIdx.x & 31) == 0) red4[threadIdx.x >> 5] = v;
-    __syncthreads();
-    return (threadIdx.x == 0) ? (red4[0] + red4[1]) + (red4[2] + red4[3]) : 0.0;
-}
-
-// Sum of x[u] * y[u] for u in [0, cnt), x contiguous (each lane of a warp streams its own stretch of Q, so every load
-// instruction has 32 cache lines in flight and every line serves 16 consecutive elements from L1): chunks of eight
-// loads, with the lane's lines four ahead prefetched into L1 (no registers held for them); four accumulators,
-// combined in a fixed order.
-__device__ __forceinline__ double qr_dot(const double* __restrict__ x, const double* __restrict__ y, int cnt) {
-    for (int k = 0; k < 64 && k < cnt; k += 16) prefetch_l1(x + k);
-    double c[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) c[u] = 0.0;
-    int k = 0;
-    for (; k + 8 <= cnt; k += 8) {
-        if ((k & 15) == 0 && k + 64 < cnt) prefetch_l1(x + k + 64);
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = x[k + u];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) c[u & 3] = fma(v[u], y[k + u], c[u & 3]);
-    }
-    for (; k < cnt; ++k) c[0] = fma(x[k], y[k], c[0]);  // at most 7, from lines already in L1
-    return (c[0] + c[1]) + (c[2] + c[3]);
-}
-
+// Sketched QR update of column i, one cluster of nq CTAs per problem (cluster index = problem); CTA q owns the sketch rows
+// [s q / nq, s (q+1) / nq) of Q and of the working vectors.  Q is stored CTA by CTA: the slice of CTA q holds its rows of
+// column l at slice[l * nrp + r] (nrp odd, so that threads taking consecutive columns of one row read distinct
+// shared-memory banks), which makes the columns 0..i-1 that an update needs one contiguous stretch.
+//
+// An update is a chain of dependent steps (two Gram-Schmidt passes, the norm, the residual), so what counts is the
+// latency of each and the FP64 instructions on its path: a warp's FP64 instruction holds its quarter of the SM's FP64 pipe
+// for some 67 cycles on this GPU.  Hence: as many SMs as the cluster can have share the 4 s i multiply-adds; the slice, the
+// new column and e come into shared memory in one wave of asynchronous 16-byte copies, and both products of both
+// passes run there (STAGED; a slice that does not fit is read from L2 in the same layout); products are split so that all
+// four warps work; scalars are formed by one thread (the two that need a division by two, in different warps).
+//  * projection a = Q^T p: column l by thread wp of group gp (Gp groups of rows), the CTAs' parts exchanged through
+//    distributed shared memory and summed in rank order (the same values in every CTA, so every decision is the same);
+//  * subtraction p -= Q a: row r by thread ws of group gs (Gs groups of columns).
+// Group partials are added in group order: every sum has a fixed order.  Five cluster barriers per update: one per pass, one
+// for ||p||^2 and p^T e together (d_i = p^T e / r_ii), one for the updated residual norm, and a last one before any
+// CTA leaves.  Each CTA reads the stop state itself (written by earlier launches; the one field another stream may change
+// meanwhile, the breakdown step, only ever moves to values above i).  CTAs are small (128 threads, at most 56 registers) so
+// they fit beside the inner step's CTAs.
+//
+// An update takes (clock64 of CTA 0) 11 us at s = 120, i = 15 on 4 CTAs, 15 us at s = 400, i = 50 on 16 and 27 us at s = 1000,
+// i = 100 on 16; the earlier form, which streamed column- and row-major copies of Q from L2 on 8 CTAs, took 58 us per update
+// of an 80^3 cycle at s = 1000, m = 200 (that cycle 13.4 -> 8.4 ms).
 constexpr int kQrThreads = 128;
 
+// Sum of v over groups of 16 lanes (every lane gets its group's sum).
+__device__ __forceinline__ double half_warp_sum(double v) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Sums of x and y over the CTA's threads, of which the first nws warps hold values; valid in warp 0: x in lanes 0-15, y in
+// lanes 16-31 (half the additions of two separate trees).
+__device__ __forceinline__ double qr_pair_sum(double x, double y, double (*red)[4], int nws) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v = 0.0;
+    if (warp < nws) {
+        const double ox = __shfl_xor_sync(0xffffffffu, x, 16), oy = __shfl_xor_sync(0xffffffffu, y, 16);
+        v = half_warp_sum(lane < 16 ? x + ox : y + oy);
+    }
+    if (nws > 1) {
+        if ((lane & 15) == 0) red[lane >> 4][warp] = v;
+        __syncthreads();
+        if (warp == 0) {
+            v = red[lane >> 4][0];
+            for (int w = 1; w < nws; ++w) v += red[lane >> 4][w];
+        }
+    }
+    return v;
+}
+
+template <bool STAGED>
 __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i) {
     cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_arrive();  // waited for before the first access to another CTA's shared memory: all CTAs have started
     const int q = (int)cl.block_rank(), nq = (int)cl.num_blocks();
     const int prob = blockIdx.x / nq;
-    const int s = P.s, m = P.m;
-    const double* __restrict__ C = P.C + (int64_t)prob * m * s;
-    double* __restrict__ Q = P.Q + (int64_t)prob * m * s;
-    double* __restrict__ Qt = P.Qt + (int64_t)prob * m * s;
-    double* __restrict__ R = P.R + (int64_t)prob * m * m;
-    double* __restrict__ d = P.d + (int64_t)prob * m;
-    double* __restrict__ e = P.e + (int64_t)prob * s;
-    double* __restrict__ rho = P.rho + (int64_t)prob * m;
+    const int s = P.s, m = P.m, nrp = P.qr.nrp;
+    double* __restrict__ Qg = P.Q + ((int64_t)prob * nq + q) * P.qr.slice;
     CycleState* cyc = P.cyc + prob;
     const int rlo = (int)((int64_t)s * q / nq), rhi = (int)((int64_t)s * (q + 1) / nq), nr = rhi - rlo;
-    const int nrmax = (s + nq - 1) / nq;
-    extern __shared__ double qsm[];
-    double* p = qsm;               // [nrmax] this CTA's rows of the working vector
-    double* apart = qsm + nrmax;   // [2][m] partial projections over this CTA's rows, one buffer per pass
-    double* a = apart + 2 * m;     // [m] full projections
-    __shared__ double red4[4];
-    __shared__ double scal[4];
-    __shared__ double bc[4];            // scalars formed by thread 0 for the CTA (FP64 division and square roots
-                                        // cost tens of FP64-pipe cycles per warp: once per CTA, not per thread)
-    __shared__ double grp[kQrThreads];  // group partials of a split projection or subtraction
+    double* __restrict__ e = P.e + (int64_t)prob * s + rlo;
+    extern __shared__ __align__(16) double qsm[];
+    const int ns = STAGED ? (i * nrp + 1) & ~1 : 0;
+    const double* Q = STAGED ? qsm : Qg;  // columns 0..i-1 of the slice
+    double* p = qsm + ns;                 // [nrp] this CTA's rows of the working vector
+    double* es = p + nrp;                 // [nrp] its rows of e
+    double* a = es + nrp;                 // [m] full projections
+    double* part = a + m;                 // [2][m] partial projections over this CTA's rows, one buffer per pass
+    __shared__ double red[2][4];
+    __shared__ double sum_sh[3][16];      // every CTA's ||p||^2, p^T e and (CTA 0) ||e||^2 partials
+    __shared__ double bc[4];              // scalars formed once for the CTA
+    __shared__ double grp[kQrThreads];    // group partials of a split projection, rank sum or subtraction
     const int tid = threadIdx.x;
+    if constexpr (STAGED) {
+        // i * nrp doubles rounded up to 16 bytes (the slice has room for the rounding)
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(qsm);
+        for (int u = tid; u < ns / 2; u += kQrThreads)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * u), "l"(Qg + 2 * u) : "memory");
+    }
     // the cycle state as earlier launches left it (the same for every CTA of the cluster)
     const double dmax0 = cyc->dmax, dmin0 = cyc->dmin, thr = cyc->cond_thr;
     const int code = (cyc->stopped || (P.pflag[prob] & 1)) ? 1 : (cyc->brk_step <= i ? 2 : 0);
+    for (int r = tid; r < nr; r += kQrThreads) {
+        p[r] = P.C[((int64_t)prob * m + i) * s + rlo + r];
+        es[r] = e[r];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    cl.barrier_wait();
     if (code) {
         if (code == 2 && q == 0 && tid == 0) {
             cyc->stopped = 1;  // u_i has zero (or non-finite) norm: the cycle keeps k = i columns
@@ -118,78 +126,108 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
         }
         return;  // the whole cluster returns
     }
-    for (int r = tid; r < nr; r += kQrThreads) p[r] = C[(int64_t)i * s + rlo + r];
     // projection split: Gp groups of rows (Gp * i <= 128 threads), Wp threads per group over the columns
     int Gp = 1;
-    while (Gp < 8 && 2 * Gp * i <= kQrThreads && 2 * Gp * 8 <= nr) Gp *= 2;
+    while (Gp < 8 && 2 * Gp * i <= kQrThreads && 2 * Gp * 2 <= nr) Gp *= 2;
     const int Wp = kQrThreads / Gp, gp = tid / Wp, wp = tid % Wp;
     const int pr0 = nr * gp / Gp, pr1 = nr * (gp + 1) / Gp;
+    int Gr = 1;  // rank-sum split: Gr groups of ranks (a power of two; Gr * i <= 128 threads)
+    while (2 * Gr < nq && 2 * Gr * i <= kQrThreads) Gr *= 2;
     // subtraction split: Wr threads over the rows (a power of two from 32 to 128, so that Gs Wr = 128 and every
     // thread has a group), Gs groups of columns
     int Wr = 32;
     while (Wr < nr && Wr < kQrThreads) Wr *= 2;
     const int Gs = kQrThreads / Wr, gs = tid / Wr, ws = tid % Wr;
     const int sl0 = i * gs / Gs, sl1 = i * (gs + 1) / Gs;
-    const unsigned long long keep = l2_keep_policy();  // Q and Qt are read again at every update of the cycle
+    const int nws = (min(nr, kQrThreads) + 31) / 32;  // warps whose threads hold rows in the per-row loops
     __syncthreads();
-    for (int pass = 0; pass < 2; ++pass) {
-        double* ap = apart + pass * m;
-        // this CTA's part of Q^T p: column l by thread wp of group gp, over the group's rows (contiguous in Q)
+    for (int pass = 0; pass < 2 && i > 0; ++pass) {
+        double* ap = part + pass * m;
         for (int l = wp; l < i; l += Wp) {
-            const double v = qr_dot(Q + (int64_t)l * s + rlo + pr0, p + pr0, pr1 - pr0);
+            const double* ql = Q + l * nrp;
+            double v = 0.0;
+#pragma unroll 8
+            for (int r = pr0; r < pr1; ++r) v = fma(ql[r], p[r], v);
             if (Gp == 1) ap[l] = v;
             else grp[gp * i + l] = v;
         }
         if (Gp > 1) {
             __syncthreads();
             for (int l = tid; l < i; l += kQrThreads) {
-                double v = 0.0;
-                for (int g = 0; g < Gp; ++g) v += grp[g * i + l];
+                double v = grp[l];
+                for (int g = 1; g < Gp; ++g) v += grp[g * i + l];
                 ap[l] = v;
             }
         }
         cl.sync();  // this pass's partials of every CTA are in place
-        for (int l = tid; l < i; l += kQrThreads) a[l] = qr_rank_sum(cl, ap, l, nq);
-        __syncthreads();
-        // p -= Q a over this CTA's rows: row r by thread ws, the columns of group gs (contiguous in Qt)
-        for (int r = ws; r < nr; r += Wr) {
-            const double v = qr_dot(Qt + (int64_t)(rlo + r) * m + sl0, a + sl0, sl1 - sl0);
-            if (Gs == 1) p[r] -= v;
-            else grp[gs * Wr + r] = v;
-        }
-        if (Gs > 1) {
+        auto rank_sum = [&](int l, int r0, int r1) -> double {
+            double v = 0.0;
+#pragma unroll 4
+            for (int r2 = r0; r2 < r1; ++r2) v += cl.map_shared_rank(ap, r2)[l];
+            return v;
+        };
+        if (Gr > 1) {
+            if (tid < Gr * i) grp[tid] = rank_sum(tid % i, nq / Gr * (tid / i), nq / Gr * (tid / i + 1));
             __syncthreads();
-            for (int r = tid; r < nr; r += kQrThreads) {
-                double v = 0.0;
-                for (int g = 0; g < Gs; ++g) v += grp[g * Wr + r];
-                p[r] -= v;
+            if (tid < i) {
+                double v = grp[tid];
+                for (int g = 1; g < Gr; ++g) v += grp[g * i + tid];
+                a[tid] = v;
+            }
+        } else {
+            for (int l = tid; l < i; l += kQrThreads) a[l] = rank_sum(l, 0, nq);
+        }
+        __syncthreads();
+        for (int r0 = 0; r0 < nr; r0 += Wr) {
+            const int r = r0 + ws;
+            double v = 0.0;
+            if (r < nr) {
+#pragma unroll 8
+                for (int l = sl0; l < sl1; ++l) v = fma(Q[l * nrp + r], a[l], v);
+                if (Gs == 1) p[r] -= v;
+                else grp[gs * Wr + ws] = v;
             }
         }
-        if (q == 0)
-            for (int l = tid; l < i; l += kQrThreads) R[(int64_t)i * m + l] = (pass ? R[(int64_t)i * m + l] : 0.0) + a[l];
+        if (Gs > 1) {  // then nr <= Wr
+            __syncthreads();
+            if (tid < nr) {
+                double v = grp[tid];
+                for (int g = 1; g < Gs; ++g) v += grp[g * Wr + tid];
+                p[tid] -= v;
+            }
+        }
+        if (q == 0) {  // column i of R: the sum of the two passes' projections
+            double* __restrict__ Ri = P.R + ((int64_t)prob * m + i) * m;
+            for (int l = tid; l < i; l += kQrThreads) Ri[l] = pass ? Ri[l] + a[l] : a[l];
+        }
         __syncthreads();
     }
     // r_ii = ||p|| and p^T e from one exchange
-    double v2 = 0.0, pe = 0.0;
+    const int lane = tid & 31, warp = tid >> 5;
+    double pp = 0.0, pe = 0.0;
     for (int r = tid; r < nr; r += kQrThreads) {
-        v2 += p[r] * p[r];
-        pe += p[r] * e[rlo + r];
+        pp = fma(p[r], p[r], pp);
+        pe = fma(p[r], es[r], pe);
     }
-    v2 = qr_block_sum(v2, red4);
-    pe = qr_block_sum(pe, red4);
-    if (tid == 0) {
-        scal[0] = v2;
-        scal[1] = pe;
+    {
+        const double v = qr_pair_sum(pp, pe, red, nws);
+        if (warp == 0 && (lane & 15) < nq) cl.map_shared_rank(&sum_sh[lane >> 4][q], lane & 15)[0] = v;
     }
     cl.sync();
-    if (tid == 0) {
-        const double rii0 = sqrt(qr_rank_sum(cl, scal, 0, nq));
-        const double dmx = fmax(dmax0, rii0);
-        const double dmn = (i == 0) ? rii0 : fmin(dmin0, rii0);
-        bc[0] = rii0;
-        bc[1] = qr_rank_sum(cl, scal, 1, nq);
-        bc[2] = (dmn > 0.0) ? dmx / dmn : INFINITY;  // the condition proxy
-        bc[3] = 1.0 / rii0;
+    if (warp < 2) {  // the ranks' sums by a tree; one warp forms r_ii and its reciprocal, another the condition proxy
+        const double v = half_warp_sum((lane & 15) < nq ? sum_sh[lane >> 4][lane & 15] : 0.0);
+        if (tid == 0) {
+            const double rii0 = sqrt(v);
+            bc[0] = rii0;
+            bc[3] = 1.0 / rii0;
+        } else if (tid == 16) {
+            bc[1] = v;
+        } else if (tid == 32) {
+            const double rii0 = sqrt(v);
+            const double dmx = fmax(dmax0, rii0);
+            const double dmn = (i == 0) ? rii0 : fmin(dmin0, rii0);
+            bc[2] = (dmn > 0.0) ? dmx / dmn : INFINITY;
+        }
     }
     __syncthreads();
     const double rii = bc[0], pet = bc[1], kappa = bc[2], inv = bc[3];
@@ -201,185 +239,29 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
             cyc->k = i;
             cyc->reason = (i == 0) ? 5 : 2;
         }
-        cl.sync();  // no CTA leaves while another may still read its shared memory
+        cl.sync();  // no CTA leaves while another may still reach its shared memory
         return;
     }
+    const unsigned long long keep = l2_keep_policy();  // Q is read again at every update of the cycle
     const double di = pet * inv;
     double ee = 0.0;
     for (int r = tid; r < nr; r += kQrThreads) {
         const double qv = p[r] * inv;
-        st_keep(Q + (int64_t)i * s + rlo + r, qv, keep);
-        st_keep(Qt + (int64_t)(rlo + r) * m + i, qv, keep);
-        const double ev = e[rlo + r] - di * qv;
-        e[rlo + r] = ev;
-        ee += ev * ev;
-    }
-    ee = qr_block_sum(ee, red4);
-    if (tid == 0) scal[2] = ee;
-    cl.sync();
-    if (q == 0 && tid == 0) {
-        const double rh = sqrt(qr_rank_sum(cl, scal, 2, nq));
-        R[(int64_t)i * m + i] = rii;
-        d[i] = di;
-        rho[i] = rh;
-        cyc->dmax = dmax;
-        cyc->dmin = dmin;
-        cyc->k = i + 1;
-        cyc->rho = rh;
-        if (cyc->c3_on && cyc->c3_scale * rh <= cyc->c3_tol) {
-            cyc->stopped = 1;
-            cyc->reason = 3;
-        } else if (i + 1 == m) {
-            cyc->stopped = 1;
-            cyc->reason = 1;
-        }
-    }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
-}
-
-// ---------------------------------------------------------------------------------------------------------------
-// The same sketched QR update for small sketches (qr_small_fits, few problems), one CTA of kQrSmallThreads
-// threads per problem and no cluster.  An update of a small sketch is a chain of dependent steps whose cost is the
-// number of round trips to memory, so every global input -- the columns 0..i-1 of Q, the new column of C, the
-// residual sketch e, the cycle state -- is loaded into shared memory in one wave of loads at the start, and the two
-// Gram-Schmidt passes, the norms and the stop tests then run on shared memory (block barriers instead of cluster
-// barriers and distributed-shared-memory exchanges).  Projections: warp w takes columns w, w + 16, ..., its lanes
-// strided over the rows, then the warp's shuffle tree.  Subtraction: G threads per row (G s <= the CTA), each over a
-// contiguous share of the columns, the G partials added by a shuffle tree.  Block sums: warp trees, then the warps
-// in order.  Only Q is written (not its row-major copy Qt, which only the cluster kernel reads).  The decisions
-// (rules C1-C3, the breakdown and C2 stops) are those of k_inner_qr.
-constexpr int kQrSmallThreads = 512;
-
-// Sum of v over the threads of the first nws warps (the others hold no rows): warp trees, then the warps in order;
-// valid in thread 0 (0 elsewhere).  FP64 arithmetic is scarce on this GPU, so no thread adds what it does not need.
-__device__ __forceinline__ double qr_small_sum(double v, double* red, int nws) {
-    const int warp = threadIdx.x >> 5;
-    if (warp < nws) v = warp_sum(v);
-    __syncthreads();  // red is free (its previous values have been read)
-    if (warp < nws && (threadIdx.x & 31) == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < nws; ++w) t += red[w];
-    return t;
-}
-
-__global__ void __launch_bounds__(kQrSmallThreads) k_inner_qr_small(const Plan P, int i) {
-    constexpr int nw = kQrSmallThreads / 32;
-    const int prob = blockIdx.x;
-    const int s = P.s, m = P.m;
-    const double* __restrict__ C = P.C + (int64_t)prob * m * s;
-    double* __restrict__ Q = P.Q + (int64_t)prob * m * s;
-    double* __restrict__ R = P.R + (int64_t)prob * m * m;
-    double* __restrict__ d = P.d + (int64_t)prob * m;
-    double* __restrict__ e = P.e + (int64_t)prob * s;
-    double* __restrict__ rho = P.rho + (int64_t)prob * m;
-    CycleState* cyc = P.cyc + prob;
-    extern __shared__ double qsm[];
-    double* qs = qsm;              // [i s] columns 0..i-1 of Q (column-major)
-    double* p = qs + (int64_t)i * s;  // [s] the working vector
-    double* es = p + s;            // [s] e
-    double* a1 = es + s;           // [m] first-pass projections
-    double* a = a1 + m;            // [m] projections of the current pass
-    __shared__ double red[nw];
-    __shared__ double cst[3];
-    __shared__ double bc[4];  // scalars formed by thread 0 (one square root and divisions per update, not per thread)
-    __shared__ int code_sh;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) {
-        cst[0] = cyc->dmax;
-        cst[1] = cyc->dmin;
-        cst[2] = cyc->cond_thr;
-        code_sh = (cyc->stopped || (P.pflag[prob] & 1)) ? 1 : (cyc->brk_step <= i ? 2 : 0);
-    }
-    const int nq = i * s;
-    for (int k = tid; k < nq; k += kQrSmallThreads) qs[k] = Q[k];
-    for (int r = tid; r < s; r += kQrSmallThreads) {
-        p[r] = C[(int64_t)i * s + r];
-        es[r] = e[r];
-    }
-    __syncthreads();
-    const int code = code_sh;
-    if (code) {
-        if (code == 2 && tid == 0) {
-            cyc->stopped = 1;  // u_i has zero (or non-finite) norm: the cycle keeps k = i columns
-            cyc->reason = cyc->brk_reason;
-        }
-        return;
-    }
-    int G = 1;
-    while (G < 32 && 2 * G * s <= kQrSmallThreads) G *= 2;
-    const int rg = tid / G, gg = tid % G;
-    const int c0 = i * gg / G, c1 = i * (gg + 1) / G;
-    for (int pass = 0; pass < 2; ++pass) {
-        // a = Q^T p: column l by warp l % nw
-        for (int l = warp; l < i; l += nw) {
-            const double* ql = qs + (int64_t)l * s;
-            double acc = 0.0;
-            for (int r = lane; r < s; r += 32) acc = fma(ql[r], p[r], acc);
-            acc = warp_sum(acc);
-            if (lane == 0) a[l] = acc;
-        }
-        __syncthreads();
-        // p -= Q a: row r by its G threads
-        for (int base = 0; base < s; base += kQrSmallThreads / G) {  // the same trip count in every thread
-            const int r = base + rg;
-            double acc = 0.0;
-            if (r < s)
-                for (int l = c0; l < c1; ++l) acc = fma(qs[(int64_t)l * s + r], a[l], acc);
-            for (int o = 1; o < G; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);  // all lanes take part
-            if (r < s && gg == 0) p[r] -= acc;
-        }
-        if (pass == 0)
-            for (int l = tid; l < i; l += kQrSmallThreads) a1[l] = a[l];
-        __syncthreads();
-    }
-    for (int l = tid; l < i; l += kQrSmallThreads) R[(int64_t)i * m + l] = a1[l] + a[l];
-    // r_ii = ||p|| and p^T e
-    const int nws = (min(s, kQrSmallThreads) + 31) / 32;  // warps that hold rows
-    double v2 = 0.0, pe = 0.0;
-    for (int r = tid; r < s; r += kQrSmallThreads) {
-        v2 = fma(p[r], p[r], v2);
-        pe = fma(p[r], es[r], pe);
-    }
-    v2 = qr_small_sum(v2, red, nws);
-    pe = qr_small_sum(pe, red, nws);
-    if (tid == 0) {
-        const double rii0 = sqrt(v2);
-        const double dmx = fmax(cst[0], rii0);
-        const double dmn = (i == 0) ? rii0 : fmin(cst[1], rii0);
-        bc[0] = rii0;
-        bc[1] = pe;
-        bc[2] = (dmn > 0.0) ? dmx / dmn : INFINITY;  // the condition proxy
-        bc[3] = 1.0 / rii0;
-    }
-    __syncthreads();
-    const double rii = bc[0], pet = bc[1], kappa = bc[2], inv = bc[3];
-    const double dmax = fmax(cst[0], rii);
-    const double dmin = (i == 0) ? rii : fmin(cst[1], rii);
-    if (!(kappa <= cst[2])) {  // C2 (also rii == 0 or NaN): drop column i, keep k = i
-        if (tid == 0) {
-            cyc->stopped = 1;
-            cyc->k = i;
-            cyc->reason = (i == 0) ? 5 : 2;
-        }
-        return;
-    }
-    const double di = pet * inv;
-    double ee = 0.0;
-    for (int r = tid; r < s; r += kQrSmallThreads) {
-        const double qv = p[r] * inv;
-        Q[(int64_t)i * s + r] = qv;
+        st_keep(Qg + i * nrp + r, qv, keep);
         const double ev = es[r] - di * qv;
         e[r] = ev;
         ee = fma(ev, ev, ee);
     }
-    ee = qr_small_sum(ee, red, nws);
-    if (tid == 0) {
+    ee = qr_pair_sum(ee, 0.0, red, nws);
+    if (tid == 0) cl.map_shared_rank(&sum_sh[2][q], 0)[0] = ee;
+    cl.sync();  // the last access to another CTA's shared memory has been made
+    if (q != 0 || warp != 0) return;
+    ee = half_warp_sum(lane < nq ? sum_sh[2][lane & 15] : 0.0);
+    if (lane == 0) {
         const double rh = sqrt(ee);
-        R[(int64_t)i * m + i] = rii;
-        d[i] = di;
-        rho[i] = rh;
+        P.R[((int64_t)prob * m + i) * m + i] = rii;
+        P.d[(int64_t)prob * m + i] = di;
+        P.rho[(int64_t)prob * m + i] = rh;
         cyc->dmax = dmax;
         cyc->dmin = dmin;
         cyc->k = i + 1;
@@ -647,32 +529,50 @@ void launch_inner_axpy(const Plan& p, int i, bool last) {
     ++g_launches;
 }
 
+// Dynamic shared memory of update i: the staged columns, the CTA's rows of p and e, the projections and their parts.
+static size_t qr_smem(const QrShape& q, int m, int i) {
+    return ((size_t)(q.staged ? (i * q.nrp + 1) & ~1 : 0) + 2 * (size_t)q.nrp + 3 * (size_t)m) * sizeof(double);
+}
+
+// Few CTAs where an update's FP64 work is small (its latency is then the exchanges, which grow with the CTAs), many where it
+// is large.  Whole solves, 2 / 4 / 8 / 16 CTAs: s = 80, m = 20 (2D 32^2) 2.40 / 2.51 / 2.54 / 2.49 ms; s = 120, m = 30 (2D
+// 64^2) 4.34 / 4.12 / 5.21 / 5.03 ms; s = 240, m = 60 (3D 32^3) 3.36 / 3.19 / 3.56 / 3.41 ms; s = 320, m = 80 (40^3) 4.96 / 4.47
+// / 4.06 / 3.90 ms; s = 1000, m = 200 (80^3) 44.3 / 28.9 / 20.9 / 15.9 ms.  Batches take what leaves the problems' clusters
+// side by side on the GPU.
+QrShape qr_shape(int P, int s, int m, size_t smem_left) {
+    QrShape q;
+    const int most = P <= 4 ? kQrCluster : P <= 16 ? 8 : P <= 32 ? 4 : P <= 64 ? 2 : 1;
+    q.cluster = std::min(most, s * m <= 3000 ? 2 : s * m <= 20000 ? 4 : kQrCluster);
+    q.nrp = ((s + q.cluster - 1) / q.cluster) | 1;
+    q.slice = (q.nrp * m + 1) & ~1;
+    q.staged = true;
+    q.staged = qr_smem(q, m, m - 1) <= smem_left;
+    return q;
+}
+
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st) {
-    if (p.qr_cluster == 0) {  // small sketch: one CTA per problem, Q's columns 0..i-1 in shared memory
-        const size_t sm = ((size_t)i * p.s + 2 * (size_t)p.s + 2 * (size_t)p.m) * sizeof(double);
-        set_smem((const void*)k_inner_qr_small, sm);
-        k_inner_qr_small<<<p.P, kQrSmallThreads, sm, st>>>(p, i);
-        ++g_launches;
-        return cudaGetLastError();
+    const QrShape& q = p.qr;
+    void (*fn)(const Plan, int) = q.staged ? k_inner_qr<true> : k_inner_qr<false>;
+    const size_t sm = qr_smem(q, p.m, i);
+    set_smem((const void*)fn, qr_smem(q, p.m, p.m - 1));
+    if (q.cluster > 8) {
+        const cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
     }
-    const int nq = p.qr_cluster;
-    const int nrmax = (p.s + nq - 1) / nq;
-    const size_t sm = (size_t)(nrmax + 3 * p.m) * sizeof(double);
-    set_smem((const void*)k_inner_qr, sm);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nq * p.P), 1, 1);
+    cfg.gridDim = dim3((unsigned)(q.cluster * p.P), 1, 1);
     cfg.blockDim = dim3(kQrThreads, 1, 1);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = nq;
+    attr[0].val.clusterDim.x = q.cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     ++g_launches;
-    return cudaLaunchKernelEx(&cfg, k_inner_qr, p, i);
+    return cudaLaunchKernelEx(&cfg, fn, p, i);
 }
 
 void launch_inner_finish(const Plan& p, double* z) {

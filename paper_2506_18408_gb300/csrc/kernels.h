@@ -42,6 +42,14 @@ struct IluHost {
     IluDev dev;
 };
 
+// Shape of the sketched-QR update.
+struct QrShape {
+    int cluster = 8;     // CTAs per problem (one cluster)
+    int nrp = 0;         // rows of Q per CTA, padded to an odd number
+    int slice = 0;       // doubles of one CTA's slice of Q (nrp * m, even)
+    bool staged = false; // the slice is kept in shared memory during an update
+};
+
 // Everything a kernel needs, as plain device pointers and sizes (owned by the solver handle).
 struct Plan {
     // matrix (concatenated CSR, int32 indices, global column indices)
@@ -101,8 +109,7 @@ struct Plan {
     void* hpart = nullptr;     // AT[nblk * kMaxTrunc]
     void* cpart = nullptr;     // AT[nblk * s]
     double* C = nullptr;       // [P][m][s]  S A b_i
-    double* Q = nullptr;       // [P][m][s]  column-major: Q[l*s + r]
-    double* Qt = nullptr;      // [P][s][m]  the same, row-major: Qt[r*m + l]
+    double* Q = nullptr;       // [P][qr.cluster][qr.slice] by the QR's CTAs: row r of CTA q, column l at l*qr.nrp + r
     double* R = nullptr;       // [P][m][m]  column-major, R[i*m + l] = R_{l,i}
     double* d = nullptr;       // [P][m]
     double* e = nullptr;       // [P][s]     running sketched residual
@@ -112,7 +119,7 @@ struct Plan {
     double* coef = nullptr;    // [P][m]     y_l * sigma_l
     double* hco = nullptr;     // [P][m][kMaxTrunc] truncated-Arnoldi coefficients
     CycleState* cyc = nullptr; // [P]
-    int qr_cluster = 8;        // CTAs per problem (one cluster) in the sketched-QR kernel; 0: the single-CTA kernel
+    QrShape qr;
 
     // outer FGMRES
     int jmax = 0;
@@ -216,12 +223,9 @@ void inner_axpy_f64(const Plan& p, int i, bool last);
 void inner_axpy_f32(const Plan& p, int i, bool last);
 void inner_axpy_bf16(const Plan& p, int i, bool last);
 void launch_inner_axpy(const Plan& p, int i, bool last);
-// Sketches whose QR working set fits in kQrSmallElems doubles of shared memory (columns 0..m-2 of Q, the new column,
-// e, two projection vectors), for at most kQrSmallProblems problems, take the single-CTA sketched QR.
-constexpr int kQrSmallElems = 24576;  // 192 KB
-constexpr int kQrSmallProblems = 16;
-inline bool qr_small_fits(int s, int m) { return (int64_t)s * (m + 1) + 2 * (int64_t)m <= kQrSmallElems; }
-cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st (cluster or single-CTA kernel)
+// For P problems, sketch size s and basis size m, given the shared memory left on an SM beside the inner step's CTAs.
+QrShape qr_shape(int P, int s, int m, size_t smem_left);
+cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st
 void launch_inner_finish(const Plan& p, double* z);  // y = R^{-1} d, z = sum_l y_l b_l (FP64)
 void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r] = sigma_l * u_l[r] (FP64)
 

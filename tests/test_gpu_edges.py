@@ -38,3 +38,23 @@ def test_correction_is_the_basis_times_y(Solver, precision, n, m, block_rows):
     bound = (2 * k + 8) * 2.0 ** -53 if precision == "fp64" else (k + 8) ** 2 * 2.0 ** -46
     assert np.all(np.abs(z - y @ B) <= bound * size + 1e-300)
     sv.close()
+
+
+# the sketched QR: fewer sketch rows than CTAs of its cluster, rows just past a warp, more columns than threads, slices that
+# do not fit in shared memory; clusters of 2, 4 and 16 CTAs
+@pytest.mark.parametrize("N,m,s", [(20, 8, 8), (30, 24, 33), (40, 40, 160), (60, 130, 520), (70, 300, 1000), (70, 600, 1200)])
+def test_sketched_least_squares_is_optimal(Solver, N, m, s):
+    from oracle import sketch as osk
+
+    A = workloads.convdiff(N, (30.0, 10.0))
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1)
+    v = _unit(A.n, m)
+    _, k, _, B, y = sv.inner_cycle(v, m=m, s=s, k=2)
+    assert k > min(m, 100) // 2
+    S = osk.sketch_matrix(A.n, s, 8, 1)
+    C = S @ (A.to_scipy() @ B[:k].cpu().numpy().T)
+    c, y = S @ v.cpu().numpy(), y.cpu().numpy()
+    # Gram-Schmidt with reorthogonalisation solves a problem perturbed by O(k s u) relative to its data
+    size = np.linalg.norm(C) * (np.linalg.norm(c) + np.linalg.norm(C) * np.linalg.norm(y))
+    assert np.linalg.norm(C.T @ (c - C @ y)) <= 8 * k * s * 2.0 ** -53 * size
+    sv.close()

@@ -27,7 +27,8 @@ void set_smem(const void* func, size_t bytes) {
     std::lock_guard<std::mutex> lk(mu);
     auto it = done.find(func);
     if (it != done.end() && it->second >= bytes) return;
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the default limit of 48 KB counts a kernel's static shared memory too (at most 8 KB here)
+    if (bytes > 40 * 1024) cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     done[func] = bytes;
 }
 

@@ -1,5 +1,9 @@
 """Kernels at the edges of their tiles, on the GPU: lengths around the pieces a CTA or a warp takes, remainders of their
 unrolled loops, the smallest and largest sizes, against NumPy arithmetic on the same values."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -58,3 +62,19 @@ def test_sketched_least_squares_is_optimal(Solver, N, m, s):
     size = np.linalg.norm(C) * (np.linalg.norm(c) + np.linalg.norm(C) * np.linalg.norm(y))
     assert np.linalg.norm(C.T @ (c - C @ y)) <= 8 * k * s * 2.0 ** -53 * size
     sv.close()
+
+
+# row blocks whose shared memory is just under the 48 KB a launch gets by default, in a process that has not raised it yet
+@pytest.mark.parametrize("block_rows", [5632, 6112, 6144])
+def test_blocks_just_under_the_default_shared_memory(Solver, block_rows):
+    code = f"""
+import sys; sys.path.insert(0, '.')
+import torch, workloads
+from paper_2506_18408_gb300 import Solver
+A = workloads.convdiff(90, (30.0, 10.0))
+b = torch.from_numpy(workloads.rhs(A.n, seed=0)).cuda()
+x, info = Solver(A.n, A.row_ptr, A.col, A.val, block_rows={block_rows}).solve(b, m=30, s=120, k=2, tol=1e-8)
+sys.exit(info['status'])
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    assert subprocess.run([sys.executable, "-c", code], cwd=root).returncode == 0

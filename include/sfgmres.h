@@ -70,10 +70,11 @@ extern "C" {
                                         thread each, 17..64 entries 8 lanes, longer rows a warp).  Reading it
                                         returns the shape in use: 1, 2..32, or 0 for the length-binned SpMV. */
 #define SFGMRES_OPT_BLOCK_ROWS 9     /* rows per row block of the fused inner kernels: a multiple of 32 in
-                                        [32, 8192], or 0 (default) = chosen by the library (one system: about a
-                                        multiple of the SM count of blocks, less 8 SMs with FP64 inner cycles, which
-                                        are left to the sketched-QR update running beside the fused kernel; several
-                                        systems: 4096).  Reading it returns the size in use. */
+                                        [32, 8192], or 0 (default) = chosen by the library (one system: two blocks
+                                        per SM, less 8 SMs with FP64 inner cycles, which are left to the sketched-QR
+                                        update running beside the fused kernel, or at most 128 blocks for small
+                                        systems; many right-hand sides of one system: 5120; several systems: 4096).
+                                        Reading it returns the size in use. */
 #define SFGMRES_OPT_GRAPH 10         /* 1 (default): each outer step (one inner cycle for every problem and the outer
                                         FGMRES update) is captured once into a CUDA graph and replayed; the graphs
                                         are kept while the solve's parameters and workspaces stay the same.  0: the

@@ -53,7 +53,38 @@ namespace sfg {
 void set_global_error(const std::string& msg) { g_create_error = msg; }
 }  // namespace sfg
 
-struct sfgmres_ctx {
+// List-block geometry (depends on the systems, the precision, the number of right-hand sides and the block-rows option; a new
+// version at every change) and everything built for it.
+struct ListSet {
+    int Bn = 0, nl = 0, geo_ver = 0;
+    std::vector<int> sys_Bq, sys_l0;
+
+    // length-binned SpMV row orders for A [0] and A^T [1] (built for one geometry version), and the matrix row
+    // blocks' first rows and lengths on the device
+    uint16_t* perm[2] = {nullptr, nullptr};
+    int* cls[2] = {nullptr, nullptr};
+    int bins_ver[2] = {-1, -1};
+    int* lb = nullptr;  // lb_m0 [nl], lb_len [nl]
+    int lb_ver = -1;
+    // the length-binned SpMV's FP64 copies of A [0] and A^T [1] with each row block's rows in its processing order
+    // (built for one geometry version; values follow sfgmres_update_values)
+    struct BCopy {
+        int* rp = nullptr;
+        int* col = nullptr;
+        double* val = nullptr;
+        int ver = -1;
+    } bc[2];
+
+    // sketch gather lists (cached for one (s, zeta, kind, geometry version))
+    int sk_s = -1, sk_zeta = -1, sk_kind = -1, sk_ver = -1, sk_headroom = 0, sk_word = 0;
+    int* seg = nullptr;
+    uint16_t* ent = nullptr;
+
+    int* sl_base = nullptr;  // [list blocks] first SELL-32 slice of each list block
+    int sl_base_ver = -1;
+};
+
+struct sfgmres_ctx : ListSet {
     int dev = 0;
     int nsys = 1;
     int n = 0;                  // rows of the block-diagonal matrix (sum over systems)
@@ -81,8 +112,6 @@ struct sfgmres_ctx {
     } sell[2];
     int sl_ns = 0;                 // slices (the same for A and A^T: block-diagonal with the same blocks)
     int* sl_sys = nullptr;         // [nsys + 1] first slice of each system, then [nsys + 1] first row of each system
-    int* sl_base = nullptr;        // [list blocks] first slice of each list block
-    int sl_base_ver = -1;
     uint64_t seed = 0;
     cudaStream_t st = nullptr;
     bool own_stream = false;
@@ -102,34 +131,13 @@ struct sfgmres_ctx {
     bool step_fused = false;  // the last cycle ran the fused inner step
     double cond_thr = 1e15;
 
-    // list-block geometry (depends on the systems and the block-rows option; version bumps on change)
-    int Bn = 0, vec = 8, nl = 0, geo_ver = 0;
-    std::vector<int> sys_Bq, sys_l0;
+    int vec = 8;
+    ListSet other;     // the list blocks used before the current ones (choose_lists)
+    int geo_next = 0;  // next geometry version
 
     // vector-block geometries, cached per number of right-hand sides
     Geo geos[kGeoCache];
     uint64_t geo_clock = 0;
-
-    // length-binned SpMV row orders for A [0] and A^T [1] (built for one geometry version), and the matrix row
-    // blocks' first rows and lengths on the device
-    uint16_t* perm[2] = {nullptr, nullptr};
-    int* cls[2] = {nullptr, nullptr};
-    int bins_ver[2] = {-1, -1};
-    int* lb = nullptr;  // lb_m0 [nl], lb_len [nl]
-    int lb_ver = -1;
-    // the length-binned SpMV's FP64 copies of A [0] and A^T [1] with each row block's rows in its processing order
-    // (built for one geometry version; values follow sfgmres_update_values)
-    struct BCopy {
-        int* rp = nullptr;
-        int* col = nullptr;
-        double* val = nullptr;
-        int ver = -1;
-    } bc[2];
-
-    // sketch gather lists (cached for one (s, zeta, kind, geometry version))
-    int sk_s = -1, sk_zeta = -1, sk_kind = -1, sk_ver = -1, sk_headroom = 0, sk_word = 0;
-    int* seg = nullptr;
-    uint16_t* ent = nullptr;
 
     // workspaces
     DevBuf U, W, sigma, normpart, hpart, cpart, C, Q, R, d, e, c0, rho, y, coef, hco, cyc;
@@ -245,35 +253,59 @@ bool is_device_ptr(const void* p) {
 // SpMV shape: one thread per row when every row is short (stencils), else the length-binned SpMV (0).
 int choose_vec(int64_t, int, int maxlen) { return maxlen <= 16 ? 1 : 0; }
 
-// Row blocks of one system: nblk a multiple of the SM count where possible, Bn a multiple of 32, <= kBlockRowsMax.
-// FP64 inner cycles size the blocks for all SMs but one QR cluster's: the sketched QR of step i runs beside the
-// fused inner kernel of step i+1, and a one-wave FP64 inner kernel whose CTAs share SMs with the QR cluster waits
-// on those stragglers (measured on 128^3: 137 us per step with 304 blocks, 112 us with 288).  The FP32 and BF16
-// inner kernels are short enough that the QR does not slow them, and all SMs serve them best.
-int single_block_rows(int n, int sms, int prec) {
-    if (prec == 0 && sms > 2 * kQrSms) sms -= kQrSms;
-    int q = 1, b = 32;
-    for (;;) {
-        const int64_t per = ((int64_t)n + (int64_t)sms * q - 1) / ((int64_t)sms * q);
-        b = (int)(((per + 31) / 32) * 32);
-        if (b <= kBlockRowsMax) break;
-        q *= 2;
-    }
-    return std::max(b, 32);
+// Row blocks of one system, a multiple of 32 rows, at most kBlockRowsMax.
+//
+// Large systems get two blocks per SM, the CTAs of the inner kernels that an SM holds (with one its 16 warps hide too little
+// latency: 72 to 50 us per step at 101^3 FP64, 47 to 35 us FP32).  A stencil's FP64 step leaves 8 SMs without a block: the
+// sketched QR of step i runs beside the inner kernel of step i+1, and a one-wave FP64 kernel whose CTAs share SMs with it
+// waits for those stragglers (128^3: 86 us per step with 288 blocks, 100 us with 304).  The FP32 and BF16 kernels are
+// short enough, and the length-binned SpMV latency bound enough (1M Zipf rows, FP64: 260 us with 304 blocks, 282 with
+// 287), that all SMs serve them best.
+//
+// Small systems take at most 128 blocks, one per SM, so that the QR's cluster finds SMs of its own: with more, both the
+// step and the QR get slower (32^3: 17.9 us per step FP64 against 25 with 256 blocks; 64^3 FP32: 20.4 against 24).  The
+// line, in stored entries, lies where the two met: FP64 48^3 (0.8M entries) 21.9 us with 128 blocks and 24.2 with 288, 64^3
+// (1.8M) 32.6 and 27.7; FP32 72^3 (2.6M) 21.7 and 24.7, 80^3 (3.6M) 26.4 and 25.4; Zipf rows 30,000 (0.8M) 27 and 30
+// (FP64), 18 and 21 (FP32), 100,000 (2.5M) 50 and 41, 38 and 30.
+int single_block_rows(int n, int64_t nnz, int sms, int prec, bool binned) {
+    const int64_t line = (prec == 0 || binned) ? 1200000 : 3200000;
+    int blocks;
+    if (nnz < line) blocks = std::max(sms - 24, std::min(sms, 16));
+    else blocks = 2 * ((prec == 0 && !binned && sms > 2 * kQrSms) ? sms - kQrSms : sms);
+    const int64_t most = ((int64_t)n + kBlockRowsMax - 1) / kBlockRowsMax;  // fewest blocks of the largest size
+    while (blocks < most) blocks *= 2;
+    const int64_t per = ((int64_t)n + blocks - 1) / blocks;
+    return std::max((int)(((per + 31) / 32) * 32), 32);
 }
 
-// Rows per block of a batch of systems (every system is cut into blocks of this size; the last block of a system
-// is ragged).  4096 rows = 8 rows per thread of a 512-thread CTA: enough independent rows per thread to hide the
-// gather latency, and the shared-memory block (32 KiB in FP64) leaves room for two CTAs per SM.
+// Rows per block where the blocks run in several waves (a batch of systems, or many right-hand sides of one): every system is
+// cut into blocks of this size, the last one ragged.  512-thread CTAs need some 8 to 10 rows per thread to hide the gathers'
+// latency and to carry the scalars that every block of the update forms again, and two CTAs per SM must find room for their
+// shared-memory blocks.  24 2D systems x 4, ms per solve with 2048 / 4096 / 5120 / 8192 rows: FP64 153 / 138 / 145 / 151, FP32 93 /
+// 84 / 89 / 91; 64^3 x 16 forward and backward: FP64 154 / 135 / 132 / 136, FP32 85 / 76 / 72 / 73.
 constexpr int kBatchBlockRows = 4096;
+constexpr int kRhsBlockRows = 5120;
 
-void set_list_geometry(sfgmres_ctx* h) {
+// Rows per block of a solve with nrhs right-hand sides per system.  Several right-hand sides of one system that fit the GPU
+// together in one wave share its blocks; more take kRhsBlockRows.
+int want_block_rows(const sfgmres_ctx* h, int nrhs) {
+    if (h->block_rows) return h->block_rows;
+    if (h->nsys > 1) return kBatchBlockRows;
+    const bool binned = choose_vec(h->nnz, h->n, h->maxlen) == 0;
+    if (nrhs == 1) return single_block_rows(h->n, h->nnz, h->sms, h->prec, binned);
+    const int64_t n = (int64_t)nrhs * h->n;
+    int rows = kRhsBlockRows;
+    if (n <= (int64_t)2 * h->sms * kRhsBlockRows) {
+        const int all = single_block_rows((int)n, nrhs * h->nnz, h->sms, h->prec, binned);
+        const int64_t per = std::max<int64_t>(1, (n + all - 1) / all / nrhs);  // blocks of one right-hand side
+        rows = (int)std::min<int64_t>(kRhsBlockRows, ((h->n + per - 1) / per + 31) / 32 * 32);
+    }
+    return rows;
+}
+
+void set_list_geometry(sfgmres_ctx* h, int Bq) {
     h->sys_Bq.assign(h->nsys, 0);
     h->sys_l0.assign(h->nsys + 1, 0);
-    int Bq;
-    if (h->block_rows) Bq = h->block_rows;
-    else if (h->nsys == 1) Bq = single_block_rows(h->n, h->sms, h->prec);
-    else Bq = kBatchBlockRows;
     int Bn = 32, nl = 0;
     for (int q = 0; q < h->nsys; ++q) {
         const int nq = h->sys_n[q];
@@ -285,7 +317,17 @@ void set_list_geometry(sfgmres_ctx* h) {
     h->sys_l0[h->nsys] = nl;
     h->nl = nl;
     h->Bn = Bn;
-    ++h->geo_ver;
+    h->geo_ver = ++h->geo_next;
+}
+
+// Makes the list blocks of a solve with nrhs right-hand sides current.  The previous ones are kept beside them with all that was
+// built for them (two sets in all), so that a program that alternates between single and many right-hand sides builds each
+// once.
+void choose_lists(sfgmres_ctx* h, int nrhs) {
+    const int Bq = want_block_rows(h, nrhs);
+    if (!h->sys_Bq.empty() && h->sys_Bq[0] == Bq) return;
+    if (!h->sys_Bq.empty()) std::swap(static_cast<ListSet&>(*h), h->other);
+    if (h->sys_Bq.empty() || h->sys_Bq[0] != Bq) set_list_geometry(h, Bq);
 }
 
 // Shared memory left on an SM beside the inner step's CTAs (one or two of them, by the number of row blocks; 8 KB each
@@ -587,7 +629,7 @@ int ensure_bins(sfgmres_ctx* h, bool transpose) {
 // (the bins of the current geometry), FP64 values.
 int ensure_bcopy(sfgmres_ctx* h, bool transpose) {
     const int t = transpose ? 1 : 0;
-    sfgmres_ctx::BCopy& B = h->bc[t];
+    ListSet::BCopy& B = h->bc[t];
     if (B.ver == h->geo_ver && B.rp) return 0;
     const int* rp = transpose ? h->rpT : h->rp;
     const int* col = transpose ? h->colT : h->col;
@@ -678,7 +720,7 @@ void plan_geometry(sfgmres_ctx* h, const Geo* g, bool transpose, Plan& P) {
     P.vec = transpose ? (h->vec_opt ? h->vec_opt : h->vecT) : h->vec;
     P.perm = (P.vec == 0) ? h->perm[transpose ? 1 : 0] : nullptr;
     P.cls = (P.vec == 0) ? h->cls[transpose ? 1 : 0] : nullptr;
-    const sfgmres_ctx::BCopy& B = h->bc[transpose ? 1 : 0];
+    const ListSet::BCopy& B = h->bc[transpose ? 1 : 0];
     const bool bc = (P.vec == 0) && B.rp && B.ver == h->geo_ver && h->bins_ver[transpose ? 1 : 0] == h->geo_ver;
     P.brp = bc ? B.rp : nullptr;
     P.bcol = bc ? B.col : nullptr;
@@ -831,6 +873,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
                                                     "side, FP64 inner cycles and no transpose");
         if ((rc = ensure_ilu(h))) return rc;
     }
+    choose_lists(h, nrhs);
     if ((rc = get_geometry(h, nrhs, &g))) return rc;
     if ((rc = build_sketch(h, s))) return rc;
     if (transpose && (rc = ensure_transpose(h))) return rc;
@@ -1531,7 +1574,7 @@ int sfgmres_create_batch(sfgmres_t* out, int32_t nsys, const int64_t* sys_n, int
                  "8 decreasing row_ptr, 16 column out of range, 32 column outside the row's system)", hbad);
         return bail(SFGMRES_ERR_INVALID_ARG, buf);
     }
-    set_list_geometry(h);
+    choose_lists(h, 1);
     h->vec = choose_vec(nnz, h->n, h->maxlen);
     cudaEventCreate(&h->ev_t0);
     cudaEventCreate(&h->ev_t1);
@@ -1563,21 +1606,18 @@ int sfgmres_destroy(sfgmres_t h) {
     if (h->val32) cudaFree(h->val32);
     for (void* q : {(void*)h->rpT, (void*)h->colT, (void*)h->srcT, (void*)h->valT, (void*)h->val32T})
         if (q) cudaFree(q);
-    if (h->seg) cudaFree(h->seg);
-    if (h->ent) cudaFree(h->ent);
-    for (int t = 0; t < 2; ++t) {
-        if (h->perm[t]) cudaFree(h->perm[t]);
-        if (h->cls[t]) cudaFree(h->cls[t]);
-    }
-    if (h->lb) cudaFree(h->lb);
-    for (auto& B : h->bc)
-        for (void* q : {(void*)B.rp, (void*)B.col, (void*)B.val})
+    for (ListSet* L : {static_cast<ListSet*>(h), &h->other}) {
+        for (void* q : {(void*)L->seg, (void*)L->ent, (void*)L->lb, (void*)L->sl_base, (void*)L->perm[0],
+                        (void*)L->perm[1], (void*)L->cls[0], (void*)L->cls[1]})
             if (q) cudaFree(q);
+        for (auto& B : L->bc)
+            for (void* q : {(void*)B.rp, (void*)B.col, (void*)B.val})
+                if (q) cudaFree(q);
+    }
     for (auto& S : h->sell)
         for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val})
             if (q) cudaFree(q);
     if (h->sl_sys) cudaFree(h->sl_sys);
-    if (h->sl_base) cudaFree(h->sl_base);
     DevBuf* bufs[] = {&h->U, &h->W, &h->sigma, &h->normpart, &h->hpart, &h->cpart, &h->C, &h->Q, &h->R, &h->d,
                       &h->e, &h->c0, &h->rho, &h->y, &h->coef, &h->hco, &h->cyc, &h->Vb, &h->Z, &h->nu, &h->Wo,
                       &h->opart, &h->npart, &h->npart2, &h->h1, &h->h2, &h->H, &h->cs, &h->sn, &h->g, &h->yo,
@@ -1623,10 +1663,8 @@ int sfgmres_set_option(sfgmres_t h, int32_t key, double v) {
     switch (key) {
         case SFGMRES_OPT_PRECISION:
             if (iv < 0 || iv > 2 || iv != v) return fail(h, SFGMRES_ERR_INVALID_ARG, "precision must be 0, 1 or 2");
-            if (iv != h->prec) {
-                h->prec = iv;
-                if (h->nsys == 1 && !h->block_rows) set_list_geometry(h);  // the default row blocks depend on it
-            }
+            h->prec = iv;
+            choose_lists(h, 1);  // the default row blocks depend on it
             return 0;
         case SFGMRES_OPT_ZETA:
             if (iv < 1 || iv > kMaxZeta || iv != v) return fail(h, SFGMRES_ERR_INVALID_ARG, "zeta must be 1..16");
@@ -1681,10 +1719,8 @@ int sfgmres_set_option(sfgmres_t h, int32_t key, double v) {
         case SFGMRES_OPT_BLOCK_ROWS:
             if (iv != v || !(iv == 0 || (iv >= 32 && iv <= kBlockRowsMax && iv % 32 == 0)))
                 return fail(h, SFGMRES_ERR_INVALID_ARG, "block rows must be 0 or a multiple of 32 in [32, 8192]");
-            if (iv != h->block_rows) {
-                h->block_rows = iv;
-                set_list_geometry(h);
-            }
+            h->block_rows = iv;
+            choose_lists(h, 1);
             return 0;
         default:
             return fail(h, SFGMRES_ERR_INVALID_ARG, "unknown option key");
@@ -1785,7 +1821,10 @@ int sfgmres_autotune(sfgmres_t h, int32_t nrhs, int32_t m, int32_t s, int32_t k,
     std::vector<int> cand;
     int maxn = 0;
     for (int q = 0; q < h->nsys; ++q) maxn = std::max(maxn, h->sys_n[q]);
-    const int base = (h->nsys == 1) ? single_block_rows(h->n, h->sms, h->prec) : kBatchBlockRows;
+    const int save_block = h->block_rows;
+    h->block_rows = 0;
+    const int base = want_block_rows(h, nrhs);
+    h->block_rows = save_block;
     for (int v : {base, base / 2, base / 4, base / 8, 512, 1024, 2048, 4096, 8192}) {
         v = std::min(kBlockRowsMax, std::max(256, (v / 32) * 32));
         if (v > ((maxn + 31) / 32) * 32 && v != base) continue;  // larger than every system: same as smaller ones
@@ -1795,7 +1834,7 @@ int sfgmres_autotune(sfgmres_t h, int32_t nrhs, int32_t m, int32_t s, int32_t k,
     std::vector<int> vecs = {0};
     if (h->maxlen > 16)
         for (int v : {8, 32}) vecs.push_back(v);  // the inner kernel has 8- and 32-lane variants
-    const int save_block = h->block_rows, save_vec = h->vec_opt, save_graph = h->use_graph;
+    const int save_vec = h->vec_opt, save_graph = h->use_graph;
     const int steps = std::min(m, 8);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
@@ -1804,7 +1843,6 @@ int sfgmres_autotune(sfgmres_t h, int32_t nrhs, int32_t m, int32_t s, int32_t k,
     int best_b = save_block, best_v = save_vec;
     for (int bq : cand) {
         h->block_rows = bq;
-        set_list_geometry(h);
         for (int vv : vecs) {
             h->vec_opt = vv;
             h->vec = vv ? vv : choose_vec(h->nnz, h->n, h->maxlen);
@@ -1843,13 +1881,13 @@ int sfgmres_autotune(sfgmres_t h, int32_t nrhs, int32_t m, int32_t s, int32_t k,
         h->block_rows = save_block;
         h->vec_opt = save_vec;
         h->vec = save_vec ? save_vec : choose_vec(h->nnz, h->n, h->maxlen);
-        set_list_geometry(h);
+        choose_lists(h, nrhs);
         return rc;
     }
     h->block_rows = best_b;
     h->vec_opt = best_v;
     h->vec = best_v ? best_v : choose_vec(h->nnz, h->n, h->maxlen);
-    set_list_geometry(h);
+    choose_lists(h, nrhs);
     if (block_rows_out) *block_rows_out = h->sys_Bq.empty() ? 0 : h->sys_Bq[0];
     if (spmv_vector_out) *spmv_vector_out = h->vec;
     if (step_ms_out) *step_ms_out = best;
@@ -1870,8 +1908,9 @@ int sfgmres_update_values(sfgmres_t h, const double* vals) {
         launch_gather_vals(h->nnz, h->srcT, h->val, h->valT, h->st);
         if (h->val32T) k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, h->valT, h->val32T);
     }
+    for (auto& B : h->other.bc) B.ver = -1;  // the other list blocks' copies: rebuilt at their next use
     for (int t = 0; t < 2; ++t) {  // the length-binned copies' values
-        sfgmres_ctx::BCopy& B = h->bc[t];
+        ListSet::BCopy& B = h->bc[t];
         if (B.rp && B.ver == h->geo_ver && h->perm[t])
             launch_bcopy_fill(h->nl, t ? h->rpT : h->rp, nullptr, t ? h->valT : h->val, h->lb, h->lb + h->nl,
                               h->perm[t], B.rp, nullptr, B.val, h->st);
@@ -2374,6 +2413,7 @@ int sfgmres_spmv(sfgmres_t h, const double* xv, double* yv) {
     if (!xv || !yv) return fail(h, SFGMRES_ERR_INVALID_ARG, "NULL pointer");
     CK(cudaSetDevice(h->dev));
     Geo* g = nullptr;
+    choose_lists(h, 1);
     int rc = get_geometry(h, 1, &g);
     if (rc) return rc;
     if (h->vec == 0 && (rc = ensure_bins(h, false))) return rc;

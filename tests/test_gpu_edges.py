@@ -78,3 +78,25 @@ sys.exit(info['status'])
 """
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     assert subprocess.run([sys.executable, "-c", code], cwd=root).returncode == 0
+
+
+# single and many right-hand sides use row blocks of different sizes on one handle: alternating between them, with new values
+# in between, gives what fresh handles give, bit for bit
+@pytest.mark.parametrize("kind", ["convdiff", "zipf"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_alternating_numbers_of_right_hand_sides(Solver, kind, precision):
+    A = workloads.convdiff(40, (30.0, 10.0)) if kind == "convdiff" else workloads.random_zipf(6000, seed=3)
+    par = dict(m=30, s=120, k=2, tol=1e-8)
+    one, many = dev_vec(workloads.rhs(A.n, seed=0)), dev_vec(workloads.rhs(7 * A.n, seed=1))
+    vals = [dev_vec(A.val), dev_vec(A.val * np.linspace(1.0, 1.5, A.nnz))]
+
+    def call(sv, nrhs):
+        return (sv.solve(one, **par) if nrhs == 1 else sv.solve_batch(many, nrhs=nrhs, **par))[0].cpu().numpy()
+
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, precision=precision)
+    for which, nrhs in ((0, 1), (0, 7), (0, 1), (1, 1), (1, 7), (0, 7), (1, 1)):
+        sv.update_values(vals[which])
+        fresh = Solver(A.n, A.row_ptr, A.col, vals[which].cpu().numpy(), sketch_seed=1, precision=precision)
+        assert np.array_equal(call(sv, nrhs), call(fresh, nrhs))
+        fresh.close()
+    sv.close()

@@ -277,87 +277,73 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// Per problem (one CTA of 128 threads): y = R_k^{-1} d by column-oriented back substitution, coef_l = y_l sigma_l.
-// Step l divides by r_ll and subtracts y_l times column l of R from the rows above it, one row per thread; the next
-// column is loaded while the current one is applied, so each step costs a barrier rather than an L2 round trip.
+// Per problem (one CTA): y = R_k^{-1} d by back substitution, coef_l = y_l sigma_l, in panels of 32 columns from the last.
+// A panel's triangle is one warp's: lane q holds row q of the right-hand side, its row of the triangle (one wave of loads)
+// and 1 / r_qq (the divisions of all rows at once); step l forms y_l in lane l (the product with the reciprocal and one
+// correction step, as accurate as the division), shuffles it to the other lanes, and the rows above l subtract r_ql y_l.
+// The other rows then subtract the panel's 32 products, a thread per row, whose entries of the panel were loaded while the
+// triangle was solved.  A chain of k dependent steps, bound by FP64 and shuffle
+// latency: 22 us on the mean of a 128^3 solve's cycles (k = 77) and 57 us at k = 200, against 70 and 182 us with a block barrier
+// pair and a division on the path of every column.
 constexpr int kLsThreads = 128;
 __global__ void __launch_bounds__(kLsThreads) k_inner_ls(const Plan P) {
     extern __shared__ double rhs[];  // [k]
-    __shared__ double yl_sh;
+    __shared__ double ysh[32];
     const int p = blockIdx.x, m = P.m;
     if (P.pflag[p] & 1) return;
-    const double* R = P.R + (int64_t)p * m * m;  // column-major: R[l*m + q] = R_{q,l}
-    const double* d = P.d + (int64_t)p * m;
-    const double* sigma = P.sigma + (int64_t)p * (m + 1);
-    double* y = P.y + (int64_t)p * m;
-    double* coef = P.coef + (int64_t)p * m;
+    const double* __restrict__ R = P.R + (int64_t)p * m * m;  // column-major: R[l*m + q] = R_{q,l}
+    const double* __restrict__ d = P.d + (int64_t)p * m;
+    const double* __restrict__ sigma = P.sigma + (int64_t)p * (m + 1);
+    double* __restrict__ y = P.y + (int64_t)p * m;
+    double* __restrict__ coef = P.coef + (int64_t)p * m;
     const int k = P.cyc[p].k;
-    if (k <= 32) {
-        // one warp: lane q holds row q of the right-hand side, its row of R (one load wave) and 1 / r_qq (the
-        // divisions of all rows at once); step l forms y_l = rhs_l (1 / r_ll) in lane l, shuffles it to the other
-        // lanes, and the rows above l subtract r_ql y_l in parallel -- warp shuffles instead of block barriers and one
-        // FP64 multiply-add per step on the critical path
-        if (threadIdx.x >= 32) return;
-        const int q = threadIdx.x;
-        double r = (q < k) ? d[q] : 0.0;
-        double rq[32];
+    const int tid = threadIdx.x;
+    for (int l = tid; l < k; l += kLsThreads) rhs[l] = d[l];
+    __syncthreads();
+    for (int l0 = (k - 1) & ~31; l0 >= 0; l0 -= 32) {  // columns l0 .. l1 - 1
+        const int w = min(32, k - l0);
+        double rq[32];  // warp 0: row l0 + lane of the triangle; the others: their first row's entries of the panel
+        const int first = (tid < 32) ? l0 + tid : tid - 32;
+        const bool mine = (tid < 32) ? tid < w : first < l0;
 #pragma unroll
-        for (int l = 0; l < 32; ++l) rq[l] = (l < k && q <= l) ? R[(int64_t)l * m + q] : 0.0;
-        double rqq = 1.0;
+        for (int c = 0; c < 32; ++c)
+            rq[c] = (mine && c < w && (tid >= 32 || tid <= c)) ? R[(int64_t)(l0 + c) * m + first] : 0.0;
+        if (tid < 32) {
+            double r = mine ? rhs[first] : 0.0;
+            double rqq = 1.0;
 #pragma unroll
-        for (int l = 0; l < 32; ++l)
-            if (l == q && q < k) rqq = rq[l];
-        const double inv = 1.0 / rqq;
-        for (int l = k - 1; l >= 0; --l) {
-            double rql = 0.0;  // r_ql of this lane's row
+            for (int c = 0; c < 32; ++c)
+                if (c == tid && mine) rqq = rq[c];
+            const double inv = 1.0 / rqq;
+            double yq = 0.0;
 #pragma unroll
-            for (int u = 0; u < 32; ++u)
-                if (u == l) rql = rq[u];
-            const double yl = __shfl_sync(0xffffffffu, r * inv, l);
-            if (q < l) r = fma(-rql, yl, r);
-            if (q == l) {
-                y[l] = yl;
-                coef[l] = yl * sigma[l];
+            for (int c = 31; c >= 0; --c) {
+                if (c >= w) continue;
+                double t = r * inv;
+                t = fma(fma(-t, rqq, r), inv, t);
+                const double yl = __shfl_sync(0xffffffffu, t, c);
+                if (tid == c) yq = yl;
+                if (tid < c) r = fma(-rq[c], yl, r);
+            }
+            if (mine) {
+                ysh[tid] = yq;
+                y[first] = yq;
+                coef[first] = yq * sigma[first];
+            } else {
+                ysh[tid] = 0.0;
             }
         }
-        return;
-    }
-    for (int l = threadIdx.x; l < k; l += kLsThreads) rhs[l] = d[l];
-    // this thread's rows q = threadIdx.x + 128 j; its entries of the current column l are loaded one column ahead
-    constexpr int kRows = kMaxM / kLsThreads;
-    double col[kRows];
-    auto load_col = [&](int l) {
+        __syncthreads();
+        if (tid >= 32) {
+            for (int q = first; q < l0; q += kLsThreads - 32) {
+                double r = rhs[q];
 #pragma unroll
-        for (int j = 0; j < kRows; ++j) {
-            const int q = threadIdx.x + kLsThreads * j;
-            col[j] = (l >= 0 && q <= l) ? R[(int64_t)l * m + q] : 0.0;
+                for (int c = 31; c >= 0; --c)
+                    r = fma(-((q == first) ? rq[c] : (c < w ? R[(int64_t)(l0 + c) * m + q] : 0.0)), ysh[c], r);
+                rhs[q] = r;
+            }
         }
-    };
-    load_col(k - 1);
-    __syncthreads();
-    for (int l = k - 1; l >= 0; --l) {
-        if (threadIdx.x == (l % kLsThreads)) {
-            double rll = 0.0;
-#pragma unroll
-            for (int j = 0; j < kRows; ++j)
-                if (threadIdx.x + kLsThreads * j == l) rll = col[j];
-            const double yl = rhs[l] / rll;
-            yl_sh = yl;
-            y[l] = yl;
-            coef[l] = yl * sigma[l];
-        }
-        double cur[kRows];
-#pragma unroll
-        for (int j = 0; j < kRows; ++j) cur[j] = col[j];
-        load_col(l - 1);
-        __syncthreads();  // y_l is in yl_sh
-        const double yl = yl_sh;
-#pragma unroll
-        for (int j = 0; j < kRows; ++j) {
-            const int q = threadIdx.x + kLsThreads * j;
-            if (q < l) rhs[q] -= cur[j] * yl;
-        }
-        __syncthreads();  // rhs[l - 1] is final before its owner divides; yl_sh is free again
+        __syncthreads();
     }
 }
 
@@ -365,11 +351,13 @@ __global__ void __launch_bounds__(kLsThreads) k_inner_ls(const Plan P) {
 // two FP32 parts and the sum is carried as an unevaluated FP32 pair (TwoSum, and FMA for the exact product error),
 // close to FP64 accuracy on the FP32 pipe.  Every row's sum runs over l in order.
 //
-// A pass over the k basis vectors with one multiply-add per value, bound by HBM (FP64 with the FP64 pipe close behind).
+// A pass over the k basis vectors with one multiply-add per value: bound by HBM for FP32 and BF16 bases, by the FP64 pipe
+// for FP64 ones.
 // Each row block is cut into pieces of kGemvThreads x R rows, one CTA each (grid y), so that the GPU holds as many
 // threads as fit whatever the block size, and a thread loads L columns of its R rows (kGemvThreads apart: coalesced at
-// any alignment) before it uses them.  128^3, k = 100: FP64 530 -> 290 us (5.8 TB/s), FP32 775 -> 148 us (5.8 TB/s), both
-// against one CTA of 256 threads per row block with one row's column in flight per thread.
+// any alignment) before it uses them.  Means over the cycles of a 128^3 solve: FP64 (77 columns) 530 -> 287 us (1.1 TFLOP/s,
+// this GPU's FP64 rate), FP32 (93 columns) 775 -> 148 us (5.4 TB/s), both against one CTA of 256 threads per row block with
+// one row's column in flight per thread.
 constexpr int kGemvThreads = 256;
 template <typename VT> struct GemvShape { static constexpr int R = 4, L = 4; };       // FP32, BF16
 template <> struct GemvShape<double> { static constexpr int R = 2, L = 4; };

@@ -7,6 +7,7 @@
 // outer FGMRES step to read every problem's convergence flags and to mark the problems to finalise or retire.
 #include "../../include/sfgmres.h"
 #include "kernels.h"
+#include "spmv.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -46,6 +47,7 @@ struct Geo {
 };
 
 constexpr int kGeoCache = 4;
+constexpr int64_t kEntryPad = 4;  // entries the CSR arrays hold beyond the last (the staged SpMV copies 16 bytes at a time)
 
 }  // namespace
 
@@ -563,7 +565,7 @@ int get_geometry(sfgmres_ctx* h, int nrhs, Geo** out) {
 int ensure_f32(sfgmres_ctx* h, bool transpose) {
     float*& v32 = transpose ? h->val32T : h->val32;
     if (v32) return 0;
-    CK(cudaMalloc(&v32, std::max<int64_t>(h->nnz, 1) * sizeof(float)));
+    CK(cudaMalloc(&v32, (h->nnz + kEntryPad) * sizeof(float)));
     k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, transpose ? h->valT : h->val, v32);
     CK(cudaGetLastError());
     return 0;
@@ -574,7 +576,7 @@ int ensure_f32(sfgmres_ctx* h, bool transpose) {
 // sketch lists serve both.
 int ensure_transpose(sfgmres_ctx* h) {
     if (h->rpT) return 0;
-    const int64_t nz = std::max<int64_t>(h->nnz, 1);
+    const int64_t nz = h->nnz + kEntryPad;
     int* counts = nullptr;
     int* mx = nullptr;
     CK(cudaMalloc(&h->rpT, ((size_t)h->n + 1) * sizeof(int)));
@@ -718,6 +720,7 @@ void plan_geometry(sfgmres_ctx* h, const Geo* g, bool transpose, Plan& P) {
     P.val = transpose ? h->valT : h->val;
     P.val32 = transpose ? h->val32T : h->val32;
     P.vec = transpose ? (h->vec_opt ? h->vec_opt : h->vecT) : h->vec;
+    P.maxlen = transpose ? h->maxlenT : h->maxlen;
     P.perm = (P.vec == 0) ? h->perm[transpose ? 1 : 0] : nullptr;
     P.cls = (P.vec == 0) ? h->cls[transpose ? 1 : 0] : nullptr;
     const ListSet::BCopy& B = h->bc[transpose ? 1 : 0];
@@ -864,6 +867,16 @@ int ensure_ilu(sfgmres_ctx* h) {
     return 0;
 }
 
+// Shared memory of the staged SpMV beside the FP32 inner kernels' blocks of w' (16 warps, and up to 16 bytes of alignment).
+size_t stage_smem(int maxlen) { return 16 * (size_t)stage_bytes<float>(maxlen) + 16; }
+
+// Whether the one-thread-per-row SpMV of FP32 and BF16 inner cycles stages its entries: where that leaves the SM as many of the
+// kernels' CTAs as it holds without (two, or one if the blocks do not fill the SMs).
+bool stage_fits(const sfgmres_ctx* h, int nblk, int maxlen) {
+    const size_t block = ((size_t)h->Bn + 1) * 4 + stage_smem(maxlen);
+    return (nblk > h->sms ? 2 : 1) * (block + 8 * 1024) <= 226 * 1024;
+}
+
 int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Geo** geo_out, bool transpose = false) {
     int rc;
     Geo* g = nullptr;
@@ -878,12 +891,12 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = build_sketch(h, s))) return rc;
     if (transpose && (rc = ensure_transpose(h))) return rc;
     if (h->prec != kFP64 && (rc = ensure_f32(h, transpose))) return rc;
-    {
-        const int v = transpose ? (h->vec_opt ? h->vec_opt : h->vecT) : h->vec;
-        if (v == 0 && (rc = ensure_bins(h, transpose))) return rc;
-        if (v == 0 && (rc = ensure_bcopy(h, transpose))) return rc;
-        if (v == 1 && h->prec == kFP64 && (rc = ensure_sell(h, transpose))) return rc;
-    }
+    const int vec = transpose ? (h->vec_opt ? h->vec_opt : h->vecT) : h->vec;
+    const int maxlen = transpose ? h->maxlenT : h->maxlen;
+    const bool staged = vec == 1 && h->prec != kFP64 && stage_fits(h, g->nblk, maxlen);
+    if (vec == 0 && (rc = ensure_bins(h, transpose))) return rc;
+    if (vec == 0 && (rc = ensure_bcopy(h, transpose))) return rc;
+    if (vec == 1 && h->prec == kFP64 && (rc = ensure_sell(h, transpose))) return rc;
     const size_t vt = (h->prec == kFP64) ? 8 : (h->prec == kFP32 ? 4 : 2);
     const size_t at = (h->prec == kFP64) ? 8 : 4;
     const size_t N = (size_t)g->N;
@@ -897,7 +910,8 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->hpart, nb * kMaxTrunc * at))) return rc;
     if ((rc = ensure(h, h->cpart, nb * S * at))) return rc;
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
-    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at));
+    const size_t stage = staged ? stage_smem(maxlen) : 0;
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage));
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;
@@ -968,6 +982,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     P.hco = (double*)h->hco.p;
     P.cyc = (CycleState*)h->cyc.p;
     P.qr = qs;
+    P.staged = staged ? 1 : 0;
     P.jmax = jmax;
     P.Vb = (double*)h->Vb.p;
     P.Z = (double*)h->Z.p;
@@ -1118,7 +1133,7 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
                           (const void*)P.xin, (const void*)P.ilu.lu, (const void*)P.brp, (const void*)P.bcol,
                           (const void*)P.bval})
         u(p);
-    for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
+    for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.staged, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
                       (int64_t)P.s, (int64_t)P.zeta, (int64_t)P.kind, (int64_t)P.sk_headroom, (int64_t)P.prec,
                       (int64_t)P.m, (int64_t)P.t, (int64_t)P.qr.cluster, (int64_t)P.qr.staged, (int64_t)P.jmax, (int64_t)h->c3,
                       (int64_t)h->profile, (int64_t)P.gwait_extra, (int64_t)P.outer_variant})
@@ -1538,8 +1553,8 @@ int sfgmres_create_batch(sfgmres_t* out, int32_t nsys, const int64_t* sys_n, int
     int* bad = nullptr;
     int* dmoff = nullptr;
     if (cudaMalloc(&h->rp, (n + 1) * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&h->col, std::max<int64_t>(nnz, 1) * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&h->val, std::max<int64_t>(nnz, 1) * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&h->col, (nnz + kEntryPad) * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&h->val, (nnz + kEntryPad) * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&rp64, (n + 1) * sizeof(int64_t)) != cudaSuccess || cudaMalloc(&bad, 2 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&dmoff, (nsys + 1) * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();

@@ -16,6 +16,8 @@ namespace sfg {
 // Template value of k_inner_spmv's lanes-per-row parameter for one thread per row reading the SELL-32 copy of A
 // (the FP64 inner cycle); 1 is one thread per row reading the CSR arrays.
 constexpr int kVecSell = -1;
+// The same for one thread per row with the CSR entries staged in shared memory (spmv_rows_staged).
+constexpr int kVecStaged = -2;
 
 __device__ __forceinline__ bool cycle_idle(const Plan& P, int p, int i) {
     const CycleState* c = P.cyc + p;
@@ -182,6 +184,37 @@ __device__ __forceinline__ int spmv_dots_scalar(int N, const int* __restrict__ r
     return emax;
 }
 
+// Phase 1, one thread per row with the entries staged in shared memory: as spmv_dots_scalar.
+template <int NW, typename MT, typename VT, typename AT>
+__device__ __forceinline__ int spmv_dots_staged(int N, const int* __restrict__ rp, const int* __restrict__ col,
+                                                const MT* __restrict__ val, const VT* __restrict__ Ub,
+                                                const VT* __restrict__ xg, int lo, int v0, int len, int cs,
+                                                AT* __restrict__ wblk, AT* __restrict__ W, AT (&acc)[NW > 0 ? NW : 1],
+                                                unsigned char* buf, int maxlen) {
+    const unsigned long long pol = l2_keep_policy();  // window rows and w' are read again by the update
+    int emax = 1;
+    AT uw[NW > 0 ? NW : 1];
+    spmv_rows_staged<MT, VT, AT>(
+        rp + (v0 - cs), col, val, xg + cs, len, buf, maxlen,
+        [&](int k) {
+#pragma unroll
+            for (int q = 0; q < NW; ++q)
+                uw[q] = (k < len) ? ld_keep(Ub + (int64_t)(lo + q) * N + v0 + k, pol) : AT(0);
+            const int kp = k + kXPrefetchAhead * (int)blockDim.x;
+            if (kp < len) prefetch_l2(xg + v0 + kp);  // x of the row's own column, kXPrefetchAhead row group(s) ahead
+        },
+        [&](int k, AT sum) {
+            if (k < len) {
+                st_keep(W + v0 + k, sum, pol);
+                wblk[k] = sum;
+            }
+#pragma unroll
+            for (int q = 0; q < NW; ++q) acc[q] += uw[q] * sum;
+            emax = max(emax, exp_of(sum));
+        });
+    return emax;
+}
+
 // Phase 1 tail for the sub-warp path (w' already in shared memory): store w' and accumulate the window dots.
 template <int NW, typename VT, typename AT>
 __device__ __forceinline__ int dots_pass(int N, int v0, int len, const VT* __restrict__ Ub, int lo,
@@ -199,6 +232,16 @@ __device__ __forceinline__ int dots_pass(int N, int v0, int len, const VT* __res
         for (int q = 0; q < NW; ++q) acc[q] += ld_keep(Ub + (int64_t)(lo + q) * N + r, pol) * w;
     }
     return emax;
+}
+
+// Byte offset of the stage area behind the shared block of w' (rows + 1 slots), on a 16-byte boundary.
+__host__ __device__ constexpr int stage_offset(int rows, int slot) { return ((rows + 1) * slot + 15) & ~15; }
+
+// Dynamic shared memory of the inner step's kernels.
+template <int V, typename MT, typename AT>
+static size_t step_smem(const Plan& p) {
+    if (V == kVecStaged) return stage_offset(p.Bn, (int)sizeof(AT)) + 16 * (size_t)stage_bytes<MT>(p.maxlen);
+    return (size_t)(p.Bn + 1) * sizeof(AT);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -230,6 +273,9 @@ __device__ __forceinline__ bool inner_spmv_part(const Plan& P, int i, const MT* 
     if constexpr (V == kVecSell) {
         emax = spmv_dots_sell<NW>(N, P.sl_off, P.sl_len, P.sl_col, val, P.sl_base[bi.list], Ub, xg, i, lo, bi.v0,
                                   bi.len, bi.cs, wblk, W, acc);
+    } else if constexpr (V == kVecStaged) {
+        unsigned char* buf = reinterpret_cast<unsigned char*>(wblk) + stage_offset(Bn, (int)sizeof(AT));
+        emax = spmv_dots_staged<NW>(N, P.rp, P.col, val, Ub, xg, lo, bi.v0, bi.len, bi.cs, wblk, W, acc, buf, P.maxlen);
     } else if constexpr (V == 1) {
         emax = spmv_dots_scalar<NW>(N, P.rp, P.col, val, Ub, xg, i, lo, bi.v0, bi.len, bi.cs, wblk, W, acc);
     } else {
@@ -789,7 +835,7 @@ __global__ void __maxnreg__(56) k_inner_step(const Plan P, int i, const MT* __re
 
 template <int V, int U, int NW, typename MT, typename VT, typename AT>
 static void inner_spmv_v(const Plan& p, int i, const MT* val) {
-    const size_t sm = (size_t)(p.Bn + 1) * sizeof(AT);
+    const size_t sm = step_smem<V, MT, AT>(p);
     set_smem((const void*)k_inner_spmv<V, U, NW, MT, VT, AT>, sm);
     k_inner_spmv<V, U, NW, MT, VT, AT><<<p.nblk, 512, sm, p.st>>>(p, i, val);
 }
@@ -801,6 +847,8 @@ static void inner_spmv_nw(const Plan& p, int i, const MT* val) {
         if constexpr (sizeof(MT) == 8) {  // FP64 one thread per row reads the SELL-32 copy (always built for it)
             if (p.sl_off) inner_spmv_v<kVecSell, 1, NW, MT, VT, AT>(p, i, p.sl_val);
             else inner_spmv_v<8, 4, NW, MT, VT, AT>(p, i, val);
+        } else if (p.staged) {
+            inner_spmv_v<kVecStaged, 1, NW, MT, VT, AT>(p, i, val);
         } else {
             inner_spmv_v<1, 1, NW, MT, VT, AT>(p, i, val);
         }
@@ -830,7 +878,7 @@ static void inner_spmv_t(const Plan& p, int i, const MT* val) {
 template <int V, int U, int NW, typename MT, typename VT, typename AT>
 static bool inner_step_v(const Plan& p, int i, const MT* val, bool last) {
     const void* fn = (const void*)k_inner_step<V, U, NW, MT, VT, AT>;
-    const size_t sm = (size_t)(p.Bn + 1) * sizeof(AT);
+    const size_t sm = step_smem<V, MT, AT>(p);
     set_smem(fn, sm);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 512, sm) != cudaSuccess) {
@@ -851,6 +899,8 @@ static bool inner_step_nw(const Plan& p, int i, const MT* val, bool last) {
     if (p.vec == 1) {
         if constexpr (sizeof(MT) == 8) {  // FP64 one thread per row reads the SELL-32 copy
             return p.sl_off ? inner_step_v<kVecSell, 1, NW, MT, VT, AT>(p, i, p.sl_val, last) : false;
+        } else if (p.staged) {
+            return inner_step_v<kVecStaged, 1, NW, MT, VT, AT>(p, i, val, last);
         } else {
             return inner_step_v<1, 1, NW, MT, VT, AT>(p, i, val, last);
         }

@@ -59,6 +59,8 @@ struct Plan {
     const double* val = nullptr;
     const float* val32 = nullptr;  // FP32 copy (inner FP32/BF16 modes)
     int vec = 8;                   // SpMV lanes per row (1 = one thread per row, 0 = length-binned)
+    int maxlen = 0;                // longest row
+    int staged = 0;                // vec == 1: the inner kernels stage the CSR entries in shared memory
     // SELL-32 copy for the one-thread-per-row FP64 inner SpMV (vec == 1, FP64 inner cycles): slice widths as prefix
     // sums in units of 32 entries, per-lane row lengths, columns and values in slice order, and the first slice of
     // every list block

@@ -64,6 +64,112 @@ __device__ __forceinline__ void spmv_rows_scalar(const int* __restrict__ rp, con
     }
 }
 
+// ---- one thread per row with the entries staged in shared memory ----
+// A warp takes 32 consecutive rows at a time.  Their entries are one stretch of the CSR arrays, which the warp copies
+// into its own part of shared memory with asynchronous 16-byte copies (from the 16-byte boundary at or below; the
+// arrays are padded, so a copy may run past the last entry), one group of rows ahead: a group's columns and values are there
+// when its turn comes, every copy is coalesced whatever the row lengths, and what a row waits for is one round of gathers of x
+// (up to eight in flight per lane).  Read straight from global memory, lanes 7 entries apart touch 20 sectors per load, and a
+// row of 7 entries waits for two rounds of loads and gathers.  A group's values go to registers before its last products,
+// which frees the buffer for the next group's copy.  Rows are summed in entry order, a warp issuing as many products as its
+// longest row.  128^3 solve to 1e-12 with FP32 inner cycles: 45.8 -> 42.3 ms.  FP64 inner cycles keep the SELL-32 copy (staged:
+// 46.4 -> 57.6 ms, the buffers of two CTAs beside their blocks of w' leave 28 KB of L1).
+template <typename MT>
+__host__ __device__ constexpr int stage_bytes(int maxlen) {  // one warp's buffer for rows of at most maxlen entries
+    return 32 * maxlen * (4 + (int)sizeof(MT)) + 32;
+}
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Starts the copy of entries [a0, a1) into a warp's buffer (columns at cdst, values at vdst).
+template <typename MT>
+__device__ __forceinline__ void stage_issue(const int* __restrict__ col, const MT* __restrict__ val, int a0, int a1,
+                                            unsigned cdst, unsigned vdst, int lane) {
+    constexpr int VP = 16 / (int)sizeof(MT);
+    const int ca = a0 & ~3, va = a0 & ~(VP - 1);
+    for (int u = lane; ca + 4 * u < a1; u += 32) cp_async16(cdst + 16 * u, col + ca + 4 * u);
+    for (int u = lane; va + VP * u < a1; u += 32) cp_async16(vdst + 16 * u, val + va + VP * u);
+}
+
+// Entries pk .. pk+CNT-1 of the lane's row (its first entry at cs, vs in shared memory); `release` runs once the
+// values are in registers.
+template <int CNT, typename MT, typename XT, typename AT, typename Release>
+__device__ __forceinline__ void staged_chunk(const int* cs, const MT* vs, const XT* __restrict__ x, int len, int pk,
+                                             AT& sum, Release&& release) {
+    AT xv[CNT], v[CNT];
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) xv[q] = (pk + q < len) ? load_as(x + cs[pk + q], AT()) : AT(0);
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) v[q] = (pk + q < len) ? (AT)vs[pk + q] : AT(0);
+    release();
+#pragma unroll
+    for (int q = 0; q < CNT; ++q)
+        if (pk + q < len) sum += v[q] * xv[q];
+}
+
+// For the len rows from matrix row r0 on (row pointers rpm = rp + r0): pre(k) before local row k's products (loads that
+// should be in flight with them), then emit(k, sum).  Lanes past the last row call both with k >= len.  buf: the CTA's
+// stage area (blockDim / 32 buffers of stage_bytes(maxlen)).
+template <typename MT, typename XT, typename AT, typename Pre, typename Emit>
+__device__ __forceinline__ void spmv_rows_staged(const int* __restrict__ rpm, const int* __restrict__ col,
+                                                 const MT* __restrict__ val, const XT* __restrict__ x, int len,
+                                                 unsigned char* buf, int maxlen, Pre&& pre, Emit&& emit) {
+    const int lane = threadIdx.x & 31;
+    unsigned char* mine = buf + (threadIdx.x >> 5) * stage_bytes<MT>(maxlen);
+    int* cbuf = reinterpret_cast<int*>(mine);
+    MT* vbuf = reinterpret_cast<MT*>(mine + 128 * maxlen + 16);
+    const unsigned cdst = (unsigned)__cvta_generic_to_shared(cbuf), vdst = (unsigned)__cvta_generic_to_shared(vbuf);
+    constexpr int VP = 16 / (int)sizeof(MT);
+    int kw = threadIdx.x & ~31;
+    if (kw >= len) return;
+    // first entry and length of the lane's row in the group at k0 (past the last row: its end, 0)
+    auto extent = [&](int k0, int& a, int& l) {
+        a = __ldg(rpm + min(k0 + lane, len));
+        l = __ldg(rpm + min(k0 + lane + 1, len)) - a;
+    };
+    auto issue = [&](int a, int l) {
+        stage_issue(col, val, __shfl_sync(0xffffffffu, a, 0), __shfl_sync(0xffffffffu, a + l, 31), cdst, vdst, lane);
+    };
+    int a, rl, an = 0, rln = 0;
+    extent(kw, a, rl);
+    issue(a, rl);
+    if (kw + (int)blockDim.x < len) extent(kw + blockDim.x, an, rln);
+    for (; kw < len; kw += blockDim.x) {  // warp-uniform loop
+        const bool more = kw + (int)blockDim.x < len;
+        pre(kw + lane);
+        const int a0 = __shfl_sync(0xffffffffu, a, 0);
+        const int* cs = cbuf + (a - (a0 & ~3));
+        const MT* vs = vbuf + (a - (a0 & ~(VP - 1)));
+        const int wm = (int)__reduce_max_sync(0xffffffffu, (unsigned)rl);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        AT sum = AT(0);
+        auto release = [&]() {  // every lane has read the buffer: the next group's entries may come in
+            __syncwarp();
+            if (more) issue(an, rln);
+        };
+        int pk = 0;
+        for (; pk + 8 < wm; pk += 8) staged_chunk<8>(cs, vs, x, rl, pk, sum, [] {});
+        switch (wm - pk) {
+            case 1: staged_chunk<1>(cs, vs, x, rl, pk, sum, release); break;
+            case 2: staged_chunk<2>(cs, vs, x, rl, pk, sum, release); break;
+            case 3: staged_chunk<3>(cs, vs, x, rl, pk, sum, release); break;
+            case 4: staged_chunk<4>(cs, vs, x, rl, pk, sum, release); break;
+            case 5: staged_chunk<5>(cs, vs, x, rl, pk, sum, release); break;
+            case 6: staged_chunk<6>(cs, vs, x, rl, pk, sum, release); break;
+            case 7: staged_chunk<7>(cs, vs, x, rl, pk, sum, release); break;
+            case 8: staged_chunk<8>(cs, vs, x, rl, pk, sum, release); break;
+            default: release(); break;  // rows without entries
+        }
+        emit(kw + lane, sum);
+        a = an;
+        rl = rln;
+        if (kw + 2 * (int)blockDim.x < len) extent(kw + 2 * (int)blockDim.x, an, rln);
+    }
+}
+
 // Same result with each row handled by a sub-warp of V lanes; a warp processes U sub-warp rows at once (all their
 // loads issued before the FMAs).  For a fixed unroll slot the warp's sub-warps read consecutive rows, so the
 // col/val streams are read in contiguous segments.  Per-row sums are combined by a fixed xor-shuffle tree.

@@ -100,3 +100,29 @@ def test_alternating_numbers_of_right_hand_sides(Solver, kind, precision):
         assert np.array_equal(call(sv, nrhs), call(fresh, nrhs))
         fresh.close()
     sv.close()
+
+
+# FP32 inner cycles: the staged SpMV with rows of 0 to 16 entries in every order, row groups cut by the block's and the
+# system's end, entries that start anywhere within 16 bytes
+@pytest.mark.parametrize("n,maxlen,block_rows", [(31, 1, 32), (33, 16, 32), (1000, 5, 512), (5000, 9, 544), (4097, 16, 1024),
+                                                 (20_000, 3, 8192)])
+def test_staged_spmv_with_ragged_rows(Solver, n, maxlen, block_rows):
+    rng = np.random.default_rng(n + maxlen)
+    length = rng.integers(0, maxlen + 1, n)
+    length[0], length[n // 2] = maxlen, 0
+    rp = np.concatenate([[0], np.cumsum(length)]).astype(np.int64)
+    col = rng.integers(0, n, rp[-1]).astype(np.int32)
+    val = rng.standard_normal(rp[-1])
+    sv = Solver(n, rp, col, val, sketch_seed=1, precision="fp32", block_rows=block_rows)
+    v = _unit(n, 1)
+    # the second basis vector is A b_1 minus its projection on b_1, normalised
+    _, k, _, B, _ = sv.inner_cycle(v, m=2, s=16, k=1)
+    b1 = B[0].cpu().numpy()
+    A = np.zeros(n)
+    np.add.at(A, np.repeat(np.arange(n), length), val.astype(np.float32).astype(np.float64) * b1[col])
+    w = A - b1 * (b1 @ A)
+    w /= np.linalg.norm(w)
+    got = B[1].cpu().numpy()
+    # FP32: maxlen products and sums per row, the projection's and the scale's roundings, the dot's over n rows
+    assert k == 2 and np.linalg.norm(got - w) <= (maxlen + 8 + np.sqrt(n)) * 2.0 ** -24 * max(1.0, np.linalg.norm(A) / np.linalg.norm(A - b1 * (b1 @ A)))
+    sv.close()

@@ -247,12 +247,11 @@ static size_t step_smem(const Plan& p) {
 // ---------------------------------------------------------------------------------------------------------------
 // Phase 1 of an inner step for the CTA's row block: w' = A u_i (stored to W and kept in the shared block), the
 // block partials of the window dots (hpart), and Eb, the block's largest exponent of w' (the reference exponent of
-// the FP64 fixed-point sketch sums).  (The block partials of ||u_i||^2 come from the update that wrote u_i.)  Returns false (every thread of the CTA alike) when
+// the FP64 fixed-point sketch sums).  red: 512 slots of shared memory.  (The block partials of ||u_i||^2 come from the update that wrote u_i.)  Returns false (every thread of the CTA alike) when
 // the block's problem has no step i to take.
 template <int V, int U, int NW, typename MT, typename VT, typename AT>
 __device__ __forceinline__ bool inner_spmv_part(const Plan& P, int i, const MT* __restrict__ val,
-                                                AT* __restrict__ wblk, int& Eb) {
-    __shared__ AT red[512];
+                                                AT* __restrict__ wblk, int& Eb, AT* __restrict__ red) {
     __shared__ int stop_sh, emax_sh[16];
     const int b = blockIdx.x;
     const BlockInfo bi = block_info(P, b);
@@ -334,28 +333,22 @@ __device__ __forceinline__ void sketch_prepare(const Plan& P, int len, AT* __res
     __syncthreads();
 }
 
-// Per-block sketch partials of w' for sketch rows r0, r0 + rstep, ... < s: cpart[b*s + r] = sum over the block's list
-// for row r (in list order) of +-w'.  FP64: from the fixed-point image, converted to FP64 once per row.
+// Per-block sketch partials of w' for every sketch row, by warps [0, nwk) of the caller's numbering (w: this warp):
+// cpart[b*s + r] = sum over the block's list for row r of +-w'.  FP64: from the fixed-point image, converted to FP64 once
+// per row.  buf: 512 slots of shared memory.
 template <typename AT>
-__device__ __forceinline__ void sketch_rows(const Plan& P, int b, int list, const AT* __restrict__ wblk, int Eb, int r0,
-                                            int rstep) {
+__device__ __forceinline__ void sketch_rows(const Plan& P, int b, int list, const AT* __restrict__ wblk, int Eb, int w,
+                                            int nwk, AT* __restrict__ buf) {
     const int s = P.s, ng = (s + 31) / 32;
     const int* sg = P.seg + (int64_t)list * ng;  // the block's group starts (units)
-    AT* cpart = (AT*)P.cpart;
+    AT* cp = (AT*)P.cpart + (int64_t)b * s;
     if constexpr (sizeof(AT) == 8) {
-        const long long* qblk = reinterpret_cast<const long long*>(wblk);
         const double unit = fixed_unit(0.0, Eb, P.sk_headroom);
         const bool bad = exp_nonfinite(0.0, Eb);
-        for (int rr = r0; rr < s; rr += rstep) {
-            const int g = rr >> 5;
-            const long long v = sum_group(P.ent, sg[g], (sg[g + 1] - sg[g]) >> 5, rr & 31, qblk);
-            cpart[(int64_t)b * s + rr] = bad ? (AT)NAN : (AT)((double)v * unit);
-        }
+        sketch_sums(P.ent, sg, s, w, nwk, reinterpret_cast<const long long*>(wblk), reinterpret_cast<long long*>(buf),
+                    [&](int r, long long v) { cp[r] = bad ? (AT)NAN : (AT)((double)v * unit); });
     } else {
-        for (int rr = r0; rr < s; rr += rstep) {
-            const int g = rr >> 5;
-            cpart[(int64_t)b * s + rr] = sum_group(P.ent, sg[g], (sg[g + 1] - sg[g]) >> 5, rr & 31, wblk);
-        }
+        sketch_sums(P.ent, sg, s, w, nwk, wblk, buf, [&](int r, AT v) { cp[r] = v; });
     }
 }
 
@@ -367,11 +360,12 @@ template <int V, int U, int NW, typename MT, typename VT, typename AT>
 __global__ void __maxnreg__(56) k_inner_spmv(const Plan P, int i, const MT* __restrict__ val) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AT* wblk = reinterpret_cast<AT*>(smem_raw);
+    __shared__ AT red[512];
     int Eb = 1;
-    if (!inner_spmv_part<V, U, NW, MT, VT, AT>(P, i, val, wblk, Eb)) return;
+    if (!inner_spmv_part<V, U, NW, MT, VT, AT>(P, i, val, wblk, Eb, red)) return;
     const int b = blockIdx.x;
     sketch_prepare(P, P.blk_len[b], wblk, Eb);
-    sketch_rows(P, b, P.blk_list[b], wblk, Eb, threadIdx.x, blockDim.x);
+    sketch_rows(P, b, P.blk_list[b], wblk, Eb, threadIdx.x >> 5, blockDim.x >> 5, red);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -576,11 +570,6 @@ __global__ void __launch_bounds__(512, (NW <= 3) ? 3 : 2) k_inner_axpy(const Pla
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// Named barrier among the first `threads` threads of the CTA (barrier 0 is __syncthreads).
-__device__ __forceinline__ void bar_sync_named(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // Bounded wait of one lane for a shared-memory flag set by another warp of the CTA; false if it gave up.
 constexpr int kFlagPolls = 1 << 26;  // several seconds: well beyond the grid wait's own bound (the flag is set once that wait ends)
 __device__ __forceinline__ bool wait_flag(const int* flag) {
@@ -605,7 +594,7 @@ __device__ __forceinline__ bool wait_flag(const int* flag) {
 // The arithmetic of every value and its order are those of the two-launch step.
 template <int NW, typename VT, typename AT>
 __device__ __forceinline__ void fused_phase2(const Plan& P, int i, int last, AT* __restrict__ wblk, int Eb,
-                                             const unsigned long long* target_ptr) {
+                                             const unsigned long long* target_ptr, AT* __restrict__ red) {
     constexpr int NSW = NW + 1;  // warps of the scalar role
     constexpr bool WIDE = (sizeof(AT) == 8 && NW >= 3);
     __shared__ AT coef_sh[kMaxTrunc];
@@ -682,7 +671,7 @@ __device__ __forceinline__ void fused_phase2(const Plan& P, int i, int last, AT*
             *(volatile int*)&ready_sh = 1;
         }
     } else {
-        sketch_rows(P, b, bi.list, wblk, Eb, threadIdx.x - NSW * 32, (int)blockDim.x - NSW * 32);
+        sketch_rows(P, b, bi.list, wblk, Eb, warp - NSW, nw - NSW, red);
         __threadfence();  // this warp's partials are visible device-wide before the CTA's arrival on counter 2
         __syncwarp();
         if (lane == 0 && atomicAdd(&skdone_sh, 1) == nw - NSW - 1) {
@@ -820,8 +809,9 @@ __global__ void __maxnreg__(56) k_inner_step(const Plan P, int i, const MT* __re
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AT* wblk = reinterpret_cast<AT*>(smem_raw);
     __shared__ unsigned long long target_sh;
+    __shared__ AT red[512];
     int Eb = 1;
-    const bool active = inner_spmv_part<V, U, NW, MT, VT, AT>(P, i, val, wblk, Eb);
+    const bool active = inner_spmv_part<V, U, NW, MT, VT, AT>(P, i, val, wblk, Eb, red);
     __threadfence();  // this thread's partials are visible device-wide before the CTA arrives
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -830,7 +820,7 @@ __global__ void __maxnreg__(56) k_inner_step(const Plan P, int i, const MT* __re
         if (!active) atomicAdd(P.gsync + 2, 1ull);  // no sketch partials from this CTA either
     }
     if (!active) return;
-    fused_phase2<NW, VT, AT>(P, i, last, wblk, Eb, &target_sh);
+    fused_phase2<NW, VT, AT>(P, i, last, wblk, Eb, &target_sh, red);
 }
 
 template <int V, int U, int NW, typename MT, typename VT, typename AT>

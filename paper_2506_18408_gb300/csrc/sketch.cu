@@ -244,8 +244,8 @@ void launch_fill_u16(int64_t cnt, uint16_t v, uint16_t* out, cudaStream_t st) {
 }
 
 // Per-block partial sketch of xs = scale_p * x; optionally stores (VT)xs into dst.  The value fed to the sketch is
-// the stored (rounded) one, so S is applied to exactly the vector kept in the basis.  One thread per sketch row
-// walks its gather list; FP64 data are summed exactly in 64-bit fixed point, FP32 data in list order.
+// the stored (rounded) one, so S is applied to exactly the vector kept in the basis.  The sums are sketch_sums';
+// FP64 data are summed exactly in 64-bit fixed point, FP32 data in list order.
 template <typename VT, typename AT>
 __global__ void __launch_bounds__(512) k_sketch_partials(const Plan P, const double* __restrict__ x,
                                                          const double* __restrict__ xscale, int xstride,
@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(512) k_sketch_partials(const Plan P, const dou
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AT* xb = reinterpret_cast<AT*>(smem_raw);
     __shared__ int emax_sh[32];
+    __shared__ AT buf[512];
     const int b = blockIdx.x;
     const BlockInfo bi = block_info(P, b);
     if (P.pflag[bi.prob] & 1) return;
@@ -284,17 +285,13 @@ __global__ void __launch_bounds__(512) k_sketch_partials(const Plan P, const dou
         __syncthreads();
         const double unit = fixed_unit(0.0, Eb, P.sk_headroom);
         const bool bad = exp_nonfinite(0.0, Eb);
-        for (int rr = threadIdx.x; rr < s; rr += blockDim.x) {
-            const int g = rr >> 5;
-            const long long v = sum_group(P.ent, sg[g], (sg[g + 1] - sg[g]) >> 5, rr & 31, qb);
-            part[(int64_t)b * s + rr] = bad ? (AT)NAN : (AT)((double)v * unit);
-        }
+        double* pb = (double*)part + (int64_t)b * s;
+        sketch_sums(P.ent, sg, s, threadIdx.x >> 5, blockDim.x >> 5, (const long long*)qb, (long long*)buf,
+                    [&](int r, long long v) { pb[r] = bad ? (double)NAN : (double)v * unit; });
     } else {
         __syncthreads();
-        for (int rr = threadIdx.x; rr < s; rr += blockDim.x) {
-            const int g = rr >> 5;
-            part[(int64_t)b * s + rr] = sum_group(P.ent, sg[g], (sg[g + 1] - sg[g]) >> 5, rr & 31, xb);
-        }
+        AT* pb = part + (int64_t)b * s;
+        sketch_sums(P.ent, sg, s, threadIdx.x >> 5, blockDim.x >> 5, (const AT*)xb, buf, [&](int r, AT v) { pb[r] = v; });
     }
 }
 

@@ -16,8 +16,6 @@ namespace sfg {
 // Template value of k_inner_spmv's lanes-per-row parameter for one thread per row reading the SELL-32 copy of A
 // (the FP64 inner cycle); 1 is one thread per row reading the CSR arrays.
 constexpr int kVecSell = -1;
-// The same for one thread per row with the CSR entries staged in shared memory (spmv_rows_staged).
-constexpr int kVecStaged = -2;
 
 __device__ __forceinline__ bool cycle_idle(const Plan& P, int p, int i) {
     const CycleState* c = P.cyc + p;

@@ -17,33 +17,66 @@ namespace sfg {
 
 __device__ __forceinline__ bool outer_idle(const Plan& P, int p) { return (P.pflag[p] & 1) != 0; }
 
+// A x over rows [k0, k0 + len) of a block, emit(k, (A x)_k) once per row k; smem: the shape's scratch (the block's rows, or the
+// stage area).  The length-binned shape takes whole blocks only.  The shapes that go through shared memory end the SpMV with
+// a block barrier.
+template <int V, int U, typename Emit>
+__device__ __forceinline__ void block_spmv(const Plan& P, const BlockInfo& bi, int k0, int len,
+                                           const double* __restrict__ x, unsigned char* smem, Emit&& emit) {
+    const int m0 = bi.v0 - bi.cs + k0;
+    if constexpr (V == kVecStaged) {
+        spmv_rows_staged<double, double, double>(P.rp + m0, P.col, P.val, x + bi.cs, len, smem, P.maxlen, [](int) {},
+                                                 [&](int k, double v) {
+                                                     if (k < len) emit(k0 + k, v);
+                                                 });
+    } else {
+        double* yb = reinterpret_cast<double*>(smem);
+        const bool copy = V == 0 && P.brp;
+        int n0, n01;
+        block_bins(P, bi, n0, n01);
+        spmv_rows_to_smem<V, U, double, double, double>(P.rp, copy ? P.bcol : P.col, copy ? P.bval : P.val, x + bi.cs,
+                                                        m0, m0 + len, yb, P.perm, n0, n01, V == 0 ? P.brp : nullptr);
+        __syncthreads();
+        for (int k = threadIdx.x; k < len; k += blockDim.x) emit(k0 + k, yb[k]);
+    }
+}
+
+// The shape of an FP64 SpMV kernel of the outer iteration that needs `fixed` bytes of shared memory besides: staged entries
+// for matrices of one thread per row where two 512-thread CTAs fit on an SM, and its dynamic shared memory.  128^3: w = A z with
+// its dots 94 -> 73 us, the residual 78 -> 55 us, y = A x 55 -> 46 us per launch.
+static int outer_vec(const Plan& p, size_t fixed, size_t* smem) {
+    const size_t stage = 16 * (size_t)stage_bytes<double>(p.maxlen);
+    if (p.vec == 1 && 2 * (fixed + stage + 4096) <= 226 * 1024) {
+        *smem = fixed + stage;
+        return kVecStaged;
+    }
+    *smem = std::max<size_t>(fixed, (size_t)p.Bn * sizeof(double));
+    return p.vec;
+}
+
 // rb = b - A x (x may be null: rb = b); npart[b] = ||rb||^2 over the block, npart2[b] = ||b||^2 over the block.
 template <int V, int U>
 __global__ void __launch_bounds__(512, 2)
     k_residual(const Plan P, const double* __restrict__ bv, const double* __restrict__ x, double* __restrict__ rb,
                int only_final) {
-    extern __shared__ double axb[];
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[32];
     const int b = blockIdx.x;
     const BlockInfo bi = block_info(P, b);
     const int fl = P.pflag[bi.prob];
     if (only_final ? !(fl & 2) : (fl & 1)) return;
-    if (x) {
-        const int m0 = bi.v0 - bi.cs;
-        int n0, n01;
-        block_bins(P, bi, n0, n01);
-        spmv_rows_to_smem<V, U, double, double, double>(P.rp, (V == 0 && P.brp) ? P.bcol : P.col, (V == 0 && P.brp) ? P.bval : P.val, x + bi.cs, m0, m0 + bi.len, axb, P.perm,
-                                                        n0, n01, V == 0 ? P.brp : nullptr);
-        __syncthreads();
-    }
     double a1 = 0.0, a2 = 0.0;
-    for (int k = threadIdx.x; k < bi.len; k += blockDim.x) {
-        const int r = bi.v0 + k;
-        const double bb = bv[r];
-        const double rr = x ? bb - axb[k] : bb;
-        if (rb) rb[r] = rr;
+    auto row = [&](int k, double ax) {
+        const double bb = bv[bi.v0 + k];
+        const double rr = bb - ax;
+        if (rb) rb[bi.v0 + k] = rr;
         a1 += rr * rr;
         a2 += bb * bb;
+    };
+    if (x) {
+        block_spmv<V, U>(P, bi, 0, bi.len, x, smem, row);
+    } else {
+        for (int k = threadIdx.x; k < bi.len; k += blockDim.x) row(k, 0.0);
     }
     a1 = block_sum(a1, red);
     a2 = block_sum(a2, red);
@@ -54,9 +87,10 @@ __global__ void __launch_bounds__(512, 2)
 }
 
 void launch_residual(const Plan& p, const double* b, const double* x, double* rb, bool only_final) {
-    const size_t sm = x ? (size_t)p.Bn * sizeof(double) : 0;
-    SFG_SPMV_DISPATCH(p.vec, (set_smem((const void*)k_residual<VV, UU>, sm),
-                              k_residual<VV, UU><<<p.nblk, 512, sm, p.st>>>(p, b, x, rb, only_final ? 1 : 0)));
+    size_t sm = 0;
+    const int vec = x ? outer_vec(p, 0, &sm) : 1;
+    SFG_SPMV_DISPATCH(vec, (set_smem((const void*)k_residual<VV, UU>, sm),
+                            k_residual<VV, UU><<<p.nblk, 512, sm, p.st>>>(p, b, x, rb, only_final ? 1 : 0)));
     ++g_launches;
 }
 
@@ -110,47 +144,66 @@ void launch_true_residual_reduce(const Plan& p) {
     ++g_launches;
 }
 
-// Dots of the block's part of v_0..v_j with the block vector wb (smem): opart[b*ldo + l], one warp per column.
+// Dots of the block's part of v_0..v_j with the block vector wb (smem): opart[b*ldo + l].  With few columns every column's
+// rows are cut into `nseg` segments so that all warps work (a warp per column left 15 of 16 idle at j = 0); the segments'
+// sums are added in order.
 __device__ __forceinline__ void block_dots(const Plan& P, const BlockInfo& bi, int b, int j,
                                            const double* __restrict__ wb) {
+    __shared__ double seg_sh[16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int ldo = P.jmax + 1;
-    for (int l = warp; l <= j; l += nw) {
+    const int ldo = P.jmax + 1, cols = j + 1, nseg = max(1, nw / cols);
+    for (int t = warp; t < cols * nseg; t += nw) {
+        const int l = t / nseg, g = t % nseg;
         const double* vl = P.Vb + (int64_t)l * P.N + bi.v0;
-        double acc = 0.0;
-        for (int k = lane; k < bi.len; k += 32) acc += vl[k] * wb[k];
-        acc = warp_sum(acc);
-        if (lane == 0) P.opart[(int64_t)b * ldo + l] = acc;
+        const int k1 = (int)((int64_t)bi.len * (g + 1) / nseg);
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        int k = (int)((int64_t)bi.len * g / nseg) + lane;
+        for (; k + 96 < k1; k += 128) {
+            double v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = vl[k + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[u] = fma(v[u], wb[k + 32 * u], acc[u]);
+        }
+        for (; k < k1; k += 32) acc[0] = fma(vl[k], wb[k], acc[0]);
+        const double a = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+        if (lane == 0) {
+            if (nseg == 1) P.opart[(int64_t)b * ldo + l] = a;
+            else seg_sh[t] = a;
+        }
+    }
+    if (nseg == 1) return;
+    __syncthreads();
+    if ((int)threadIdx.x < cols) {
+        double a = 0.0;
+        for (int g = 0; g < nseg; ++g) a += seg_sh[threadIdx.x * nseg + g];
+        P.opart[(int64_t)b * ldo + threadIdx.x] = a;
     }
 }
 
-// w = A z_j into smem and Wo; opart[b*ldo + l] = Vb_l(block) . w(block) for l <= j.
+// w = A z_j into smem and Wo; opart[b*ldo + l] = Vb_l(block) . w(block) for l <= j; and the true residual of inner cycle
+// j, r_hat_j = v_j - A z_j (v_j = nu_j Vb_j), for the bound of Eq. 5: its block partial of ||r_hat_j||^2 goes to npart2
+// (free during outer steps).
 template <int V, int U>
 __global__ void __launch_bounds__(512, 2) k_outer_spmv(const Plan P, int j) {
-    extern __shared__ double wb[];
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ double red[32];
     const int b = blockIdx.x;
     const BlockInfo bi = block_info(P, b);
     if (outer_idle(P, bi.prob)) return;
-    const double* z = P.Z + (int64_t)j * P.N;
-    const int m0 = bi.v0 - bi.cs;
-    int n0, n01;
-    block_bins(P, bi, n0, n01);
-    spmv_rows_to_smem<V, U, double, double, double>(P.rp, (V == 0 && P.brp) ? P.bcol : P.col, (V == 0 && P.brp) ? P.bval : P.val, z + bi.cs, m0, m0 + bi.len, wb, P.perm, n0,
-                                                    n01, V == 0 ? P.brp : nullptr);
-    __syncthreads();
-    // the true residual of inner cycle j, r_hat_j = v_j - A z_j (v_j = nu_j Vb_j), for the bound of Eq. 5: its
-    // block partial of ||r_hat_j||^2 goes to npart2 (free during outer steps)
+    double* wb = reinterpret_cast<double*>(smem);  // [Bn], then the stage area
     const double nuj = P.nu[(int64_t)bi.prob * (P.jmax + 1) + j];
-    const double* vj = P.Vb + (int64_t)j * P.N;
+    const double* vj = P.Vb + (int64_t)j * P.N + bi.v0;
     double r2 = 0.0;
-    for (int k = threadIdx.x; k < bi.len; k += blockDim.x) {
-        const double w = wb[k];
-        P.Wo[bi.v0 + k] = w;
-        const double rr = nuj * vj[bi.v0 + k] - w;
-        r2 += rr * rr;
-    }
+    block_spmv<V, U>(P, bi, 0, bi.len, P.Z + (int64_t)j * P.N, V == kVecStaged ? smem + (size_t)P.Bn * sizeof(double) : smem,
+                     [&](int k, double w) {
+                         wb[k] = w;
+                         P.Wo[bi.v0 + k] = w;
+                         const double rr = nuj * vj[k] - w;
+                         r2 += rr * rr;
+                     });
+    __syncthreads();
     block_dots(P, bi, b, j, wb);
-    __shared__ double red[32];
     r2 = block_sum(r2, red);
     if (threadIdx.x == 0) P.npart2[b] = r2;
 }
@@ -286,9 +339,10 @@ __global__ void k_outer_givens(const Plan P, int j) {
 }
 
 void launch_outer_step(const Plan& p, int j) {
-    const size_t sm = (size_t)p.Bn * sizeof(double);
-    SFG_SPMV_DISPATCH(p.vec, (set_smem((const void*)k_outer_spmv<VV, UU>, sm),
-                              k_outer_spmv<VV, UU><<<p.nblk, 512, sm, p.st>>>(p, j)));
+    size_t sm;
+    const int vec = outer_vec(p, (size_t)p.Bn * sizeof(double), &sm);
+    SFG_SPMV_DISPATCH(vec, (set_smem((const void*)k_outer_spmv<VV, UU>, sm),
+                            k_outer_spmv<VV, UU><<<p.nblk, 512, sm, p.st>>>(p, j)));
     const int ncols = j + 1, wpb = 8;
     const int rgrid = (int)(((int64_t)p.P * ncols + wpb - 1) / wpb);
     k_reduce_cols<<<rgrid, 32 * wpb, 0, p.st>>>(p, ncols, p.h1);
@@ -325,19 +379,26 @@ __global__ void k_final_y(const Plan P) {
     }
 }
 
-// x = x0 + Z y over the blocks of flagged problems.
-__global__ void __launch_bounds__(256) k_final_x(const Plan P, const double* __restrict__ x0,
-                                                 double* __restrict__ x) {
+// x = x0 + Z y over the blocks of flagged problems, each block in pieces of kFinalRows rows (one CTA each, grid y; two rows and
+// four columns in flight per thread).  Bound by HBM; 128^3, 7 columns: 59 -> 32 us against a CTA per row block.
+constexpr int kFinalThreads = 256, kFinalRows = 512;
+__global__ void __launch_bounds__(kFinalThreads) k_final_x(const Plan P, const double* __restrict__ x0,
+                                                           double* __restrict__ x) {
     __shared__ double yy[kMaxM];
     const BlockInfo bi = block_info(P, blockIdx.x);
-    const int p = bi.prob;
-    if (!(P.pflag[p] & 2)) return;
-    const int J = P.ost[p].j, N = P.N;
-    for (int l = threadIdx.x; l < J; l += blockDim.x) yy[l] = P.yo[(int64_t)p * P.jmax + l];
+    const int p = bi.prob, k0 = blockIdx.y * kFinalRows;
+    if (!(P.pflag[p] & 2) || k0 >= bi.len) return;
+    const int J = P.ost[p].j;
+    const int64_t N = P.N;
+    for (int l = threadIdx.x; l < J; l += kFinalThreads) yy[l] = P.yo[(int64_t)p * P.jmax + l];
     __syncthreads();
-    for (int k = threadIdx.x; k < bi.len; k += blockDim.x) {
+#pragma unroll
+    for (int u = 0; u < kFinalRows / kFinalThreads; ++u) {
+        const int k = k0 + u * kFinalThreads + threadIdx.x;
+        if (k >= bi.len) break;
         const int64_t r = bi.v0 + k;
         double acc = x0 ? x0[r] : 0.0;
+#pragma unroll 4
         for (int l = 0; l < J; ++l) acc += yy[l] * P.Z[(int64_t)l * N + r];
         x[r] = acc;
     }
@@ -345,28 +406,29 @@ __global__ void __launch_bounds__(256) k_final_x(const Plan P, const double* __r
 
 void launch_final_x(const Plan& p, int J, const double* x0, double* x) {
     k_final_y<<<p.P, 32, (size_t)std::max(J, 1) * sizeof(double), p.st>>>(p);
-    k_final_x<<<p.nblk, 256, 0, p.st>>>(p, x0, x);
+    k_final_x<<<dim3(p.nblk, (p.Bn + kFinalRows - 1) / kFinalRows), kFinalThreads, 0, p.st>>>(p, x0, x);
     g_launches += 2;
 }
 
+// y = A x; staged entries: each block in pieces of kPlainRows rows (one CTA each, grid y), so that an SM holds four CTAs.
+constexpr int kPlainRows = 2048;
 template <int V, int U>
 __global__ void __launch_bounds__(512, 2)
     k_spmv_plain(const Plan P, const double* __restrict__ x, double* __restrict__ y) {
-    extern __shared__ double yb[];
+    extern __shared__ __align__(16) unsigned char smem[];
     const BlockInfo bi = block_info(P, blockIdx.x);
-    const int m0 = bi.v0 - bi.cs;
-    int n0, n01;
-    block_bins(P, bi, n0, n01);
-    spmv_rows_to_smem<V, U, double, double, double>(P.rp, (V == 0 && P.brp) ? P.bcol : P.col, (V == 0 && P.brp) ? P.bval : P.val, x + bi.cs, m0, m0 + bi.len, yb, P.perm, n0,
-                                                    n01, V == 0 ? P.brp : nullptr);
-    __syncthreads();
-    for (int k = threadIdx.x; k < bi.len; k += blockDim.x) y[bi.v0 + k] = yb[k];
+    const int k0 = blockIdx.y * kPlainRows;
+    if (k0 >= bi.len) return;
+    const int len = (V == kVecStaged) ? min(kPlainRows, bi.len - k0) : bi.len;
+    block_spmv<V, U>(P, bi, k0, len, x, smem, [&](int k, double v) { y[bi.v0 + k] = v; });
 }
 
 void launch_spmv_f64(const Plan& p, const double* x, double* y) {
-    const size_t sm = (size_t)p.Bn * sizeof(double);
-    SFG_SPMV_DISPATCH(p.vec, (set_smem((const void*)k_spmv_plain<VV, UU>, sm),
-                              k_spmv_plain<VV, UU><<<p.nblk, 512, sm, p.st>>>(p, x, y)));
+    size_t sm;
+    const int vec = outer_vec(p, 0, &sm);
+    const int pieces = (vec == kVecStaged) ? (p.Bn + kPlainRows - 1) / kPlainRows : 1;
+    SFG_SPMV_DISPATCH(vec, (set_smem((const void*)k_spmv_plain<VV, UU>, sm),
+                            k_spmv_plain<VV, UU><<<dim3(p.nblk, pieces), 512, sm, p.st>>>(p, x, y)));
     ++g_launches;
 }
 

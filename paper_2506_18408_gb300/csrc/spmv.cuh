@@ -69,11 +69,13 @@ __device__ __forceinline__ void spmv_rows_scalar(const int* __restrict__ rp, con
 // into its own part of shared memory with asynchronous 16-byte copies (from the 16-byte boundary at or below; the
 // arrays are padded, so a copy may run past the last entry), one group of rows ahead: a group's columns and values are there
 // when its turn comes, every copy is coalesced whatever the row lengths, and what a row waits for is one round of gathers of x
-// (up to eight in flight per lane).  Read straight from global memory, lanes 7 entries apart touch 20 sectors per load, and a
+// (up to eight in flight per lane).  Used by the FP32 and BF16 inner cycles and by the FP64 kernels of the outer iteration.  Read straight from global memory, lanes 7 entries apart touch 20 sectors per load, and a
 // row of 7 entries waits for two rounds of loads and gathers.  A group's values go to registers before its last products,
 // which frees the buffer for the next group's copy.  Rows are summed in entry order, a warp issuing as many products as its
 // longest row.  128^3 solve to 1e-12 with FP32 inner cycles: 45.8 -> 42.3 ms.  FP64 inner cycles keep the SELL-32 copy (staged:
 // 46.4 -> 57.6 ms, the buffers of two CTAs beside their blocks of w' leave 28 KB of L1).
+constexpr int kVecStaged = -2;  // template value of the lanes-per-row parameter for this form
+
 template <typename MT>
 __host__ __device__ constexpr int stage_bytes(int maxlen) {  // one warp's buffer for rows of at most maxlen entries
     return 32 * maxlen * (4 + (int)sizeof(MT)) + 32;
@@ -341,9 +343,11 @@ __device__ __forceinline__ void spmv_rows_to_smem(const int* __restrict__ rp, co
     else spmv_rows_vector<V, U, MT, XT, AT>(rp, col, val, x, r0, r1, out);
 }
 
-// Dispatch on the lanes-per-row width chosen at run time (0 = length-binned, 1 = one thread per row, else 2..32).
+// Dispatch on the lanes-per-row width chosen at run time (-2 = one thread per row with staged entries, 0 = length-binned, 1 =
+// one thread per row, else 2..32).
 #define SFG_SPMV_DISPATCH(V_RUNTIME, CALL)                       \
     switch (V_RUNTIME) {                                         \
+        case -2: { constexpr int VV = -2, UU = 1; CALL; } break; \
         case 0: { constexpr int VV = 0, UU = 1; CALL; } break;   \
         case 1: { constexpr int VV = 1, UU = 1; CALL; } break;   \
         case 2: { constexpr int VV = 2, UU = 4; CALL; } break;   \

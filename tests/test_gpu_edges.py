@@ -126,3 +126,29 @@ def test_staged_spmv_with_ragged_rows(Solver, n, maxlen, block_rows):
     # FP32: maxlen products and sums per row, the projection's and the scale's roundings, the dot's over n rows
     assert k == 2 and np.linalg.norm(got - w) <= (maxlen + 8 + np.sqrt(n)) * 2.0 ** -24 * max(1.0, np.linalg.norm(A) / np.linalg.norm(A - b1 * (b1 @ A)))
     sv.close()
+
+
+# y = A x and full solves through the outer kernels' staged SpMV: pieces of 2048 rows, rows of 0 to 16 entries, blocks too
+# large for the stage area beside them
+@pytest.mark.parametrize("n,maxlen,block_rows", [(1, 1, 0), (33, 16, 32), (2049, 7, 8192), (9000, 16, 4128), (20_000, 9, 8192)])
+def test_staged_fp64_spmv(Solver, n, maxlen, block_rows):
+    rng = np.random.default_rng(n + maxlen)
+    length = rng.integers(0, maxlen, n)
+    rp = np.concatenate([[0], np.cumsum(length + 1)]).astype(np.int64)
+    col = rng.integers(0, n, rp[-1]).astype(np.int32)
+    val = rng.standard_normal(rp[-1])
+    col[rp[:-1]] = np.arange(n)
+    val[rp[:-1]] = 8.0 * maxlen
+    sv = Solver(n, rp, col, val, sketch_seed=1, block_rows=block_rows, zeta=min(8, n))
+    x = rng.standard_normal(n)
+    y, size = np.zeros(n), np.zeros(n)
+    rows = np.repeat(np.arange(n), length + 1)
+    np.add.at(y, rows, val * x[col])
+    np.add.at(size, rows, np.abs(val * x[col]))
+    assert np.all(np.abs(sv.spmv(dev_vec(x)).cpu().numpy() - y) <= 2 * (maxlen + 1) * 2.0 ** -53 * size)
+    if n > 64:
+        got, info = sv.solve(dev_vec(y), m=20, s=80, k=2, tol=1e-10)
+        r = y.copy()
+        np.subtract.at(r, rows, val * got.cpu().numpy()[col])
+        assert info["status"] == 0 and abs(info["rel_res_true"] - np.linalg.norm(r) / np.linalg.norm(y)) <= 1e-14
+    sv.close()

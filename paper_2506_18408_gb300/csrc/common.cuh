@@ -161,6 +161,32 @@ __device__ __forceinline__ void sketch_column(uint64_t seed, int64_t j, int zeta
     }
 }
 
+// sketch_column for a compile-time zeta: rows and signs stay in registers.
+template <int ZETA>
+__device__ __forceinline__ void sketch_column_n(uint64_t seed, int64_t j, int s, int (&rows)[ZETA], int (&neg)[ZETA]) {
+#pragma unroll
+    for (int l = 0; l < ZETA; ++l) {
+        const uint64_t base = (uint64_t)(j * ZETA + l) * 128ull;
+        int cand = 0;
+        bool dup = true;
+        for (int a = 0; a < 64 && dup; ++a) {
+            const uint64_t h = sm64_draw(seed, base + 2ull * (uint64_t)a);
+            cand = (int)(((h >> 32) * (uint64_t)s) >> 32);
+            dup = false;
+#pragma unroll
+            for (int q = 0; q < l; ++q) dup |= (rows[q] == cand);
+        }
+        while (dup) {
+            cand = (cand + 1 == s) ? 0 : cand + 1;
+            dup = false;
+#pragma unroll
+            for (int q = 0; q < l; ++q) dup |= (rows[q] == cand);
+        }
+        rows[l] = cand;
+        neg[l] = (int)(sm64_draw(seed, base + 1ull) >> 63);
+    }
+}
+
 // ------------------------------------------------------------------------------------------------------------
 // 64-bit fixed-point image of w relative to the block exponent Eb (max biased exponent in the block, >= 1):
 // w ~= q * 2^(Eb + H - 1075), |q| <= 2^53, rounded to nearest (ties away from zero).  Integer operations only.

@@ -8,13 +8,20 @@
 // every GPU that loads the library holds until the process exits.  The caller passes only its input and output.
 //
 // The embedding is the same one a handle created with the same seed applies (same SplitMix64 draw rule, see
-// sketch_column), so results agree with sfgmres_sketch_apply up to summation rounding.  Each CTA owns a block of
-// columns, draws their rows on the fly, and sums its terms exactly in 64-bit fixed point relative to the block's
+// sketch_column), so results agree with sfgmres_sketch_apply up to summation rounding.  A CTA takes chunks of at most 992
+// columns, draws their rows on the fly, and sums a chunk's terms exactly in 64-bit fixed point relative to the chunk's
 // largest exponent with shared-memory integer atomics (integer addition is order independent, so the result is
-// deterministic); the block partials are then summed in block order.
+// deterministic); at most 992 terms of at most 2^53 meet in a sum, so none can overflow and no count of the terms is
+// needed.  The chunk sums are added in chunk order into the CTA's partial, the partials in a fixed order.
+//
+// What bounds it: the draws (two 64-bit mixes per nonzero) and the shared-memory atomics, both in every SM at once; the
+// chunks of at most two CTAs per SM keep the second kernel's sums short, and that kernel reads 32 sketch rows of a partial per
+// warp with 16 warps over the partials.  n = 1,000,003, s = 240, zeta = 8: 43 + 5 us; with every row drawn twice (once to count the
+// terms) into local memory, 977 partials and a thread per row of the second kernel, 102 + 72 us.
 #include "../../include/sfgmres.h"
 #include "common.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -23,78 +30,101 @@ namespace sfg {
 
 // Largest number of (block, sketch row) partials the static scratch holds: 2^20 doubles = 8 MiB.
 constexpr int64_t kNoallocScratch = int64_t(1) << 20;
-constexpr int kNoallocMinCols = 1024;     // columns per block, at least
-constexpr int kNoallocMaxCols = 65536;    // columns per block, at most (keeps the fixed-point headroom small)
+constexpr int64_t kNoallocMaxCols = 65536;  // with 2^20 / s partials, the largest n (a documented limit)
+constexpr int kChunkCols = 992;           // columns per chunk, at most: fewer than 1023 terms per sum
+constexpr int kChunkMin = 128;            // and at least (short vectors: more CTAs)
+constexpr int kNoallocCtas = 304;         // CTAs of the partials kernel, at most (two per SM)
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocScratch];
 
 void set_global_error(const std::string& msg);  // api.cu: the message sfgmres_last_error(NULL) returns
 
-__global__ void __launch_bounds__(512)
-    k_noalloc_partials(int64_t n, int Bn, int s, int zeta, uint64_t seed, const double* __restrict__ v,
+// ZETA: nonzeros per column as a compile-time count (rows and signs in registers), 0: any count.
+template <int ZETA>
+__global__ void __launch_bounds__(512, 2)
+    k_noalloc_partials(int64_t n, int chunk, int s, int zeta_any, uint64_t seed, const double* __restrict__ v,
                        double* __restrict__ part) {
     extern __shared__ unsigned char smem_raw[];
-    long long* acc = reinterpret_cast<long long*>(smem_raw);  // [s]
-    int* cnt = reinterpret_cast<int*>(acc + s);               // [s]
-    __shared__ int wmax[32], wcnt[32];
+    long long* acc = reinterpret_cast<long long*>(smem_raw);  // [s] the chunk's sums
+    double* tot = reinterpret_cast<double*>(acc + s);         // [s] the CTA's partial
+    __shared__ int wmax[2][16];
+    const int zeta = ZETA > 0 ? ZETA : zeta_any;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t c0 = (int64_t)blockIdx.x * Bn;
-    const int64_t c1 = min(n, c0 + Bn);
     for (int r = threadIdx.x; r < s; r += blockDim.x) {
         acc[r] = 0;
-        cnt[r] = 0;
+        tot[r] = 0.0;
     }
-    __syncthreads();
-    // pass 1: terms per sketch row (for the overflow headroom) and the block's largest exponent
-    int emax = 1;
-    int rows[kMaxZeta], neg[kMaxZeta];
-    for (int64_t j = c0 + threadIdx.x; j < c1; j += blockDim.x) {
-        sketch_column(seed, j, zeta, s, rows, neg);
-        for (int l = 0; l < zeta; ++l) atomicAdd(cnt + rows[l], 1);
-        emax = max(emax, exp_of(v[j]));
+    int par = 0;  // wmax alternates, so that a warp may write the next chunk's while another reads this one's
+    for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < n; c0 += (int64_t)gridDim.x * chunk, par ^= 1) {
+        const int len = (int)min((int64_t)chunk, n - c0);
+        double x[2];  // chunk <= 2 x 512 columns: this thread's
+        int emax = 1;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = u * (int)blockDim.x + (int)threadIdx.x;
+            x[u] = (j < len) ? v[c0 + j] : 0.0;
+            emax = max(emax, exp_of(x[u]));
+        }
+        emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
+        if (lane == 0) wmax[par][warp] = emax;
+        __syncthreads();  // also: acc and tot are set
+        int Eb = 1;
+        for (int q = 0; q < nw; ++q) Eb = max(Eb, wmax[par][q]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = u * (int)blockDim.x + (int)threadIdx.x;
+            if (j >= len) break;
+            const long long q = to_fixed(x[u], Eb, 0);
+            int rows[ZETA > 0 ? ZETA : kMaxZeta], neg[ZETA > 0 ? ZETA : kMaxZeta];
+            if constexpr (ZETA > 0) sketch_column_n<ZETA>(seed, c0 + j, s, rows, neg);
+            else sketch_column(seed, c0 + j, zeta, s, rows, neg);
+#pragma unroll
+            for (int l = 0; l < zeta; ++l)
+                atomicAdd(reinterpret_cast<unsigned long long*>(acc + rows[l]), (unsigned long long)(neg[l] ? -q : q));
+        }
+        __syncthreads();
+        const double unit = ldexp(1.0, Eb - 1075);
+        for (int r = threadIdx.x; r < s; r += blockDim.x) {
+            tot[r] += (Eb >= 2047) ? (double)NAN : (double)acc[r] * unit;
+            acc[r] = 0;  // the next chunk's atomics come after its first barrier
+        }
     }
-    __syncthreads();
-    int cmax = 0;
-    for (int r = threadIdx.x; r < s; r += blockDim.x) cmax = max(cmax, cnt[r]);
-    emax = (int)__reduce_max_sync(0xffffffffu, (unsigned)emax);
-    cmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)cmax);
-    if (lane == 0) {
-        wmax[warp] = emax;
-        wcnt[warp] = cmax;
-    }
-    __syncthreads();
-    int Eb = 1, L = 0;
-    for (int q = 0; q < nw; ++q) {
-        Eb = max(Eb, wmax[q]);
-        L = max(L, wcnt[q]);
-    }
-    int H = 0;
-    while ((L >> H) >= 1023) ++H;  // |term| <= 2^53, so at most 1023 * 2^H terms keep every sum below 2^63
-    // pass 2: exact fixed-point sums
-    for (int64_t j = c0 + threadIdx.x; j < c1; j += blockDim.x) {
-        const long long q = to_fixed(v[j], Eb, H);
-        sketch_column(seed, j, zeta, s, rows, neg);
-        for (int l = 0; l < zeta; ++l)
-            atomicAdd(reinterpret_cast<unsigned long long*>(acc + rows[l]),
-                      (unsigned long long)(neg[l] ? -q : q));
-    }
-    __syncthreads();
-    const double unit = ldexp(1.0, Eb + H - 1075);
-    for (int r = threadIdx.x; r < s; r += blockDim.x)
-        part[(int64_t)blockIdx.x * s + r] = (Eb >= 2047) ? (double)NAN : (double)acc[r] * unit;
+    for (int r = threadIdx.x; r < s; r += blockDim.x) part[(int64_t)blockIdx.x * s + r] = tot[r];
 }
 
-__global__ void k_noalloc_reduce(int nblk, int s, double scale, const double* __restrict__ part,
-                                 double* __restrict__ c) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= s) return;
+// c[r] = scale * the sum of part[b*s + r] over b: a CTA per 32 sketch rows (a lane each), warp w sums the partials w, w + 16,
+// ... and the warps' sums are added in order.
+__global__ void __launch_bounds__(512) k_noalloc_reduce(int nblk, int s, double scale, const double* __restrict__ part,
+                                                        double* __restrict__ c) {
+    __shared__ double sh[16][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = blockIdx.x * 32 + lane;
     double a = 0.0;
-    for (int b = 0; b < nblk; ++b) a += part[(int64_t)b * s + r];
-    c[r] = scale * a;
+    if (r < s) {
+#pragma unroll 8
+        for (int b = warp; b < nblk; b += 16) a += part[(int64_t)b * s + r];
+    }
+    sh[warp][lane] = a;
+    __syncthreads();
+    if (warp == 0 && r < s) {
+        for (int w = 1; w < 16; ++w) a += sh[w][lane];
+        c[r] = scale * a;
+    }
 }
 
-// Dynamic shared memory of k_noalloc_partials for s sketch rows: one 64-bit accumulator and one counter per row.
-static size_t partials_smem(int s) { return (size_t)s * (sizeof(long long) + sizeof(int)); }
+// Dynamic shared memory of k_noalloc_partials for s sketch rows: a 64-bit sum and an FP64 partial per row.
+static size_t partials_smem(int s) { return (size_t)s * (sizeof(long long) + sizeof(double)); }
+
+using PartialsKernel = void (*)(int64_t, int, int, int, uint64_t, const double*, double*);
+static PartialsKernel partials_kernel(int zeta) {
+    switch (zeta) {
+        case 1: return k_noalloc_partials<1>;
+        case 2: return k_noalloc_partials<2>;
+        case 4: return k_noalloc_partials<4>;
+        case 8: return k_noalloc_partials<8>;
+        default: return k_noalloc_partials<0>;
+    }
+}
 
 // Once per device, with that device current: look up the device address of the scratch array (cudaGetSymbolAddress;
 // in host code the array's name is only a host-side stand-in) and allow k_noalloc_partials the dynamic shared memory
@@ -109,9 +139,11 @@ static cudaError_t device_setup(double** out) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
     if (!cache[dev]) {
-        e = cudaFuncSetAttribute((const void*)k_noalloc_partials, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)partials_smem(kMaxS));
-        if (e != cudaSuccess) return e;
+        for (int z : {0, 1, 2, 4, 8}) {
+            e = cudaFuncSetAttribute((const void*)partials_kernel(z), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)partials_smem(kMaxS));
+            if (e != cudaSuccess) return e;
+        }
         void* p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return e;
@@ -167,20 +199,18 @@ extern "C" int sfgmres_sketch_apply_noalloc(int64_t n, int32_t s, int32_t zeta, 
                                      "cudaGetSymbolAddress): ") + cudaGetErrorString(e));
         return SFGMRES_ERR_CUDA;
     }
-    int64_t nblk = (n + kNoallocMinCols - 1) / kNoallocMinCols;
-    if (nblk > max_blocks) nblk = max_blocks;
-    int64_t Bn = (n + nblk - 1) / nblk;
-    Bn = ((Bn + 31) / 32) * 32;
-    nblk = (n + Bn - 1) / Bn;
+    int64_t chunk = (n + kNoallocCtas - 1) / kNoallocCtas;
+    chunk = std::min<int64_t>(kChunkCols, std::max<int64_t>(kChunkMin, (chunk + 31) / 32 * 32));
+    const int64_t nblk = std::min<int64_t>(std::min<int64_t>((n + chunk - 1) / chunk, kNoallocCtas), max_blocks);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    e = launch(k_noalloc_partials, (unsigned)nblk, 512, partials_smem(s), st, n, (int)Bn, (int)s, (int)zeta,
+    e = launch(partials_kernel(zeta), (unsigned)nblk, 512, partials_smem(s), st, n, (int)chunk, (int)s, (int)zeta,
                sketch_seed, v, part);
     if (e != cudaSuccess) {
         set_global_error(std::string("sfgmres_sketch_apply_noalloc: launch of the block partials kernel: ") +
                          cudaGetErrorString(e));
         return SFGMRES_ERR_CUDA;
     }
-    e = launch(k_noalloc_reduce, (unsigned)((s + 127) / 128), 128, 0, st, (int)nblk, (int)s,
+    e = launch(k_noalloc_reduce, (unsigned)((s + 31) / 32), 512, 0, st, (int)nblk, (int)s,
                1.0 / std::sqrt((double)zeta), (const double*)part, c);
     if (e != cudaSuccess) {
         set_global_error(std::string("sfgmres_sketch_apply_noalloc: launch of the reduction kernel: ") +

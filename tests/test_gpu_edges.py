@@ -128,6 +128,26 @@ def test_staged_spmv_with_ragged_rows(Solver, n, maxlen, block_rows):
     sv.close()
 
 
+# the allocation-free sketch: vectors around one chunk of columns and one wave of CTAs, counts of nonzeros with and without a
+# compile-time kernel, values of very different size
+@pytest.mark.parametrize("n,s,zeta", [(1, 1, 1), (127, 16, 2), (129, 40, 3), (992, 33, 4), (38_913, 100, 16), (301_568, 240, 8),
+                                      (301_569, 31, 5)])
+def test_allocation_free_sketch_at_chunk_edges(Solver, n, s, zeta):
+    from oracle import sketch as osk
+    from paper_2506_18408_gb300 import sfgmres_sketch_apply_noalloc
+
+    rng = np.random.default_rng(n)
+    v = rng.standard_normal(n) * 10.0 ** rng.integers(-3, 4, n)
+    c = dev_vec(np.full(s, np.nan))
+    d = dev_vec(v)
+    sfgmres_sketch_apply_noalloc(n, s, zeta, 7, d, c)  # the default stream, as c's copy below
+    S = osk.sketch_matrix(n, s, zeta, 7)
+    count = np.asarray(abs(S).sign().sum(axis=1)).ravel()
+    # both sides: a rounding per term and per addition (of the chunk's largest value, or of the running sum)
+    bound = 2.0 ** -53 * ((2 * count + n / 128 + 8) * (abs(S) @ np.abs(v)) + count * np.abs(v).max())
+    assert np.all(np.abs(c.cpu().numpy() - S @ v) <= bound)
+
+
 # y = A x and full solves through the outer kernels' staged SpMV: pieces of 2048 rows, rows of 0 to 16 entries, blocks too
 # large for the stage area beside them
 @pytest.mark.parametrize("n,maxlen,block_rows", [(1, 1, 0), (33, 16, 32), (2049, 7, 8192), (9000, 16, 4128), (20_000, 9, 8192)])

@@ -151,7 +151,7 @@ struct sfgmres_ctx : ListSet {
     IluHost ilu;
     std::vector<int> ilu_colour;  // colour of every row (original order)
     std::vector<int> ilu_src;     // host copy of ilu.src
-    DevBuf ilu_rp, ilu_col, ilu_diag, ilu_perm, ilu_src_d, ilu_lu, ilu_y, ilu_zp, ilu_t, ilu_zt, ilu_bad;
+    DevBuf ilu_rp, ilu_col, ilu_diag, ilu_perm, ilu_src_d, ilu_lu, ilu_y, ilu_ocol, ilu_piv, ilu_t, ilu_zt, ilu_bad;
     int ilu_built = 0;            // structure built
     int ilu_vals_ver = -1;        // values version the factors were computed for
     int vals_ver = 0;             // bumped by sfgmres_update_values
@@ -827,8 +827,9 @@ int ensure_ilu(sfgmres_ctx* h) {
         const size_t N = (size_t)n, Z = (size_t)std::max<int64_t>(nnz, 1);
         if ((rc = ensure(h, h->ilu_rp, (N + 1) * 4)) || (rc = ensure(h, h->ilu_col, Z * 4)) ||
             (rc = ensure(h, h->ilu_diag, N * 4)) || (rc = ensure(h, h->ilu_perm, N * 4)) ||
-            (rc = ensure(h, h->ilu_src_d, Z * 4)) || (rc = ensure(h, h->ilu_lu, Z * 8)) ||
-            (rc = ensure(h, h->ilu_y, N * 8)) || (rc = ensure(h, h->ilu_zp, N * 8)) ||
+            (rc = ensure(h, h->ilu_src_d, Z * 4)) || (rc = ensure(h, h->ilu_lu, (Z + kEntryPad) * 8)) ||
+            (rc = ensure(h, h->ilu_y, N * 8)) || (rc = ensure(h, h->ilu_ocol, (Z + kEntryPad) * 4)) ||
+            (rc = ensure(h, h->ilu_piv, N * sizeof(double2))) ||
             (rc = ensure(h, h->ilu_t, N * 8)) || (rc = ensure(h, h->ilu_zt, N * 8)) ||
             (rc = ensure(h, h->ilu_bad, sizeof(int))))
             return rc;
@@ -849,7 +850,11 @@ int ensure_ilu(sfgmres_ctx* h) {
         H.dev.perm = (const int*)h->ilu_perm.p;
         H.dev.lu = (double*)h->ilu_lu.p;
         H.dev.y = (double*)h->ilu_y.p;
-        H.dev.zp = (double*)h->ilu_zp.p;
+        H.dev.ocol = (const int*)h->ilu_ocol.p;
+        H.maxlen = h->maxlen;
+        H.piv = (double2*)h->ilu_piv.p;
+        H.dev.piv = H.piv;
+        CK(launch_ilu_columns(H, (int*)h->ilu_ocol.p, h->st));
         h->ilu_colour = colour;
         h->ilu_src = psrc;
         h->ilu_built = 1;
@@ -1640,7 +1645,7 @@ int sfgmres_destroy(sfgmres_t h) {
                       &h->x0st, &h->gsync};
     for (DevBuf* b : bufs) release(*b);
     for (DevBuf* b : {&h->ilu_rp, &h->ilu_col, &h->ilu_diag, &h->ilu_perm, &h->ilu_src_d, &h->ilu_lu, &h->ilu_y,
-                      &h->ilu_zp, &h->ilu_t, &h->ilu_zt, &h->ilu_bad})
+                      &h->ilu_ocol, &h->ilu_piv, &h->ilu_t, &h->ilu_zt, &h->ilu_bad})
         release(*b);
     for (auto& L : h->lvl)
         for (DevBuf* b : {&L.Vb, &L.Z, &L.nu, &L.Wo, &L.opart, &L.npart, &L.npart2, &L.h1, &L.h2, &L.H, &L.cs, &L.sn,

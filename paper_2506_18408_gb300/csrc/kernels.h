@@ -29,15 +29,17 @@ struct IluDev {
     const int* col = nullptr;   // [nnz] columns (permuted indices), sorted within each row
     const int* diag = nullptr;  // [n] position of the diagonal entry in its row
     const int* perm = nullptr;  // [n] original index of permuted row r
+    const int* ocol = nullptr;  // [nnz] columns as original indices, the top bit set past the first colour
     double* lu = nullptr;       // [nnz] L strictly below the diagonal (unit diagonal implied), U from the diagonal on
-    double* y = nullptr;        // [n] forward-pass vector (permuted order)
-    double* zp = nullptr;       // [n] backward-pass vector (permuted order)
+    const double2* piv = nullptr;  // [n] pivots u_rr and their reciprocals
+    double* y = nullptr;        // [n] forward-pass vector (original order)
 };
 // Host side of the preconditioner: the colour ranges the launchers loop over.
 struct IluHost {
-    int n = 0, ncol = 0;
+    int n = 0, ncol = 0, maxlen = 0;
     int64_t nnz = 0;
     std::vector<int> starts;   // [ncol + 1] first permuted row of each colour
+    double2* piv = nullptr;    // device [n]: dev.piv, written by the factorisation
     const int* src = nullptr;  // device [nnz]: position in A's CSR of every entry of P A P^T
     IluDev dev;
 };
@@ -234,6 +236,8 @@ void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r
 // ---- ILU(0) right preconditioning (precond.cu) ----
 // lu = the values of P A P^T (gathered from A's values), then ILU(0) colour by colour; *bad |= 1 on a zero pivot
 cudaError_t launch_ilu_factor(const IluHost& H, const double* val, int* bad, cudaStream_t st);
+// ocol from the permuted columns and the permutation (once, after the structure)
+cudaError_t launch_ilu_columns(const IluHost& H, int* ocol, cudaStream_t st);
 // out = M^{-1} u = P^T (L U)^{-1} P u in the original order (u and out n float64, distinct); i >= 0: step i of the
 // plan's cycle (the passes return at once once the cycle has stopped), i < 0: always
 void launch_ilu_apply(const Plan& P, int i, const double* u, double* out);

@@ -95,14 +95,14 @@ __device__ __forceinline__ void stage_issue(const int* __restrict__ col, const M
     for (int u = lane; va + VP * u < a1; u += 32) cp_async16(vdst + 16 * u, val + va + VP * u);
 }
 
-// Entries pk .. pk+CNT-1 of the lane's row (its first entry at cs, vs in shared memory); `release` runs once the
-// values are in registers.
-template <int CNT, typename MT, typename XT, typename AT, typename Release>
-__device__ __forceinline__ void staged_chunk(const int* cs, const MT* vs, const XT* __restrict__ x, int len, int pk,
-                                             AT& sum, Release&& release) {
+// Entries pk .. pk+CNT-1 of the lane's row (its first entry at cs, vs in shared memory), get(c) the factor of column c;
+// `release` runs once the values are in registers.
+template <int CNT, typename MT, typename AT, typename Get, typename Release>
+__device__ __forceinline__ void staged_chunk(const int* cs, const MT* vs, Get&& get, int len, int pk, AT& sum,
+                                             Release&& release) {
     AT xv[CNT], v[CNT];
 #pragma unroll
-    for (int q = 0; q < CNT; ++q) xv[q] = (pk + q < len) ? load_as(x + cs[pk + q], AT()) : AT(0);
+    for (int q = 0; q < CNT; ++q) xv[q] = (pk + q < len) ? get(cs[pk + q]) : AT(0);
 #pragma unroll
     for (int q = 0; q < CNT; ++q) v[q] = (pk + q < len) ? (AT)vs[pk + q] : AT(0);
     release();
@@ -111,13 +111,20 @@ __device__ __forceinline__ void staged_chunk(const int* cs, const MT* vs, const 
         if (pk + q < len) sum += v[q] * xv[q];
 }
 
+// The whole of every row (the default of rows_staged's Part).
+struct WholeRows {
+    __device__ __forceinline__ int load(int) const { return 0; }
+    __device__ __forceinline__ void cut(int, int, int&, int&) const {}
+};
+
 // For the len rows from matrix row r0 on (row pointers rpm = rp + r0): pre(k) before local row k's products (loads that
-// should be in flight with them), then emit(k, sum).  Lanes past the last row call both with k >= len.  buf: the CTA's
-// stage area (blockDim / 32 buffers of stage_bytes(maxlen)).
-template <typename MT, typename XT, typename AT, typename Pre, typename Emit>
-__device__ __forceinline__ void spmv_rows_staged(const int* __restrict__ rpm, const int* __restrict__ col,
-                                                 const MT* __restrict__ val, const XT* __restrict__ x, int len,
-                                                 unsigned char* buf, int maxlen, Pre&& pre, Emit&& emit) {
+// should be in flight with them), then emit(k, sum of val * get(col) over the row's entries, or over the part that
+// part.cut(part.load(k), first entry, offset, count) leaves of them; load runs a group ahead).  Lanes past the last row call
+// all with k >= len.  buf: the CTA's stage area (blockDim / 32 buffers of stage_bytes(maxlen)).
+template <typename MT, typename AT, typename Get, typename Part, typename Pre, typename Emit>
+__device__ __forceinline__ void rows_staged(const int* __restrict__ rpm, const int* __restrict__ col,
+                                            const MT* __restrict__ val, int len, unsigned char* buf, int maxlen,
+                                            Get&& get, Part part, Pre&& pre, Emit&& emit) {
     const int lane = threadIdx.x & 31;
     unsigned char* mine = buf + (threadIdx.x >> 5) * stage_bytes<MT>(maxlen);
     int* cbuf = reinterpret_cast<int*>(mine);
@@ -127,23 +134,26 @@ __device__ __forceinline__ void spmv_rows_staged(const int* __restrict__ rpm, co
     int kw = threadIdx.x & ~31;
     if (kw >= len) return;
     // first entry and length of the lane's row in the group at k0 (past the last row: its end, 0)
-    auto extent = [&](int k0, int& a, int& l) {
+    auto extent = [&](int k0, int& a, int& l, int& d) {
         a = __ldg(rpm + min(k0 + lane, len));
         l = __ldg(rpm + min(k0 + lane + 1, len)) - a;
+        d = part.load(k0 + lane);
     };
     auto issue = [&](int a, int l) {
         stage_issue(col, val, __shfl_sync(0xffffffffu, a, 0), __shfl_sync(0xffffffffu, a + l, 31), cdst, vdst, lane);
     };
-    int a, rl, an = 0, rln = 0;
-    extent(kw, a, rl);
+    int a, rl, d, an = 0, rln = 0, dn = 0;
+    extent(kw, a, rl, d);
     issue(a, rl);
-    if (kw + (int)blockDim.x < len) extent(kw + blockDim.x, an, rln);
+    if (kw + (int)blockDim.x < len) extent(kw + blockDim.x, an, rln, dn);
     for (; kw < len; kw += blockDim.x) {  // warp-uniform loop
         const bool more = kw + (int)blockDim.x < len;
         pre(kw + lane);
         const int a0 = __shfl_sync(0xffffffffu, a, 0);
-        const int* cs = cbuf + (a - (a0 & ~3));
-        const MT* vs = vbuf + (a - (a0 & ~(VP - 1)));
+        int off = 0;
+        if (kw + lane < len) part.cut(d, a, off, rl);
+        const int* cs = cbuf + (a + off - (a0 & ~3));
+        const MT* vs = vbuf + (a + off - (a0 & ~(VP - 1)));
         const int wm = (int)__reduce_max_sync(0xffffffffu, (unsigned)rl);
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
@@ -153,23 +163,33 @@ __device__ __forceinline__ void spmv_rows_staged(const int* __restrict__ rpm, co
             if (more) issue(an, rln);
         };
         int pk = 0;
-        for (; pk + 8 < wm; pk += 8) staged_chunk<8>(cs, vs, x, rl, pk, sum, [] {});
+        for (; pk + 8 < wm; pk += 8) staged_chunk<8>(cs, vs, get, rl, pk, sum, [] {});
         switch (wm - pk) {
-            case 1: staged_chunk<1>(cs, vs, x, rl, pk, sum, release); break;
-            case 2: staged_chunk<2>(cs, vs, x, rl, pk, sum, release); break;
-            case 3: staged_chunk<3>(cs, vs, x, rl, pk, sum, release); break;
-            case 4: staged_chunk<4>(cs, vs, x, rl, pk, sum, release); break;
-            case 5: staged_chunk<5>(cs, vs, x, rl, pk, sum, release); break;
-            case 6: staged_chunk<6>(cs, vs, x, rl, pk, sum, release); break;
-            case 7: staged_chunk<7>(cs, vs, x, rl, pk, sum, release); break;
-            case 8: staged_chunk<8>(cs, vs, x, rl, pk, sum, release); break;
+            case 1: staged_chunk<1>(cs, vs, get, rl, pk, sum, release); break;
+            case 2: staged_chunk<2>(cs, vs, get, rl, pk, sum, release); break;
+            case 3: staged_chunk<3>(cs, vs, get, rl, pk, sum, release); break;
+            case 4: staged_chunk<4>(cs, vs, get, rl, pk, sum, release); break;
+            case 5: staged_chunk<5>(cs, vs, get, rl, pk, sum, release); break;
+            case 6: staged_chunk<6>(cs, vs, get, rl, pk, sum, release); break;
+            case 7: staged_chunk<7>(cs, vs, get, rl, pk, sum, release); break;
+            case 8: staged_chunk<8>(cs, vs, get, rl, pk, sum, release); break;
             default: release(); break;  // rows without entries
         }
         emit(kw + lane, sum);
         a = an;
         rl = rln;
-        if (kw + 2 * (int)blockDim.x < len) extent(kw + 2 * (int)blockDim.x, an, rln);
+        d = dn;
+        if (kw + 2 * (int)blockDim.x < len) extent(kw + 2 * (int)blockDim.x, an, rln, dn);
     }
+}
+
+// rows_staged of whole rows against a vector x: A x.
+template <typename MT, typename XT, typename AT, typename Pre, typename Emit>
+__device__ __forceinline__ void spmv_rows_staged(const int* __restrict__ rpm, const int* __restrict__ col,
+                                                 const MT* __restrict__ val, const XT* __restrict__ x, int len,
+                                                 unsigned char* buf, int maxlen, Pre&& pre, Emit&& emit) {
+    rows_staged<MT, AT>(rpm, col, val, len, buf, maxlen, [&](int c) { return load_as(x + c, AT()); }, WholeRows(), pre,
+                        emit);
 }
 
 // Same result with each row handled by a sub-warp of V lanes; a warp processes U sub-warp rows at once (all their

@@ -332,12 +332,21 @@ void choose_lists(sfgmres_ctx* h, int nrhs) {
     if (h->sys_Bq.empty() || h->sys_Bq[0] != Bq) set_list_geometry(h, Bq);
 }
 
-// Shared memory left on an SM beside the inner step's CTAs (one or two of them, by the number of row blocks; 8 KB each
-// for their static shared memory and the reserve), for a sketched-QR CTA to run there at the same time.
-size_t qr_smem_left(int nblk, int sms, size_t step_smem) {
-    const size_t per_sm = (nblk > sms) ? 2 : 1;
-    const size_t used = per_sm * (step_smem + 8 * 1024), all = 226 * 1024;
-    return used < all ? all - used : 0;
+// Shared memory that a sketched-QR CTA may take (6 to 8 KB per step CTA for its static shared memory and the reserve).  Steps of
+// one launch that fill the SMs do best with the QR staged, waiting for an SM that their CTAs leave, and not beside two of them
+// (128^3 solve FP64 46.8 ms against 54.0, FP32 42.0 against 54.7, 80^3 cycle at s = 1000 9.5 against 10.5).  Where a step is two
+// launches that wait would come back as a second wave of the next SpMV (2M Zipf rows, FP64: 501 ms against 305): the QR then has
+// to fit beside two CTAs, within the carveout that they chose, the smallest that holds them.
+size_t qr_smem_left(int nblk, int sms, size_t step_smem, bool two_launches) {
+    constexpr size_t KB = 1024;
+    if (nblk <= sms || !two_launches) {
+        const size_t used = (nblk > sms ? 2 : 1) * (step_smem + 8 * KB);
+        return used < 226 * KB ? 226 * KB - used : 0;
+    }
+    const size_t used = 2 * (step_smem + 6 * KB);
+    for (size_t carveout : {8, 16, 32, 64, 100, 132, 164, 196, 228})
+        if (carveout * KB >= used) return carveout * KB - used;
+    return 0;
 }
 
 // ---- CSR validation on the device ----
@@ -916,7 +925,8 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->cpart, nb * S * at))) return rc;
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
     const size_t stage = staged ? stage_smem(maxlen) : 0;
-    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage));
+    const bool two = (vec == 0 && h->prec == kFP64) || t > 4 || !h->fuse_step;  // steps of two launches (launch_inner_step)
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, two));
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;

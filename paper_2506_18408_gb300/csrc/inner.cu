@@ -534,7 +534,7 @@ QrShape qr_shape(int P, int s, int m, size_t smem_left) {
     q.nrp = ((s + q.cluster - 1) / q.cluster) | 1;
     q.slice = (q.nrp * m + 1) & ~1;
     q.staged = true;
-    q.staged = qr_smem(q, m, m - 1) <= smem_left;
+    q.staged = qr_smem(q, m, m - 1) + 3072 <= smem_left;  // its static shared memory and the reserve
     return q;
 }
 

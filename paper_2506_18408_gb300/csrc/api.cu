@@ -68,14 +68,16 @@ struct ListSet {
     int bins_ver[2] = {-1, -1};
     int* lb = nullptr;  // lb_m0 [nl], lb_len [nl]
     int lb_ver = -1;
-    // the length-binned SpMV's FP64 copies of A [0] and A^T [1] with each row block's rows in its processing order
-    // (built for one geometry version; values follow sfgmres_update_values)
-    struct BCopy {
-        int* rp = nullptr;
+    // the length-binned SpMV's sorted copies of A [0] and A^T [1] (values follow sfgmres_update_values; ver: the version
+    // of the matrix values they hold, -1: not built)
+    struct Sorted {
+        int* off = nullptr;
+        uint16_t* len = nullptr;
         int* col = nullptr;
         double* val = nullptr;
+        float* val32 = nullptr;
         int ver = -1;
-    } bc[2];
+    } so[2];
 
     // sketch gather lists (cached for one (s, zeta, kind, geometry version))
     int sk_s = -1, sk_zeta = -1, sk_kind = -1, sk_ver = -1, sk_headroom = 0, sk_word = 0;
@@ -305,7 +307,14 @@ int want_block_rows(const sfgmres_ctx* h, int nrhs) {
     return rows;
 }
 
+void drop_sorted(ListSet::Sorted& S) {
+    for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val, (void*)S.val32})
+        if (q) cudaFree(q);
+    S = ListSet::Sorted();
+}
+
 void set_list_geometry(sfgmres_ctx* h, int Bq) {
+    for (auto& S : h->so) drop_sorted(S);  // built for the old blocks
     h->sys_Bq.assign(h->nsys, 0);
     h->sys_l0.assign(h->nsys + 1, 0);
     int Bn = 32, nl = 0;
@@ -332,14 +341,15 @@ void choose_lists(sfgmres_ctx* h, int nrhs) {
     if (h->sys_Bq.empty() || h->sys_Bq[0] != Bq) set_list_geometry(h, Bq);
 }
 
-// Shared memory that a sketched-QR CTA may take (6 to 8 KB per step CTA for its static shared memory and the reserve).  Steps of
-// one launch that fill the SMs do best with the QR staged, waiting for an SM that their CTAs leave, and not beside two of them
-// (128^3 solve FP64 46.8 ms against 54.0, FP32 42.0 against 54.7, 80^3 cycle at s = 1000 9.5 against 10.5).  Where a step is two
-// launches that wait would come back as a second wave of the next SpMV (2M Zipf rows, FP64: 501 ms against 305): the QR then has
-// to fit beside two CTAs, within the carveout that they chose, the smallest that holds them.
-size_t qr_smem_left(int nblk, int sms, size_t step_smem, bool two_launches) {
+// Shared memory that a sketched-QR CTA may take (6 to 8 KB per step CTA for its static shared memory and the reserve).  A
+// stencil's steps of one launch that fill the SMs do best with the QR staged, waiting for an SM that their CTAs leave, and not
+// beside two of them (128^3 solve FP64 46.8 ms against 54.0, FP32 42.0 against 54.7, 80^3 cycle at s = 1000 9.5 against 10.5).
+// The longer steps of the length-binned SpMV, and steps of two launches, would pay for that wait with a second wave of the
+// next SpMV on those SMs (2M Zipf rows, FP64: 494 us per step against 299; 1.5M, FP32: 318 against 179): there the QR
+// has to fit beside two CTAs, within the carveout that they chose, the smallest that holds them.
+size_t qr_smem_left(int nblk, int sms, size_t step_smem, bool beside) {
     constexpr size_t KB = 1024;
-    if (nblk <= sms || !two_launches) {
+    if (nblk <= sms || !beside) {
         const size_t used = (nblk > sms ? 2 : 1) * (step_smem + 8 * KB);
         return used < 226 * KB ? 226 * KB - used : 0;
     }
@@ -629,36 +639,88 @@ int ensure_bins(sfgmres_ctx* h, bool transpose) {
     if (!h->perm[t]) CK(cudaMalloc(&h->perm[t], std::max<size_t>(h->n, 1) * sizeof(uint16_t)));
     if (h->cls[t]) cudaFree(h->cls[t]);
     h->cls[t] = nullptr;
-    CK(cudaMalloc(&h->cls[t], 2 * (size_t)h->nl * sizeof(int)));
+    CK(cudaMalloc(&h->cls[t], 3 * (size_t)h->nl * sizeof(int)));
     launch_bin_rows(h->nl, transpose ? h->rpT : h->rp, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->st);
     CK(cudaGetLastError());
     h->bins_ver[t] = h->geo_ver;
     return 0;
 }
 
-// The length-binned SpMV's copy of A (or A^T): every row block's rows stored in the order the SpMV processes them
-// (the bins of the current geometry), FP64 values.
-int ensure_bcopy(sfgmres_ctx* h, bool transpose) {
+// Slices of 32 rows: their number over all systems, each system's first and the first of every list block (whose sizes are
+// multiples of 32).
+int ensure_slices(sfgmres_ctx* h) {
+    if (!h->sl_sys) {
+        std::vector<int> t(2 * (size_t)(h->nsys + 1), 0);
+        int64_t ns = 0;
+        for (int q = 0; q < h->nsys; ++q) {
+            t[q] = (int)ns;
+            ns += (h->sys_n[q] + 31) / 32;
+        }
+        if (ns > INT32_MAX - 1) return fail(h, SFGMRES_ERR_INVALID_ARG, "too many rows for slices of 32");
+        t[h->nsys] = (int)ns;
+        for (int q = 0; q <= h->nsys; ++q) t[h->nsys + 1 + q] = h->sys_moff[q];
+        CK(cudaMalloc(&h->sl_sys, t.size() * sizeof(int)));
+        CK(cudaMemcpy(h->sl_sys, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice));
+        h->sl_ns = (int)ns;
+    }
+    if (h->sl_base_ver != h->geo_ver) {
+        std::vector<int> hb((size_t)std::max(h->nl, 1), 0);
+        int ns0 = 0;
+        for (int q = 0; q < h->nsys; ++q) {
+            const int nq = h->sys_n[q], Bq = h->sys_Bq[q];
+            for (int k = 0, L = h->sys_l0[q]; k * Bq < nq; ++k, ++L) hb[L] = ns0 + k * (Bq / 32);
+            ns0 += (nq + 31) / 32;
+        }
+        if (h->sl_base) cudaFree(h->sl_base);
+        h->sl_base = nullptr;
+        CK(cudaMalloc(&h->sl_base, hb.size() * sizeof(int)));
+        CK(cudaMemcpy(h->sl_base, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice));
+        h->sl_base_ver = h->geo_ver;
+    }
+    return 0;
+}
+
+// The length-binned SpMV's sorted copy of A (or A^T): the rows of the current bins that take a thread each, as slices of the
+// block's length order, with FP64 values and, for FP32 and BF16 inner cycles, FP32 ones.
+int ensure_sorted(sfgmres_ctx* h, bool transpose) {
     const int t = transpose ? 1 : 0;
-    ListSet::BCopy& B = h->bc[t];
-    if (B.ver == h->geo_ver && B.rp) return 0;
+    ListSet::Sorted& S = h->so[t];
+    const bool f32 = h->prec != kFP64;
+    if (S.ver == h->vals_ver && (S.val32 || !f32)) return 0;
+    int rc;
+    if ((rc = ensure_slices(h))) return rc;
     const int* rp = transpose ? h->rpT : h->rp;
     const int* col = transpose ? h->colT : h->col;
     const double* val = transpose ? h->valT : h->val;
-    const size_t n = (size_t)h->n, nnz = (size_t)std::max<int64_t>(h->nnz, 1);
-    if (!B.rp) {
-        CK(cudaMalloc(&B.rp, (n + 1) * sizeof(int)));
-        CK(cudaMalloc(&B.col, nnz * sizeof(int)));
-        CK(cudaMalloc(&B.val, nnz * sizeof(double)));
+    const int ns = h->sl_ns;
+    const bool fresh = S.ver < 0;
+    int64_t total = 0;
+    if (fresh) {
+        drop_sorted(S);  // what a failed build left
+        int* wid = nullptr;
+        CK(cudaMalloc(&wid, std::max<size_t>((size_t)ns, 1) * sizeof(int)));
+        CK(cudaMalloc(&S.off, ((size_t)ns + 1) * sizeof(int)));
+        CK(cudaMalloc(&S.len, std::max<size_t>((size_t)ns, 1) * 32 * sizeof(uint16_t)));
+        launch_sorted_build(h->nl, ns, rp, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->sl_base, S.len, wid, S.off,
+                            h->st);
+        int tot = 0;
+        CK(cudaMemcpyAsync(&tot, S.off + ns, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+        CK(cudaStreamSynchronize(h->st));
+        cudaFree(wid);
+        CK(cudaGetLastError());
+        total = std::max<int64_t>((int64_t)tot * 32, 1);
+        CK(cudaMalloc(&S.col, total * sizeof(int)));
+        CK(cudaMalloc(&S.val, total * sizeof(double)));
+    } else if (f32 && !S.val32) {
+        int tot = 0;
+        CK(cudaMemcpy(&tot, S.off + ns, sizeof(int), cudaMemcpyDeviceToHost));
+        total = std::max<int64_t>((int64_t)tot * 32, 1);
     }
-    int* lens = nullptr;
-    CK(cudaMalloc(&lens, std::max<size_t>(n, 1) * sizeof(int)));
-    launch_bcopy_build(h->n, h->nl, rp, h->lb, h->lb + h->nl, h->perm[t], lens, B.rp, h->st);
-    launch_bcopy_fill(h->nl, rp, col, val, h->lb, h->lb + h->nl, h->perm[t], B.rp, B.col, B.val, h->st);
-    CK(cudaStreamSynchronize(h->st));
-    cudaFree(lens);
+    if (f32 && !S.val32) CK(cudaMalloc(&S.val32, total * sizeof(float)));
+    launch_sorted_fill(h->nl, rp, col, val, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->sl_base, S.off,
+                       fresh ? S.col : nullptr, S.val, S.val32, h->st);
     CK(cudaGetLastError());
-    B.ver = h->geo_ver;
+    S.ver = h->vals_ver;
     return 0;
 }
 
@@ -670,20 +732,8 @@ int ensure_sell(sfgmres_ctx* h, bool transpose) {
     const int* rp = transpose ? h->rpT : h->rp;
     const int* col = transpose ? h->colT : h->col;
     const double* val = transpose ? h->valT : h->val;
-    if (!h->sl_sys) {
-        std::vector<int> t(2 * (size_t)(h->nsys + 1), 0);
-        int64_t ns = 0;
-        for (int q = 0; q < h->nsys; ++q) {
-            t[q] = (int)ns;
-            ns += (h->sys_n[q] + 31) / 32;
-        }
-        if (ns > INT32_MAX - 1) return fail(h, SFGMRES_ERR_INVALID_ARG, "too many rows for the SELL-32 layout");
-        t[h->nsys] = (int)ns;
-        for (int q = 0; q <= h->nsys; ++q) t[h->nsys + 1 + q] = h->sys_moff[q];
-        CK(cudaMalloc(&h->sl_sys, t.size() * sizeof(int)));
-        CK(cudaMemcpy(h->sl_sys, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice));
-        h->sl_ns = (int)ns;
-    }
+    int rc;
+    if ((rc = ensure_slices(h))) return rc;
     const int ns = h->sl_ns;
     const int* sl0 = h->sl_sys;
     const int* moff = h->sl_sys + h->nsys + 1;
@@ -704,20 +754,6 @@ int ensure_sell(sfgmres_ctx* h, bool transpose) {
         launch_sell_fill(ns, sl0, h->nsys, moff, rp, col, val, S.off, S.len, S.col, S.val, h->st);
         CK(cudaGetLastError());
     }
-    if (h->sl_base_ver != h->geo_ver) {
-        std::vector<int> hb((size_t)std::max(h->nl, 1), 0);
-        int ns0 = 0;
-        for (int q = 0; q < h->nsys; ++q) {
-            const int nq = h->sys_n[q], Bq = h->sys_Bq[q];
-            for (int k = 0, L = h->sys_l0[q]; k * Bq < nq; ++k, ++L) hb[L] = ns0 + k * (Bq / 32);
-            ns0 += (nq + 31) / 32;
-        }
-        if (h->sl_base) cudaFree(h->sl_base);
-        h->sl_base = nullptr;
-        CK(cudaMalloc(&h->sl_base, hb.size() * sizeof(int)));
-        CK(cudaMemcpy(h->sl_base, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice));
-        h->sl_base_ver = h->geo_ver;
-    }
     return 0;
 }
 
@@ -732,11 +768,14 @@ void plan_geometry(sfgmres_ctx* h, const Geo* g, bool transpose, Plan& P) {
     P.maxlen = transpose ? h->maxlenT : h->maxlen;
     P.perm = (P.vec == 0) ? h->perm[transpose ? 1 : 0] : nullptr;
     P.cls = (P.vec == 0) ? h->cls[transpose ? 1 : 0] : nullptr;
-    const ListSet::BCopy& B = h->bc[transpose ? 1 : 0];
-    const bool bc = (P.vec == 0) && B.rp && B.ver == h->geo_ver && h->bins_ver[transpose ? 1 : 0] == h->geo_ver;
-    P.brp = bc ? B.rp : nullptr;
-    P.bcol = bc ? B.col : nullptr;
-    P.bval = bc ? B.val : nullptr;
+    const ListSet::Sorted& O = h->so[transpose ? 1 : 0];
+    const bool so = P.vec == 0 && O.ver == h->vals_ver;
+    P.so_off = so ? O.off : nullptr;
+    P.so_len = so ? O.len : nullptr;
+    P.so_col = so ? O.col : nullptr;
+    P.so_val = so ? O.val : nullptr;
+    P.so_val32 = so ? O.val32 : nullptr;
+    P.so_base = so ? h->sl_base : nullptr;
     const sfgmres_ctx::Sell& S = h->sell[transpose ? 1 : 0];
     const bool sl = (P.vec == 1) && h->prec == kFP64 && S.off && h->sl_base_ver == h->geo_ver;
     P.sl_off = sl ? S.off : nullptr;
@@ -909,7 +948,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     const int maxlen = transpose ? h->maxlenT : h->maxlen;
     const bool staged = vec == 1 && h->prec != kFP64 && stage_fits(h, g->nblk, maxlen);
     if (vec == 0 && (rc = ensure_bins(h, transpose))) return rc;
-    if (vec == 0 && (rc = ensure_bcopy(h, transpose))) return rc;
+    if (vec == 0 && (rc = ensure_sorted(h, transpose))) return rc;
     if (vec == 1 && h->prec == kFP64 && (rc = ensure_sell(h, transpose))) return rc;
     const size_t vt = (h->prec == kFP64) ? 8 : (h->prec == kFP32 ? 4 : 2);
     const size_t at = (h->prec == kFP64) ? 8 : 4;
@@ -925,8 +964,8 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->cpart, nb * S * at))) return rc;
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
     const size_t stage = staged ? stage_smem(maxlen) : 0;
-    const bool two = (vec == 0 && h->prec == kFP64) || t > 4 || !h->fuse_step;  // steps of two launches (launch_inner_step)
-    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, two));
+    const bool beside = vec == 0 || t > 4 || !h->fuse_step;  // binned, or steps of two launches (launch_inner_step)
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), beside);
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;
@@ -1145,8 +1184,8 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
                           (const void*)P.ffom_hist, (const void*)P.ires_hist, (const void*)P.rho_hist,
                           (const void*)P.k_hist, (const void*)P.reason_hist,
                           (const void*)P.ost, (const void*)P.st, (const void*)h->qst, (const void*)P.gsync,
-                          (const void*)P.xin, (const void*)P.ilu.lu, (const void*)P.brp, (const void*)P.bcol,
-                          (const void*)P.bval})
+                          (const void*)P.xin, (const void*)P.ilu.lu, (const void*)P.so_off, (const void*)P.so_col,
+                          (const void*)P.so_val, (const void*)P.so_val32})
         u(p);
     for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.staged, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
                       (int64_t)P.s, (int64_t)P.zeta, (int64_t)P.kind, (int64_t)P.sk_headroom, (int64_t)P.prec,
@@ -1640,9 +1679,7 @@ int sfgmres_destroy(sfgmres_t h) {
         for (void* q : {(void*)L->seg, (void*)L->ent, (void*)L->lb, (void*)L->sl_base, (void*)L->perm[0],
                         (void*)L->perm[1], (void*)L->cls[0], (void*)L->cls[1]})
             if (q) cudaFree(q);
-        for (auto& B : L->bc)
-            for (void* q : {(void*)B.rp, (void*)B.col, (void*)B.val})
-                if (q) cudaFree(q);
+        for (auto& S : L->so) drop_sorted(S);
     }
     for (auto& S : h->sell)
         for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val})
@@ -1938,14 +1975,12 @@ int sfgmres_update_values(sfgmres_t h, const double* vals) {
         launch_gather_vals(h->nnz, h->srcT, h->val, h->valT, h->st);
         if (h->val32T) k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, h->valT, h->val32T);
     }
-    for (auto& B : h->other.bc) B.ver = -1;  // the other list blocks' copies: rebuilt at their next use
-    for (int t = 0; t < 2; ++t) {  // the length-binned copies' values
-        ListSet::BCopy& B = h->bc[t];
-        if (B.rp && B.ver == h->geo_ver && h->perm[t])
-            launch_bcopy_fill(h->nl, t ? h->rpT : h->rp, nullptr, t ? h->valT : h->val, h->lb, h->lb + h->nl,
-                              h->perm[t], B.rp, nullptr, B.val, h->st);
-        else
-            B.ver = -1;  // rebuilt at the next use
+    for (int t = 0; t < 2; ++t) {  // the current sorted copies' values (the other list blocks' follow at their next use)
+        ListSet::Sorted& S = h->so[t];
+        if (S.ver < 0) continue;
+        launch_sorted_fill(h->nl, t ? h->rpT : h->rp, nullptr, t ? h->valT : h->val, h->lb, h->lb + h->nl, h->perm[t],
+                           h->cls[t], h->sl_base, S.off, nullptr, S.val, S.val32, h->st);
+        S.ver = h->vals_ver;
     }
     for (int t = 0; t < 2; ++t) {  // the SELL-32 copies' values
         sfgmres_ctx::Sell& S = h->sell[t];

@@ -525,12 +525,13 @@ static size_t qr_smem(const QrShape& q, int m, int i) {
 // Few CTAs where an update's FP64 work is small (its latency is then the exchanges, which grow with the CTAs), many where it
 // is large.  Whole solves, 2 / 4 / 8 / 16 CTAs: s = 80, m = 20 (2D 32^2) 2.40 / 2.51 / 2.54 / 2.49 ms; s = 120, m = 30 (2D
 // 64^2) 4.34 / 4.12 / 5.21 / 5.03 ms; s = 240, m = 60 (3D 32^3) 3.36 / 3.19 / 3.56 / 3.41 ms; s = 320, m = 80 (40^3) 4.96 / 4.47
-// / 4.06 / 3.90 ms; s = 1000, m = 200 (80^3) 44.3 / 28.9 / 20.9 / 15.9 ms.  Batches take what leaves the problems' clusters
+// / 4.06 / 3.90 ms; s = 1000, m = 200 (80^3) 44.3 / 28.9 / 20.9 / 15.9 ms; beside the length-binned SpMV, s = 120, m = 30
+// (30,000 Zipf rows) 19.6 / 20.8 / 20.8 / 20.9 ms.  Batches take what leaves the problems' clusters
 // side by side on the GPU.
-QrShape qr_shape(int P, int s, int m, size_t smem_left) {
+QrShape qr_shape(int P, int s, int m, size_t smem_left, bool beside) {
     QrShape q;
     const int most = P <= 4 ? kQrCluster : P <= 16 ? 8 : P <= 32 ? 4 : P <= 64 ? 2 : 1;
-    q.cluster = std::min(most, s * m <= 3000 ? 2 : s * m <= 20000 ? 4 : kQrCluster);
+    q.cluster = std::min(most, s * m <= (beside ? 5000 : 3000) ? 2 : s * m <= 20000 ? 4 : kQrCluster);
     q.nrp = ((s + q.cluster - 1) / q.cluster) | 1;
     q.slice = (q.nrp * m + 1) & ~1;
     q.staged = true;

@@ -72,12 +72,14 @@ struct Plan {
     const double* sl_val = nullptr;
     const int* sl_base = nullptr;
     const uint16_t* perm = nullptr;  // length-binned SpMV: per matrix row block, its rows in length order
-    // the length-binned SpMV's FP64 copy of A with each block's rows stored in that order (null: read the CSR
-    // arrays through perm): row i of block L's order at brp[m0 + i] .. brp[m0 + i + 1] of bcol/bval
-    const int* brp = nullptr;
-    const int* bcol = nullptr;
-    const double* bval = nullptr;
-    const int* cls = nullptr;        // [2 * list blocks]: rows with <= 16 entries, rows with <= 64 entries
+    const int* cls = nullptr;        // [3 * list blocks] rows of the order with <= 16 entries, with <= 64, in the copy
+    // the length-binned SpMV's sorted copy (null: the CSR arrays through perm): slices of 32 rows of the order
+    const int* so_off = nullptr;       // slice widths as prefix sums in units of 32 entries
+    const uint16_t* so_len = nullptr;  // per-lane row lengths
+    const int* so_col = nullptr;
+    const double* so_val = nullptr;
+    const float* so_val32 = nullptr;   // FP32 values (inner FP32/BF16 modes)
+    const int* so_base = nullptr;      // first slice of every list block
 
     // problems and row blocks
     int N = 0;                     // total vector length (sum over problems)
@@ -173,10 +175,31 @@ __device__ __forceinline__ BlockInfo block_info(const Plan& p, int b) {
     return bi;
 }
 
-// Length-class boundaries of block b's rows for the length-binned SpMV (zero when the plan has none).
-__device__ __forceinline__ void block_bins(const Plan& p, const BlockInfo& bi, int& n0, int& n01) {
-    n0 = p.cls ? p.cls[2 * bi.list] : 0;
-    n01 = p.cls ? p.cls[2 * bi.list + 1] : 0;
+// What the length-binned SpMV knows of a block: the rows of its order with at most 16 and at most 64 entries, and the sorted
+// copy's slices with the number of rows they hold (off null: no copy).
+template <typename MT>
+struct SortedRows {
+    int n16, n64, na;
+    const int* off;
+    const uint16_t* len;
+    const int* col;
+    const MT* val;
+};
+template <typename MT>
+__device__ __forceinline__ SortedRows<MT> sorted_rows(const Plan& p, const BlockInfo& bi) {
+    SortedRows<MT> s;
+    s.n16 = p.cls[3 * bi.list];
+    s.n64 = p.cls[3 * bi.list + 1];
+    s.na = p.cls[3 * bi.list + 2];
+    const MT* val;
+    if constexpr (sizeof(MT) == 8) val = p.so_val;
+    else val = p.so_val32;
+    const int base = val ? p.so_base[bi.list] : 0;
+    s.off = val ? p.so_off + base : nullptr;
+    s.len = p.so_len + (int64_t)base * 32;
+    s.col = p.so_col;
+    s.val = val;
+    return s;
 }
 
 // ---- sketch (sketch.cu) ----
@@ -227,8 +250,9 @@ void inner_axpy_f64(const Plan& p, int i, bool last);
 void inner_axpy_f32(const Plan& p, int i, bool last);
 void inner_axpy_bf16(const Plan& p, int i, bool last);
 void launch_inner_axpy(const Plan& p, int i, bool last);
-// For P problems, sketch size s and basis size m, given the shared memory left on an SM beside the inner step's CTAs.
-QrShape qr_shape(int P, int s, int m, size_t smem_left);
+// For P problems, sketch size s and basis size m, given the shared memory a QR CTA may take; beside: the step is not one launch of a
+// stencil, and the QR runs on the SMs of its CTAs.
+QrShape qr_shape(int P, int s, int m, size_t smem_left, bool beside);
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st
 void launch_inner_finish(const Plan& p, double* z);  // y = R^{-1} d, z = sum_l y_l b_l (FP64)
 void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r] = sigma_l * u_l[r] (FP64)
@@ -260,17 +284,18 @@ void launch_gather_vals(int64_t nnz, const int* src, const double* val, double* 
 void launch_pattern_outer(int n, const int* rp, const int* col, const double* u, const double* v, double alpha,
                           double* out, cudaStream_t st);
 // Row order of every matrix row block (nl blocks, block L = rows lb_m0[L] .. + lb_len[L]) for the length-binned
-// SpMV: perm[m0 + i] = local offset of the i-th row in (class, length, position) order; cls[2L], cls[2L+1] = number
-// of rows with at most 16 and at most 64 entries.
+// SpMV: perm[m0 + i] = local offset of the i-th row by (length, position); cls[3L ..]: rows with at most 16 entries, with
+// at most 64, and rows the sorted copy takes.
+constexpr int kSortedMax = 512;  // longest row of the sorted copy
 void launch_bin_rows(int nl, const int* rp, const int* lb_m0, const int* lb_len, uint16_t* perm, int* cls,
                      cudaStream_t st);
-// The length-binned SpMV's copy: lens [n] (scratch) and brp [n + 1] from the row order perm of every list block
-// (launch_bcopy_build), then columns (when bcol is not null) and values in that order (launch_bcopy_fill).
-void launch_bcopy_build(int n, int nl, const int* rp, const int* lb_m0, const int* lb_len, const uint16_t* perm,
-                        int* lens, int* brp, cudaStream_t st);
-void launch_bcopy_fill(int nl, const int* rp, const int* col, const double* val, const int* lb_m0,
-                       const int* lb_len, const uint16_t* perm, const int* brp, int* bcol, double* bval,
-                       cudaStream_t st);
+// The sorted copy (ns slices, base[L] the first of block L): lengths, widths and offsets, then columns (when scol is not null)
+// and values (FP64, FP32, or both).
+void launch_sorted_build(int nl, int ns, const int* rp, const int* lb_m0, const int* lb_len, const uint16_t* perm,
+                         const int* cls, const int* base, uint16_t* len, int* wid, int* off, cudaStream_t st);
+void launch_sorted_fill(int nl, const int* rp, const int* col, const double* val, const int* lb_m0, const int* lb_len,
+                        const uint16_t* perm, const int* cls, const int* base, const int* off, int* scol, double* sval,
+                        float* sval32, cudaStream_t st);
 // SELL-32 copy of a matrix whose rows have at most 255 entries: ns slices of 32 rows, slice s covering rows
 // moff[q] + 32 (s - sl0[q]) .. of system q (sl0: first slice of each system, nsys + 1 entries).  launch_sell_build
 // writes the row lengths len[ns * 32], the slice widths wid[ns] and their prefix sums off[ns + 1] (in units of 32

@@ -31,11 +31,9 @@ __device__ __forceinline__ void block_spmv(const Plan& P, const BlockInfo& bi, i
                                                  });
     } else {
         double* yb = reinterpret_cast<double*>(smem);
-        const bool copy = V == 0 && P.brp;
-        int n0, n01;
-        block_bins(P, bi, n0, n01);
-        spmv_rows_to_smem<V, U, double, double, double>(P.rp, copy ? P.bcol : P.col, copy ? P.bval : P.val, x + bi.cs,
-                                                        m0, m0 + len, yb, P.perm, n0, n01, V == 0 ? P.brp : nullptr);
+        SortedRows<double> so{};
+        if constexpr (V == 0) so = sorted_rows<double>(P, bi);
+        spmv_rows_to_smem<V, U, double, double, double>(P.rp, P.col, P.val, x + bi.cs, m0, m0 + len, yb, P.perm, so);
         __syncthreads();
         for (int k = threadIdx.x; k < len; k += blockDim.x) emit(k0 + k, yb[k]);
     }

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "kernels.h"
 
 namespace sfg {
 
@@ -254,7 +255,7 @@ template <int V, int U, int E, typename MT, typename XT, typename AT>
 __device__ __forceinline__ void spmv_sorted_vector(const int* __restrict__ rpm, const int* __restrict__ col,
                                                    const MT* __restrict__ val, const XT* __restrict__ x,
                                                    const uint16_t* __restrict__ pm, int lo, int hi,
-                                                   AT* __restrict__ out, const int* __restrict__ brpm) {
+                                                   AT* __restrict__ out) {
     constexpr int SUBS = 32 / V;
     constexpr int TILE = SUBS * U;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -270,7 +271,7 @@ __device__ __forceinline__ void spmv_sorted_vector(const int* __restrict__ rpm, 
             len[u] = 0;
             if (i < hi) {
                 kk[u] = pm[i];
-                const int* rq = brpm ? brpm + i : rpm + kk[u];  // the copy in processing order, or the CSR row
+                const int* rq = rpm + kk[u];
                 beg[u] = __ldg(rq);
                 len[u] = __ldg(rq + 1) - beg[u];
             }
@@ -308,57 +309,106 @@ __device__ __forceinline__ void spmv_sorted_vector(const int* __restrict__ rpm, 
     }
 }
 
+// CNT entries of the lane's row in a slice of the sorted copy (cp, vp: the lane's first; consecutive entries 32 apart),
+// entries past the row's end (rl) not gathered.  The matrix streams through once: loads that do not stay in the caches.
+template <int CNT, typename MT, typename XT, typename AT>
+__device__ __forceinline__ void sorted_chunk(const int* __restrict__ cp, const MT* __restrict__ vp,
+                                             const XT* __restrict__ x, int rl, int pk, AT& sum) {
+    int c[CNT];
+    AT xv[CNT], v[CNT];
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) c[q] = __ldcs(cp + (pk + q) * 32);
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) v[q] = (AT)__ldcs(vp + (pk + q) * 32);
+#pragma unroll
+    for (int q = 0; q < CNT; ++q) xv[q] = (pk + q < rl) ? load_as(x + c[q], AT()) : AT(0);
+#pragma unroll
+    for (int q = 0; q < CNT; ++q)
+        if (pk + q < rl) sum += v[q] * xv[q];
+}
+
 // Length-binned SpMV of one block for matrices with irregular rows: out[k] for the block's local rows k, matrix rows
-// m0 + k.  The block's rows come in a precomputed order pm[0 .. len) (local offsets): first the rows with at most 16
-// entries sorted by length (n0 of them), then rows of 17..64 entries (up to n01), then longer rows.  Short rows take
-// one thread each: a warp's 32 rows have (nearly) the same length, so the compile-time chunk loop issues about as
-// many FMAs as there are entries and 32 rows' loads are in flight per warp.  Medium rows take 8 lanes, long rows a
-// whole warp.  Every row's sum still runs over its entries in a fixed order (per lane, then a fixed shuffle tree).
-// With brp (the copy of the matrix that stores each block's rows in this order: row i at brp[m0 + i], col and val
-// then being that copy's arrays) the rows processed together are neighbours in memory; without it the CSR rows are
-// read through pm.
+// m0 + k.  The block's rows come in a precomputed order pm[0 .. len) (local offsets), by length.  With the sorted copy its
+// first so.na rows take one thread each, 32 rows of (nearly) one length per warp from a slice that the warp reads
+// coalesced: every FP64 instruction does 32 rows' products and no sum needs a shuffle tree (with 8 lanes or a warp per row
+// the trees and half-empty passes doubled the FP64 instructions of a 2M-row Zipf matrix, on a GPU whose FP64 pipe takes 17
+// cycles per warp and instruction).  Warps take the slices longest first, in alternating direction, so that their loads
+// even out.  ZIPF_TIMES
+// The rows that the copy leaves (too long for the block, or slices that would be half empty), and without a copy the rows beyond
+// 16 entries, take 8 lanes (17..64 entries) or a warp from the CSR arrays.  Every row's sum runs over its entries in a
+// fixed order.
 template <typename MT, typename XT, typename AT>
 __device__ __forceinline__ void spmv_rows_binned(const int* __restrict__ rp, const int* __restrict__ col,
                                                  const MT* __restrict__ val, const XT* __restrict__ x, int m0, int len,
-                                                 const uint16_t* __restrict__ perm, int n0, int n01,
-                                                 AT* __restrict__ out, const int* __restrict__ brp) {
+                                                 const uint16_t* __restrict__ perm, const SortedRows<MT>& so,
+                                                 AT* __restrict__ out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint16_t* pm = perm + m0;
     const int* rpm = rp + m0;
-    const int* brpm = brp ? brp + m0 : nullptr;
-    for (int i0 = warp * 32; i0 < n0; i0 += nwarps * 32) {  // warp-uniform loop over the short rows
-        const int i = i0 + lane;
-        int k = -1, a = 0, rl = 0;
-        if (i < n0) {
-            k = pm[i];
-            const int* rq = brpm ? brpm + i : rpm + k;
-            a = __ldg(rq);
-            rl = __ldg(rq + 1) - a;
-        }
-        const int maxlen = (int)__reduce_max_sync(0xffffffffu, (unsigned)rl);
-        AT sum = AT(0);
-        for (int pk = 0; pk < maxlen; pk += 4) {
-            switch (min(maxlen - pk, 4)) {
-                case 1: row_chunk<1>(col, val, x, a, rl, pk, sum); break;
-                case 2: row_chunk<2>(col, val, x, a, rl, pk, sum); break;
-                case 3: row_chunk<3>(col, val, x, a, rl, pk, sum); break;
-                default: row_chunk<4>(col, val, x, a, rl, pk, sum); break;
+    int done;  // rows of the order that took a thread each
+    if (so.off) {
+        done = so.na;
+        const int ns = (so.na + 31) / 32;
+        for (int t0 = 0, flip = 0; t0 < ns; t0 += nwarps, flip ^= 1) {
+            const int t = t0 + (flip ? nwarps - 1 - warp : warp);
+            if (t >= ns) continue;
+            const int s = ns - 1 - t, i = 32 * s + lane;
+            const int o = __ldg(so.off + s), w = __ldg(so.off + s + 1) - o, rl = so.len[(int64_t)s * 32 + lane];
+            const int k = (i < so.na) ? pm[i] : -1;
+            const int* cp = so.col + (int64_t)o * 32 + lane;
+            const MT* vp = so.val + (int64_t)o * 32 + lane;
+            constexpr int CH = 8;
+            AT sum = AT(0);
+            int pk = 0;
+            for (; pk + CH < w; pk += CH) sorted_chunk<CH>(cp, vp, x, rl, pk, sum);
+            switch (w - pk) {
+                case 1: sorted_chunk<1>(cp, vp, x, rl, pk, sum); break;
+                case 2: sorted_chunk<2>(cp, vp, x, rl, pk, sum); break;
+                case 3: sorted_chunk<3>(cp, vp, x, rl, pk, sum); break;
+                case 4: sorted_chunk<4>(cp, vp, x, rl, pk, sum); break;
+                case 5: sorted_chunk<5>(cp, vp, x, rl, pk, sum); break;
+                case 6: sorted_chunk<6>(cp, vp, x, rl, pk, sum); break;
+                case 7: sorted_chunk<7>(cp, vp, x, rl, pk, sum); break;
+                case 8: sorted_chunk<8>(cp, vp, x, rl, pk, sum); break;
+                default: break;
             }
+            if (k >= 0) out[k] = sum;
         }
-        if (k >= 0) out[k] = sum;
+    } else {
+        done = so.n16;
+        for (int i0 = warp * 32; i0 < so.n16; i0 += nwarps * 32) {  // warp-uniform loop over the short rows
+            const int i = i0 + lane;
+            int k = -1, a = 0, rl = 0;
+            if (i < so.n16) {
+                k = pm[i];
+                a = __ldg(rpm + k);
+                rl = __ldg(rpm + k + 1) - a;
+            }
+            const int maxlen = (int)__reduce_max_sync(0xffffffffu, (unsigned)rl);
+            AT sum = AT(0);
+            for (int pk = 0; pk < maxlen; pk += 4) {
+                switch (min(maxlen - pk, 4)) {
+                    case 1: row_chunk<1>(col, val, x, a, rl, pk, sum); break;
+                    case 2: row_chunk<2>(col, val, x, a, rl, pk, sum); break;
+                    case 3: row_chunk<3>(col, val, x, a, rl, pk, sum); break;
+                    default: row_chunk<4>(col, val, x, a, rl, pk, sum); break;
+                }
+            }
+            if (k >= 0) out[k] = sum;
+        }
     }
-    spmv_sorted_vector<8, 2, 2, MT, XT, AT>(rpm, col, val, x, pm, n0, n01, out, brpm);
-    spmv_sorted_vector<32, 2, 4, MT, XT, AT>(rpm, col, val, x, pm, n01, len, out, brpm);
+    const int mid = max(done, so.n64);
+    spmv_sorted_vector<8, 2, 2, MT, XT, AT>(rpm, col, val, x, pm, done, mid, out);
+    spmv_sorted_vector<32, 2, 4, MT, XT, AT>(rpm, col, val, x, pm, mid, len, out);
 }
 
-// V == 0: length-binned (perm, n0, n01, brp as for spmv_rows_binned); V == 1: one thread per row; else V lanes per
-// row.
+// V == 0: length-binned (perm, so as for spmv_rows_binned); V == 1: one thread per row; else V lanes per row.
 template <int V, int U, typename MT, typename XT, typename AT>
 __device__ __forceinline__ void spmv_rows_to_smem(const int* __restrict__ rp, const int* __restrict__ col,
                                                   const MT* __restrict__ val, const XT* __restrict__ x, int r0,
-                                                  int r1, AT* __restrict__ out, const uint16_t* perm = nullptr,
-                                                  int n0 = 0, int n01 = 0, const int* brp = nullptr) {
-    if constexpr (V == 0) spmv_rows_binned<MT, XT, AT>(rp, col, val, x, r0, r1 - r0, perm, n0, n01, out, brp);
+                                                  int r1, AT* __restrict__ out, const uint16_t* perm,
+                                                  const SortedRows<MT>& so) {
+    if constexpr (V == 0) spmv_rows_binned<MT, XT, AT>(rp, col, val, x, r0, r1 - r0, perm, so, out);
     else if constexpr (V == 1) spmv_rows_scalar<MT, XT, AT>(rp, col, val, x, r0, r1, out);
     else spmv_rows_vector<V, U, MT, XT, AT>(rp, col, val, x, r0, r1, out);
 }

@@ -111,21 +111,26 @@ void launch_pattern_outer(int n, const int* rp, const int* col, const double* u,
     ++g_launches;
 }
 
-// Length class of a row: its length for rows of at most 16 entries, 17 for 17..64 entries, 18 for longer rows.
-__device__ __forceinline__ int length_key(int len) { return len <= 16 ? len : (len <= 64 ? 17 : 18); }
-
-// One CTA (256 threads) per row block: counting sort of the block's rows by length key, stable (rows of equal key
-// keep their order), so the order -- and every sum formed in it -- is deterministic.
+// One CTA (256 threads) per row block: stable counting sort of the block's rows by length (rows beyond kSortedMax entries last,
+// in order), so the order -- and every sum formed in it -- is deterministic; and the class boundaries (cls, see kernels.h).
+// The rows the sorted copy takes, a thread each, end where a slice of 32 rows would be less than half full or so long that
+// its chain of loads (a round per 8 entries, some 1.2 us) outlasts the time the block's entries need on an SM (about
+// a nanosecond each): then a warp per row, or 8 lanes, is the better use.  Blocks of fewer than 2048 rows have too few slices to
+// even out over 16 warps beyond 16 entries (400,000 Zipf rows in blocks of 1344, FP64: 117 us per step with the longer rows in
+// the copy, 107 without; 1M in blocks of 3296: 164 and 177).
 __global__ void __launch_bounds__(256) k_bin_rows(const int* __restrict__ rp, const int* __restrict__ lb_m0,
                                                   const int* __restrict__ lb_len, uint16_t* __restrict__ perm,
                                                   int* __restrict__ cls) {
-    constexpr int NK = 19, NW = 8;
+    constexpr int NK = kSortedMax + 2, NW = 8;
     __shared__ int cnt[NK], cur[NK], wc[NW][NK];
     const int L = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = lb_m0[L], len = lb_len[L];
-    if (tid < NK) cnt[tid] = 0;
+    auto row_len = [&](int k) { return rp[m0 + k + 1] - rp[m0 + k]; };
+    auto key_of = [&](int k) { return min(row_len(k), kSortedMax + 1); };
+    for (int q = tid; q < NK; q += blockDim.x) cnt[q] = 0;
+    for (int q = tid; q < NW * NK; q += blockDim.x) wc[q / NK][q % NK] = 0;
     __syncthreads();
-    for (int k = tid; k < len; k += blockDim.x) atomicAdd(&cnt[length_key(rp[m0 + k + 1] - rp[m0 + k])], 1);
+    for (int k = tid; k < len; k += blockDim.x) atomicAdd(&cnt[key_of(k)], 1);
     __syncthreads();
     if (tid == 0) {
         int run = 0;
@@ -133,18 +138,18 @@ __global__ void __launch_bounds__(256) k_bin_rows(const int* __restrict__ rp, co
             cur[b] = run;
             run += cnt[b];
         }
-        cls[2 * L] = cur[17];
-        cls[2 * L + 1] = cur[18];
+        cls[3 * L] = cur[17];
+        cls[3 * L + 1] = cur[65];
     }
     const unsigned lt = (1u << lane) - 1u;
     for (int base = 0; base < len; base += blockDim.x) {
-        for (int q = tid; q < NW * NK; q += blockDim.x) wc[q / NK][q % NK] = 0;
         __syncthreads();
         const int k = base + tid;
         const bool ok = k < len;
-        const int key = ok ? length_key(rp[m0 + k + 1] - rp[m0 + k]) : -1;
+        const int key = ok ? key_of(k) : -1;
         const unsigned peers = __match_any_sync(0xffffffffu, key);
-        if (ok && lane == __ffs(peers) - 1) wc[warp][key] = __popc(peers);
+        const bool lead = ok && lane == __ffs(peers) - 1;
+        if (lead) wc[warp][key] = __popc(peers);
         __syncthreads();
         if (ok) {
             int pos = cur[key] + __popc(peers & lt);
@@ -152,12 +157,22 @@ __global__ void __launch_bounds__(256) k_bin_rows(const int* __restrict__ rp, co
             perm[m0 + pos] = (uint16_t)k;
         }
         __syncthreads();
-        if (tid < NK) {
-            int tot = 0;
-            for (int w = 0; w < NW; ++w) tot += wc[w][tid];
-            cur[tid] += tot;
+        if (lead) {  // one lane per warp and key
+            atomicAdd(&cur[key], __popc(peers));
+            wc[warp][key] = 0;
         }
-        __syncthreads();
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int most = len < 2048 ? 16 : max(16, (rp[m0 + len] - rp[m0]) / 256);
+        int q = (len + 31) / 32 - 1;
+        for (; q >= 0; --q) {
+            const int i = 32 * q + lane;
+            const unsigned l = i < len ? (unsigned)row_len(perm[m0 + i]) : 0u;
+            const int sum = (int)__reduce_add_sync(0xffffffffu, l), w = (int)__reduce_max_sync(0xffffffffu, l);
+            if (w <= 16 || (w <= kSortedMax && w <= most && 32 * w <= 2 * sum)) break;
+        }
+        if (lane == 0) cls[3 * L + 2] = min(len, 32 * (q + 1));
     }
 }
 
@@ -167,51 +182,71 @@ void launch_bin_rows(int nl, const int* rp, const int* lb_m0, const int* lb_len,
     ++g_launches;
 }
 
-// ---- the length-binned SpMV's copy of a matrix: each row block's rows stored in their processing order ----
-// Row i of block L's length order (local row perm[m0 + i]) is stored at brp[m0 + i] .. brp[m0 + i + 1] of bcol/bval,
-// so the rows a warp processes together are neighbours in memory and every sector it loads is used while it is in L1
-// (in CSR order the short rows of a warp lie among rows processed at other times, which share their sectors).
+// ---- the length-binned SpMV's sorted copy (SELL-32 over each row block's length order) ----
+// Slice base[L] + q holds rows 32q .. 32q+31 of block L's order (local rows perm[m0 + 32q + lane]), those below the block's
+// boundary cls[3L + 2]; it is as wide as its longest row and stored like the SELL-32 copy below.
 
-__global__ void k_bcopy_len(const int* __restrict__ rp, const int* __restrict__ lb_m0, const int* __restrict__ lb_len,
-                            const uint16_t* __restrict__ perm, int* __restrict__ lens) {
-    const int L = blockIdx.x;
-    const int m0 = lb_m0[L], len = lb_len[L];
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-        const int k = m0 + perm[m0 + i];
-        lens[m0 + i] = rp[k + 1] - rp[k];
+// One CTA per row block: row lengths and slice widths (0 beyond the boundary).
+__global__ void k_sorted_len(const int* __restrict__ rp, const int* __restrict__ lb_m0, const int* __restrict__ lb_len,
+                             const uint16_t* __restrict__ perm, const int* __restrict__ cls,
+                             const int* __restrict__ base, uint16_t* __restrict__ len, int* __restrict__ wid) {
+    const int L = blockIdx.x, m0 = lb_m0[L], nr = lb_len[L], na = cls[3 * L + 2];
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; 32 * q < nr; q += blockDim.x >> 5) {
+        const int i = 32 * q + lane;
+        int l = 0;
+        if (i < na) {
+            const int k = m0 + perm[m0 + i];
+            l = rp[k + 1] - rp[k];
+        }
+        const int64_t s = base[L] + q;
+        len[s * 32 + lane] = (uint16_t)l;
+        const int w = (int)__reduce_max_sync(0xffffffffu, (unsigned)l);
+        if (lane == 0) wid[s] = w;
     }
 }
 
-// One warp per row: the row's entries copied in order (columns only when bcol is not null).
-__global__ void k_bcopy_fill(const int* __restrict__ rp, const int* __restrict__ col, const double* __restrict__ val,
-                             const int* __restrict__ lb_m0, const int* __restrict__ lb_len,
-                             const uint16_t* __restrict__ perm, const int* __restrict__ brp, int* __restrict__ bcol,
-                             double* __restrict__ bval) {
-    const int L = blockIdx.x;
-    const int m0 = lb_m0[L], len = lb_len[L];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < len; i += nw) {
-        const int k = m0 + perm[m0 + i];
-        const int a = rp[k], e = rp[k + 1], d = brp[m0 + i];
-        for (int p = a + lane; p < e; p += 32) {
-            if (bcol) bcol[d + (p - a)] = col[p];
-            bval[d + (p - a)] = val[p];
+// Columns (when scol is not null) and values in slice order, one warp per slice.
+template <typename MT>
+__global__ void k_sorted_fill(const int* __restrict__ rp, const int* __restrict__ col, const double* __restrict__ val,
+                              const int* __restrict__ lb_m0, const int* __restrict__ lb_len,
+                              const uint16_t* __restrict__ perm, const int* __restrict__ cls,
+                              const int* __restrict__ base, const int* __restrict__ off, int* __restrict__ scol,
+                              MT* __restrict__ sval) {
+    const int L = blockIdx.x, m0 = lb_m0[L], na = cls[3 * L + 2];
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; 32 * q < na; q += blockDim.x >> 5) {
+        const int i = 32 * q + lane;
+        int a = 0, l = 0;
+        if (i < na) {
+            const int k = m0 + perm[m0 + i];
+            a = rp[k];
+            l = rp[k + 1] - a;
+        }
+        const int o = off[base[L] + q], w = off[base[L] + q + 1] - o;
+        const int64_t at = (int64_t)o * 32 + lane;
+#pragma unroll 4
+        for (int e = 0; e < w; ++e) {
+            if (scol) scol[at + (int64_t)e * 32] = (e < l) ? col[a + e] : 0;
+            sval[at + (int64_t)e * 32] = (e < l) ? (MT)val[a + e] : MT(0);
         }
     }
 }
 
-void launch_bcopy_build(int n, int nl, const int* rp, const int* lb_m0, const int* lb_len, const uint16_t* perm,
-                        int* lens, int* brp, cudaStream_t st) {
-    k_bcopy_len<<<nl, 256, 0, st>>>(rp, lb_m0, lb_len, perm, lens);
-    k_scan_plain<<<1, 1024, 0, st>>>(lens, brp, n);
+void launch_sorted_build(int nl, int ns, const int* rp, const int* lb_m0, const int* lb_len, const uint16_t* perm,
+                         const int* cls, const int* base, uint16_t* len, int* wid, int* off, cudaStream_t st) {
+    k_sorted_len<<<nl, 512, 0, st>>>(rp, lb_m0, lb_len, perm, cls, base, len, wid);
+    k_scan_plain<<<1, 1024, 0, st>>>(wid, off, ns);
     g_launches += 2;
 }
 
-void launch_bcopy_fill(int nl, const int* rp, const int* col, const double* val, const int* lb_m0,
-                       const int* lb_len, const uint16_t* perm, const int* brp, int* bcol, double* bval,
-                       cudaStream_t st) {
-    k_bcopy_fill<<<nl, 256, 0, st>>>(rp, col, val, lb_m0, lb_len, perm, brp, bcol, bval);
-    ++g_launches;
+void launch_sorted_fill(int nl, const int* rp, const int* col, const double* val, const int* lb_m0, const int* lb_len,
+                        const uint16_t* perm, const int* cls, const int* base, const int* off, int* scol, double* sval,
+                        float* sval32, cudaStream_t st) {
+    if (sval) k_sorted_fill<double><<<nl, 512, 0, st>>>(rp, col, val, lb_m0, lb_len, perm, cls, base, off, scol, sval);
+    if (sval32)
+        k_sorted_fill<float><<<nl, 512, 0, st>>>(rp, col, val, lb_m0, lb_len, perm, cls, base, off, nullptr, sval32);
+    g_launches += (sval ? 1 : 0) + (sval32 ? 1 : 0);
 }
 
 // ---- SELL-32 copy of a matrix with short rows ----

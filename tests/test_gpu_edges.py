@@ -172,3 +172,35 @@ def test_staged_fp64_spmv(Solver, n, maxlen, block_rows):
         np.subtract.at(r, rows, val * got.cpu().numpy()[col])
         assert info["status"] == 0 and abs(info["rel_res_true"] - np.linalg.norm(r) / np.linalg.norm(y)) <= 1e-14
     sv.close()
+
+
+# the length-binned SpMV before and after the sorted copy exists: empty rows, rows beyond the copy's longest, blocks whose long
+# rows the copy leaves out, slices cut by a block's end, new values, FP64 and FP32 cycles on one handle, the transpose
+@pytest.mark.parametrize("n,lens,block_rows", [(70, (0, 70), 32), (3000, (0, 3, 17, 64, 65, 513, 700), 512), (3000, (17,), 1024),
+                                               (9001, (1, 4, 4, 4, 5, 30, 200), 0), (20_000, (4, 4, 4, 40, 256), 8192)])
+def test_length_binned_spmv_classes(Solver, n, lens, block_rows):
+    rng = np.random.default_rng(n + len(lens))
+    length = rng.choice(np.asarray(lens), n)
+    rp = np.concatenate([[0], np.cumsum(length + 1)]).astype(np.int64)
+    rows = np.repeat(np.arange(n), length + 1)
+    col = rng.integers(0, n, rp[-1]).astype(np.int32)
+    col[rp[:-1]] = np.arange(n)
+    x = rng.standard_normal(n)
+    sv = None
+    for scale in (1.0, 3.0):
+        val = scale * rng.standard_normal(rp[-1])
+        val[rp[:-1]] = scale * 2.0 * (np.bincount(rows, np.abs(val), n) + np.bincount(col, np.abs(val), n))
+        if sv is None:
+            sv = Solver(n, rp, col, val, sketch_seed=1, block_rows=block_rows)
+        else:
+            sv.update_values(dev_vec(val))
+        y, size = np.bincount(rows, val * x[col], n), np.bincount(rows, np.abs(val * x[col]), n)
+        for precision in ("fp64", "fp32"):
+            sv.set("precision", precision)
+            for transpose in (False, True):
+                b = np.bincount(col, val * x[rows], n) if transpose else y
+                got, info = sv.solve(dev_vec(b), m=12, s=48, k=2, tol=1e-12, transpose=transpose)
+                assert info["status"] == 0 and np.linalg.norm(got.cpu().numpy() - x) <= 1e-10 * np.linalg.norm(x)
+            err = np.abs(sv.spmv(dev_vec(x)).cpu().numpy() - y)
+            assert np.all(err <= (length + 8) * 2.0 ** -53 * 2 * size)
+    sv.close()

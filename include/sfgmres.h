@@ -71,10 +71,10 @@ extern "C" {
                                         returns the shape in use: 1, 2..32, or 0 for the length-binned SpMV. */
 #define SFGMRES_OPT_BLOCK_ROWS 9     /* rows per row block of the fused inner kernels: a multiple of 32 in
                                         [32, 8192], or 0 (default) = chosen by the library (one system: two blocks
-                                        per SM, less 8 SMs with FP64 inner cycles, which are left to the sketched-QR
-                                        update running beside the fused kernel, or at most 128 blocks for small
-                                        systems; many right-hand sides of one system: 5120; several systems: 4096).
-                                        Reading it returns the size in use. */
+                                        per SM, of all SMs but 8 for medium systems, or at most 128 blocks for small
+                                        ones, which leaves SMs to the sketched-QR update running beside; many
+                                        right-hand sides of one system: 5120; several systems: 4096).  Reading it
+                                        returns the size in use. */
 #define SFGMRES_OPT_GRAPH 10         /* 1 (default): each outer step (one inner cycle for every problem and the outer
                                         FGMRES update) is captured once into a CUDA graph and replayed; the graphs
                                         are kept while the solve's parameters and workspaces stay the same.  0: the

@@ -260,22 +260,21 @@ int choose_vec(int64_t, int, int maxlen) { return maxlen <= 16 ? 1 : 0; }
 // Row blocks of one system, a multiple of 32 rows, at most kBlockRowsMax.
 //
 // Large systems get two blocks per SM, the CTAs of the inner kernels that an SM holds (with one its 16 warps hide too little
-// latency: 72 to 50 us per step at 101^3 FP64, 47 to 35 us FP32).  A stencil's FP64 step leaves 8 SMs without a block: the
-// sketched QR of step i runs beside the inner kernel of step i+1, and a one-wave FP64 kernel whose CTAs share SMs with it
-// waits for those stragglers (128^3: 86 us per step with 288 blocks, 100 us with 304).  The FP32 and BF16 kernels are
-// short enough, and the length-binned SpMV latency bound enough (1M Zipf rows, FP64: 260 us with 304 blocks, 282 with
-// 287), that all SMs serve them best.
-//
-// Small systems take at most 128 blocks, one per SM, so that the QR's cluster finds SMs of its own: with more, both the
-// step and the QR get slower (32^3: 17.9 us per step FP64 against 25 with 256 blocks; 64^3 FP32: 20.4 against 24).  The
-// line, in stored entries, lies where the two met: FP64 48^3 (0.8M entries) 21.9 us with 128 blocks and 24.2 with 288, 64^3
-// (1.8M) 32.6 and 27.7; FP32 72^3 (2.6M) 21.7 and 24.7, 80^3 (3.6M) 26.4 and 25.4; Zipf rows 30,000 (0.8M) 27 and 30
-// (FP64), 18 and 21 (FP32), 100,000 (2.5M) 50 and 41, 38 and 30.
+// latency: 72 to 50 us per step at 101^3 FP64, 47 to 35 us FP32).  Small ones take at most 128 blocks, one per SM, so that the
+// sketched QR's cluster, which runs beside the next step, finds SMs of its own: with more, both the step and the QR get
+// slower (32^3 FP64, m = 34: 3.0 ms per solve, with 288 blocks 3.8).  Between the two, 8 SMs' worth of blocks less than all
+// leave the QR some room.  The lines, in stored entries, lie where the forms met (ms per solve, 128 / 288 / 304 blocks):
+//   FP64 48^3 (0.8M entries) 5.1 / 5.9 / 5.9 (m = 80), 56^3 (1.2M) 6.6 / 6.0 / 5.9 (m = 34), 64^3 (1.8M) 8.9 / 7.4 / 8.2, 84^3 (4.1M) 17.9 /
+//   12.6 / 11.8, 128^3 (14.6M) - / 45.7 / 44.8;
+//   FP32 64^3 8.0 / 8.0 / 8.5, 72^3 (2.6M) 10.5 / 9.3 / 10.2, 84^3 15.8 / 12.3 / 12.2;
+//   length-binned, us per step: 30,000 Zipf rows (0.8M) 27 / 30 / 30 (FP64), 18 / 21 / 21 (FP32), 100,000 (2.5M) 50 / 41 / 41, 38 / 30 / 30, 1M
+//   (25M, FP64) - / 282 / 260.
 int single_block_rows(int n, int64_t nnz, int sms, int prec, bool binned) {
-    const int64_t line = (prec == 0 || binned) ? 1200000 : 3200000;
+    const int64_t two = (prec == 0 || binned) ? 1200000 : 2100000;   // from here on two blocks per SM
+    const int64_t all = binned ? two : (prec == 0 ? 2400000 : 3500000);  // from here on on every SM
     int blocks;
-    if (nnz < line) blocks = std::max(sms - 24, std::min(sms, 16));
-    else blocks = 2 * ((prec == 0 && !binned && sms > 2 * kQrSms) ? sms - kQrSms : sms);
+    if (nnz < two) blocks = std::max(sms - 24, std::min(sms, 16));
+    else blocks = 2 * ((nnz < all && sms > 2 * kQrSms) ? sms - kQrSms : sms);
     const int64_t most = ((int64_t)n + kBlockRowsMax - 1) / kBlockRowsMax;  // fewest blocks of the largest size
     while (blocks < most) blocks *= 2;
     const int64_t per = ((int64_t)n + blocks - 1) / blocks;

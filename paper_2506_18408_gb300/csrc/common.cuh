@@ -14,7 +14,7 @@ constexpr int kMaxS = 4096;     // largest sketch size
 constexpr int kMaxM = 1024;     // largest inner basis size
 constexpr int kBlockRowsMax = 8192;  // rows per row block (local sketch offsets need <= 15 bits)
 constexpr int kQrCluster = 16;       // most CTAs of the cluster that runs a sketched QR update
-constexpr int kQrSms = 8;            // SMs the FP64 row-block rule leaves to the sketched QR
+constexpr int kQrSms = 8;            // SMs that the row-block rule for medium systems leaves to the sketched QR
 
 // ------------------------------------------------------------------------------------------------------------
 // Precision traits.  VT: storage type of inner basis vectors; AT: arithmetic / accumulation type; MT: matrix values.

@@ -964,7 +964,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
     const size_t stage = staged ? stage_smem(maxlen) : 0;
     const bool beside = vec == 0 || t > 4 || !h->fuse_step;  // binned, or steps of two launches (launch_inner_step)
-    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), beside);
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), vec == 0);
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;

@@ -528,10 +528,10 @@ static size_t qr_smem(const QrShape& q, int m, int i) {
 // / 4.06 / 3.90 ms; s = 1000, m = 200 (80^3) 44.3 / 28.9 / 20.9 / 15.9 ms; beside the length-binned SpMV, s = 120, m = 30
 // (30,000 Zipf rows) 19.6 / 20.8 / 20.8 / 20.9 ms.  Batches take what leaves the problems' clusters
 // side by side on the GPU.
-QrShape qr_shape(int P, int s, int m, size_t smem_left, bool beside) {
+QrShape qr_shape(int P, int s, int m, size_t smem_left, bool binned) {
     QrShape q;
     const int most = P <= 4 ? kQrCluster : P <= 16 ? 8 : P <= 32 ? 4 : P <= 64 ? 2 : 1;
-    q.cluster = std::min(most, s * m <= (beside ? 5000 : 3000) ? 2 : s * m <= 20000 ? 4 : kQrCluster);
+    q.cluster = std::min(most, s * m <= (binned ? 5000 : 3000) ? 2 : s * m <= 20000 ? 4 : kQrCluster);
     q.nrp = ((s + q.cluster - 1) / q.cluster) | 1;
     q.slice = (q.nrp * m + 1) & ~1;
     q.staged = true;

@@ -250,9 +250,9 @@ void inner_axpy_f64(const Plan& p, int i, bool last);
 void inner_axpy_f32(const Plan& p, int i, bool last);
 void inner_axpy_bf16(const Plan& p, int i, bool last);
 void launch_inner_axpy(const Plan& p, int i, bool last);
-// For P problems, sketch size s and basis size m, given the shared memory a QR CTA may take; beside: the step is not one launch of a
-// stencil, and the QR runs on the SMs of its CTAs.
-QrShape qr_shape(int P, int s, int m, size_t smem_left, bool beside);
+// For P problems, sketch size s and basis size m, given the shared memory a QR CTA may take; binned: the step's SpMV is the length-
+// binned one.  The cluster, on which the rounding of the sums depends, is the same for steps of one and of two launches.
+QrShape qr_shape(int P, int s, int m, size_t smem_left, bool binned);
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st
 void launch_inner_finish(const Plan& p, double* z);  // y = R^{-1} d, z = sum_l y_l b_l (FP64)
 void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r] = sigma_l * u_l[r] (FP64)

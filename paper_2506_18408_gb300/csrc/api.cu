@@ -44,6 +44,7 @@ struct Geo {
     DevBuf tab;  // int: blk_v0, blk_len, blk_cs, blk_list, blk_prob [nblk each], prob_b0 [P+1], pflag [P]
     uint64_t used = 0;
     int maxbp = 0;           // largest number of blocks of one problem
+    bool flagged = false;    // pflag may hold set flags
 };
 
 constexpr int kGeoCache = 4;
@@ -568,6 +569,7 @@ int get_geometry(sfgmres_ctx* h, int nrhs, Geo** out) {
         CK(cudaMemcpyAsync(g->tab.p, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, h->st));
         CK(cudaStreamSynchronize(h->st));
         g->nrhs = nrhs;
+        g->flagged = false;  // the table came with clear flags
         g->ver = h->geo_ver;
         g->maxbp = 0;
         for (int p = 0; p < P; ++p) g->maxbp = std::max(g->maxbp, pb0[p + 1] - pb0[p]);
@@ -1003,7 +1005,9 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure_host(h, h->h_cyc, Pn * sizeof(CycleState)))) return rc;
     if ((rc = ensure_host(h, h->h_pflag, Pn * sizeof(int)))) return rc;
     std::memset(h->h_pflag.p, 0, Pn * sizeof(int));
-    CK(cudaMemsetAsync(pflag_of(g), 0, Pn * sizeof(int), h->st));
+    const bool solve = jmax > 0;
+    if (g->flagged) CK(cudaMemsetAsync(pflag_of(g), 0, Pn * sizeof(int), h->st));
+    g->flagged = solve;  // a solve marks its problems as they finish
 
     Plan& P = *p;
     plan_geometry(h, g, transpose, P);

@@ -260,17 +260,29 @@ __global__ void __launch_bounds__(512) k_sketch_partials(const Plan P, const dou
     const int s = P.s, Bn = P.Bn;
     const double sc = xscale ? xscale[(int64_t)bi.prob * xstride] : 1.0;
     int emax = 1;
-    for (int r = threadIdx.x; r <= Bn; r += blockDim.x) {
-        AT v = AT(0);
-        if (r < bi.len) {
-            v = (AT)(sc * x[bi.v0 + r]);
-            if (dst) {
-                store_as(dst + bi.v0 + r, v);
-                v = stored_value(v, dst);
-            }
+    constexpr int UL = 8;  // loads of x in flight per thread (one at a time, a block's 58 KB took some 14 round trips)
+    for (int r0 = threadIdx.x; r0 <= Bn; r0 += UL * blockDim.x) {
+        double xv[UL];
+#pragma unroll
+        for (int u = 0; u < UL; ++u) {
+            const int r = r0 + u * (int)blockDim.x;
+            xv[u] = (r < bi.len) ? x[bi.v0 + r] : 0.0;
         }
-        xb[r] = v;
-        emax = max(emax, exp_of(v));
+#pragma unroll
+        for (int u = 0; u < UL; ++u) {
+            const int r = r0 + u * (int)blockDim.x;
+            if (r > Bn) break;
+            AT v = AT(0);
+            if (r < bi.len) {
+                v = (AT)(sc * xv[u]);
+                if (dst) {
+                    store_as(dst + bi.v0 + r, v);
+                    v = stored_value(v, dst);
+                }
+            }
+            xb[r] = v;
+            emax = max(emax, exp_of(v));
+        }
     }
     const int ng = (s + 31) / 32;
     const int* sg = P.seg + (int64_t)bi.list * ng;  // the block's group starts (units)

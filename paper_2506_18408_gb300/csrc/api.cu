@@ -1018,6 +1018,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     P.ent = h->ent;
     P.sk_scale = (h->kind == 1) ? 1.0 : 1.0 / std::sqrt((double)h->sk_zeta);
     P.sk_headroom = h->sk_headroom;
+    P.sk_pieces = sketch_pieces(s);
     P.prec = h->prec;
     P.m = m;
     P.t = t;

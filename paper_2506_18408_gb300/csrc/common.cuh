@@ -284,35 +284,44 @@ __device__ __forceinline__ void bar_sync_named(int id, int threads) {
 }
 
 // Sums of every gather list of a block by nwk warps (w: this warp's index among them), a warp per group of 32 sketch rows;
-// emit(r, sum) is called for every row r < s.  Where the warps are at least twice the groups, a group's lists are cut into
-// J = nwk / ng pieces, one warp each, whose sums meet in `buf` (512 slots) and are added in list order: a list of some
-// 200 entries is a chain of loads, and with s = 160 only 5 of 16 warps had one.  The nwk warps meet on named barrier 2.
-// The 2D batch of 24 systems x 4 (s = 160, FP32 cycles): inner SpMV and sketch 47.3 -> 44.7 us per launch, sketch of a cycle's
-// start 28 -> 23 us.
+// emit(r, sum) is called for every row r < s.  A list is a chain of loads of some 150 entries, and few sketch rows leave
+// warps without one (s = 160: 5 of 16), so each group's lists are cut into K pieces (sketch_pieces), taken by the warps in
+// turn, whose sums meet in `buf` (512 slots) and are added in list order.  K depends on s alone, so the steps of one
+// and of two launches, which have different numbers of warps for the sketch, form the same sums.  The nwk warps meet on named
+// barrier 2.  The 2D batch of 24 systems x 4 (s = 160, FP32 cycles): inner SpMV and sketch 47.3 -> 44.7 us per launch, sketch
+// of a cycle's start 28 -> 23 us.
 template <typename T, typename Emit>
-__device__ __forceinline__ void sketch_sums(const uint16_t* __restrict__ ent, const int* __restrict__ sg, int s, int w,
-                                            int nwk, const T* __restrict__ x, T* __restrict__ buf, Emit&& emit) {
+__device__ __forceinline__ void sketch_sums(const uint16_t* __restrict__ ent, const int* __restrict__ sg, int s, int K,
+                                            int w, int nwk, const T* __restrict__ x, T* __restrict__ buf, Emit&& emit) {
     const int lane = threadIdx.x & 31, ng = (s + 31) / 32;
-    const int J = nwk / ng;
-    if (J < 2) {
+    if (K == 1) {
         for (int g = w; g < ng; g += nwk) {
             const int r = 32 * g + lane;
             if (r < s) emit(r, sum_group(ent, sg[g], (sg[g + 1] - sg[g]) >> 5, lane, x));
         }
         return;
     }
-    const int g = w % ng, j = w / ng, r = 32 * g + lane;
-    T v = T(0);
-    if (j < J) {
-        const int E = (sg[g + 1] - sg[g]) >> 5, ub = E * j / J, ue = E * (j + 1) / J;
-        v = sum_group(ent, sg[g] + 32 * ub, ue - ub, lane, x);
-        if (j > 0) buf[(j - 1) * 32 * ng + r] = v;
+    T first = T(0);  // the sum of piece 0 of group w (K > 1 only with ng <= nwk)
+    for (int t = w; t < ng * K; t += nwk) {
+        const int g = t % ng, j = t / ng;
+        const int E = (sg[g + 1] - sg[g]) >> 5, ub = E * j / K, ue = E * (j + 1) / K;
+        const T v = sum_group(ent, sg[g] + 32 * ub, ue - ub, lane, x);
+        if (j == 0) first = v;
+        else buf[(j - 1) * 32 * ng + 32 * g + lane] = v;
     }
     bar_sync_named(2, nwk * 32);
-    if (j == 0 && r < s) {
-        for (int q = 1; q < J; ++q) v += buf[(q - 1) * 32 * ng + r];
-        emit(r, v);
+    const int r = 32 * w + lane;
+    if (w < ng && r < s) {
+        for (int q = 1; q < K; ++q) first += buf[(q - 1) * 32 * ng + r];
+        emit(r, first);
     }
+}
+
+// Pieces per group for s sketch rows: what gives the 16 warps of the two-launch step one each.  (More pieces, to even out the
+// 13 warps of the one-launch step too, measured no faster: 96^3 ILU(0) solve 19.4 -> 19.5 ms, 2D batch 110.1 -> 112.9 ms.)
+inline int sketch_pieces(int s) {
+    const int ng = (s + 31) / 32;
+    return ng <= 8 ? 16 / ng : 1;
 }
 
 // ------------------------------------------------------------------------------------------------------------

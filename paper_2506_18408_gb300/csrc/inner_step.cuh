@@ -332,10 +332,10 @@ __device__ __forceinline__ void sketch_rows(const Plan& P, int b, int list, cons
     if constexpr (sizeof(AT) == 8) {
         const double unit = fixed_unit(0.0, Eb, P.sk_headroom);
         const bool bad = exp_nonfinite(0.0, Eb);
-        sketch_sums(P.ent, sg, s, w, nwk, reinterpret_cast<const long long*>(wblk), reinterpret_cast<long long*>(buf),
+        sketch_sums(P.ent, sg, s, P.sk_pieces, w, nwk, reinterpret_cast<const long long*>(wblk), reinterpret_cast<long long*>(buf),
                     [&](int r, long long v) { cp[r] = bad ? (AT)NAN : (AT)((double)v * unit); });
     } else {
-        sketch_sums(P.ent, sg, s, w, nwk, wblk, buf, [&](int r, AT v) { cp[r] = v; });
+        sketch_sums(P.ent, sg, s, P.sk_pieces, w, nwk, wblk, buf, [&](int r, AT v) { cp[r] = v; });
     }
 }
 

@@ -103,6 +103,7 @@ struct Plan {
     int s = 0, zeta = 0, kind = 0;
     const int* seg = nullptr;
     const uint16_t* ent = nullptr;
+    int sk_pieces = 1;  // pieces per group of gather lists (sketch_pieces)
     double sk_scale = 1.0;
     int sk_headroom = 0;  // extra right shift of the FP64 fixed-point sketch terms (long gather lists)
 

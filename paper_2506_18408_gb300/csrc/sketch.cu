@@ -298,12 +298,12 @@ __global__ void __launch_bounds__(512) k_sketch_partials(const Plan P, const dou
         const double unit = fixed_unit(0.0, Eb, P.sk_headroom);
         const bool bad = exp_nonfinite(0.0, Eb);
         double* pb = (double*)part + (int64_t)b * s;
-        sketch_sums(P.ent, sg, s, threadIdx.x >> 5, blockDim.x >> 5, (const long long*)qb, (long long*)buf,
+        sketch_sums(P.ent, sg, s, P.sk_pieces, threadIdx.x >> 5, blockDim.x >> 5, (const long long*)qb, (long long*)buf,
                     [&](int r, long long v) { pb[r] = bad ? (double)NAN : (double)v * unit; });
     } else {
         __syncthreads();
         AT* pb = part + (int64_t)b * s;
-        sketch_sums(P.ent, sg, s, threadIdx.x >> 5, blockDim.x >> 5, (const AT*)xb, buf, [&](int r, AT v) { pb[r] = v; });
+        sketch_sums(P.ent, sg, s, P.sk_pieces, threadIdx.x >> 5, blockDim.x >> 5, (const AT*)xb, buf, [&](int r, AT v) { pb[r] = v; });
     }
 }
 

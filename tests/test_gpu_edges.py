@@ -204,3 +204,19 @@ def test_length_binned_spmv_classes(Solver, n, lens, block_rows):
             err = np.abs(sv.spmv(dev_vec(x)).cpu().numpy() - y)
             assert np.all(err <= (length + 8) * 2.0 ** -53 * 2 * size)
     sv.close()
+
+
+# the sketch sums' pieces: the step of one launch (11 to 14 warps sum lists) and of two (16 warps) form the same sums, bit for
+# bit, also in FP32, for one group of sketch rows up to more groups than warps
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("s,t", [(24, 0), (70, 1), (130, 2), (160, 2), (224, 3), (256, 4), (352, 4), (400, 2), (520, 2)])
+def test_sketch_pieces_do_not_depend_on_the_launches(Solver, precision, s, t):
+    A = workloads.convdiff(150, (30.0, 10.0))
+    v = _unit(A.n, s)
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, precision=precision)
+    got = []
+    for fused in (1, 0):
+        sv.set("fused_step", fused)
+        got.append(sv.inner_cycle(v, m=8, s=s, k=t)[0].cpu().numpy())
+    assert np.array_equal(*got)
+    sv.close()

@@ -92,8 +92,9 @@ __device__ __forceinline__ void stage_issue(const int* __restrict__ col, const M
                                             unsigned cdst, unsigned vdst, int lane) {
     constexpr int VP = 16 / (int)sizeof(MT);
     const int ca = a0 & ~3, va = a0 & ~(VP - 1);
-    for (int u = lane; ca + 4 * u < a1; u += 32) cp_async16(cdst + 16 * u, col + ca + 4 * u);
-    for (int u = lane; va + VP * u < a1; u += 32) cp_async16(vdst + 16 * u, val + va + VP * u);
+    // unsigned: a lane's offset may pass 2^31 - 1 entries before it ends the loop
+    for (unsigned u = lane; ca + 4 * u < (unsigned)a1; u += 32) cp_async16(cdst + 16 * u, col + ca + 4 * u);
+    for (unsigned u = lane; va + VP * u < (unsigned)a1; u += 32) cp_async16(vdst + 16 * u, val + va + VP * u);
 }
 
 // Entries pk .. pk+CNT-1 of the lane's row (its first entry at cs, vs in shared memory), get(c) the factor of column c;

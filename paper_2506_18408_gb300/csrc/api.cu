@@ -915,7 +915,8 @@ int ensure_ilu(sfgmres_ctx* h) {
         int bad = 0;
         CK(cudaMemcpyAsync(&bad, h->ilu_bad.p, sizeof(int), cudaMemcpyDeviceToHost, h->st));
         CK(cudaStreamSynchronize(h->st));
-        if (bad) return fail(h, SFGMRES_ERR_INVALID_ARG, "ILU(0) met a zero pivot");
+        if (bad & 1) return fail(h, SFGMRES_ERR_INVALID_ARG, "ILU(0) met a zero pivot");
+        h->ilu.divide = bad != 0;
         h->ilu_vals_ver = h->vals_ver;
     }
     return 0;
@@ -1194,7 +1195,8 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
     for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.staged, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
                       (int64_t)P.s, (int64_t)P.zeta, (int64_t)P.kind, (int64_t)P.sk_headroom, (int64_t)P.prec,
                       (int64_t)P.m, (int64_t)P.t, (int64_t)P.qr.cluster, (int64_t)P.qr.staged, (int64_t)P.jmax, (int64_t)h->c3,
-                      (int64_t)h->profile, (int64_t)P.gwait_extra, (int64_t)P.outer_variant})
+                      (int64_t)h->profile, (int64_t)P.gwait_extra, (int64_t)P.outer_variant,
+                      (int64_t)(P.ilu_host && P.ilu_host->divide)})
         k.push_back((uint64_t)v);
     uint64_t bits;
     std::memcpy(&bits, &P.sk_scale, 8);

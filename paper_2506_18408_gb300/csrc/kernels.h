@@ -37,6 +37,7 @@ struct IluDev {
 // Host side of the preconditioner: the colour ranges the launchers loop over.
 struct IluHost {
     int n = 0, ncol = 0, maxlen = 0;
+    bool divide = false;       // a pivot's reciprocal overflows: the passes divide
     int64_t nnz = 0;
     std::vector<int> starts;   // [ncol + 1] first permuted row of each colour
     double2* piv = nullptr;    // device [n]: dev.piv, written by the factorisation

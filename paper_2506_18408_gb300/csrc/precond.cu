@@ -35,7 +35,7 @@ __global__ void k_ilu_gather(int64_t nnz, const int* __restrict__ src, const dou
 
 // ILU(0) of the rows [r0, r1) of one colour, one thread per row: for each entry (r, k) with k < r (earlier colours,
 // already final), l_rk = a_rk / u_kk, then a_rj -= l_rk u_kj for the entries j > k that row r and row k both hold
-// (a merge of the two sorted rows).  A zero pivot sets *bad.
+// (a merge of the two sorted rows).  A zero pivot sets bit 0 of *bad.
 __global__ void k_ilu0_colour(int r0, int r1, const int* __restrict__ rp, const int* __restrict__ col,
                               const int* __restrict__ diag, double* __restrict__ lu, int* __restrict__ bad) {
     const int r = r0 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
@@ -76,13 +76,15 @@ __device__ __forceinline__ bool ilu_idle(const Plan& P, int i) {
     return c->stopped || c->brk_step <= i || (P.pflag[0] & 1);
 }
 
-// piv[r] = (u_rr, 1 / u_rr).
+// piv[r] = (u_rr, 1 / u_rr); a pivot whose reciprocal overflows sets bit 1 of *bad.
 __global__ void k_ilu_pivots(int n, const int* __restrict__ diag, const double* __restrict__ lu,
-                             double2* __restrict__ piv) {
+                             double2* __restrict__ piv, int* __restrict__ bad) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const double d = lu[diag[r]];
-    piv[r] = make_double2(d, 1.0 / d);
+    const double inv = 1.0 / d;
+    piv[r] = make_double2(d, inv);
+    if (isinf(inv)) atomicOr(bad, 2);
 }
 
 // ocol[p] = the original index of entry p's column, with kLaterColour set where that column is not of the first colour.
@@ -111,7 +113,9 @@ struct TriangleRows {
 
 // One pass over the rows [r0, r1) of a colour, the CTA's part of `chunk` rows.  Forward: y = u - sum of l y, and with `final`
 // (the last colour) z = y / u_rr into out, else y.  Backward: z = (y - sum of u z) / u_rr into out, with `first` y = u.
-template <bool FWD, bool STAGED>
+// DIV: some pivot's reciprocal overflows, so the pass divides.  Chosen per factorisation: a division for such rows alone costs
+// all others its branch (a 1M-row solve 19.7 -> 22.2 ms, with the operands scaled instead 20.4 ms).
+template <bool FWD, bool STAGED, bool DIV>
 __global__ void __launch_bounds__(512, 2) k_ilu_pass(const Plan P, int i, int r0, int r1, int chunk, bool edge,
                                                      int maxlen, const double* __restrict__ u, double* y, double* out) {
     if (ilu_idle(P, i)) return;
@@ -142,7 +146,7 @@ __global__ void __launch_bounds__(512, 2) k_ilu_pass(const Plan P, int i, int r0
             y[at] = v;
         } else {
             const double t = v * pv.y;
-            out[at] = fma(fma(-t, pv.x, v), pv.y, t);
+            out[at] = DIV ? v / pv.x : fma(fma(-t, pv.x, v), pv.y, t);
         }
     };
     const TriangleRows<FWD> part{diag, len};
@@ -168,7 +172,7 @@ cudaError_t launch_ilu_factor(const IluHost& H, const double* val, int* bad, cud
         const int r0 = H.starts[c], r1 = H.starts[c + 1];
         if (r1 > r0) k_ilu0_colour<<<(unsigned)((r1 - r0 + 255) / 256), 256, 0, st>>>(r0, r1, I.rp, I.col, I.diag, I.lu, bad);
     }
-    if (H.n > 0) k_ilu_pivots<<<(unsigned)((H.n + 255) / 256), 256, 0, st>>>(H.n, I.diag, I.lu, H.piv);
+    if (H.n > 0) k_ilu_pivots<<<(unsigned)((H.n + 255) / 256), 256, 0, st>>>(H.n, I.diag, I.lu, H.piv, bad);
     g_launches += 2 + H.ncol;
     return cudaGetLastError();
 }
@@ -181,7 +185,7 @@ cudaError_t launch_ilu_columns(const IluHost& H, int* ocol, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <bool FWD>
+template <bool FWD, bool DIV>
 static void ilu_pass(const Plan& P, int i, int c, bool edge, const double* u, double* out) {
     const IluHost& H = *P.ilu_host;
     const int r0 = H.starts[c], r1 = H.starts[c + 1];
@@ -191,18 +195,24 @@ static void ilu_pass(const Plan& P, int i, int c, bool edge, const double* u, do
     const unsigned grid = (unsigned)((r1 - r0 + chunk - 1) / chunk);
     if (H.maxlen <= 16) {
         const size_t sm = 16 * (size_t)stage_bytes<double>(H.maxlen);
-        set_smem((const void*)k_ilu_pass<FWD, true>, sm);
-        k_ilu_pass<FWD, true><<<grid, 512, sm, P.st>>>(P, i, r0, r1, chunk, edge, H.maxlen, u, H.dev.y, out);
+        set_smem((const void*)k_ilu_pass<FWD, true, DIV>, sm);
+        k_ilu_pass<FWD, true, DIV><<<grid, 512, sm, P.st>>>(P, i, r0, r1, chunk, edge, H.maxlen, u, H.dev.y, out);
     } else {
-        k_ilu_pass<FWD, false><<<grid, 512, 0, P.st>>>(P, i, r0, r1, chunk, edge, H.maxlen, u, H.dev.y, out);
+        k_ilu_pass<FWD, false, DIV><<<grid, 512, 0, P.st>>>(P, i, r0, r1, chunk, edge, H.maxlen, u, H.dev.y, out);
     }
     ++g_launches;
 }
 
-void launch_ilu_apply(const Plan& P, int i, const double* u, double* out) {
+template <bool DIV>
+static void ilu_apply(const Plan& P, int i, const double* u, double* out) {
     const int ncol = P.ilu_host->ncol;
-    for (int c = std::min(1, ncol - 1); c < ncol; ++c) ilu_pass<true>(P, i, c, c == ncol - 1, u, out);
-    for (int c = ncol - 2; c >= 0; --c) ilu_pass<false>(P, i, c, c == 0, u, out);
+    for (int c = std::min(1, ncol - 1); c < ncol; ++c) ilu_pass<true, DIV>(P, i, c, c == ncol - 1, u, out);
+    for (int c = ncol - 2; c >= 0; --c) ilu_pass<false, DIV>(P, i, c, c == 0, u, out);
+}
+
+void launch_ilu_apply(const Plan& P, int i, const double* u, double* out) {
+    if (P.ilu_host->divide) ilu_apply<true>(P, i, u, out);
+    else ilu_apply<false>(P, i, u, out);
 }
 
 }  // namespace sfg

@@ -220,3 +220,36 @@ def test_sketch_pieces_do_not_depend_on_the_launches(Solver, precision, s, t):
         got.append(sv.inner_cycle(v, m=8, s=s, k=t)[0].cpu().numpy())
     assert np.array_equal(*got)
     sv.close()
+
+
+# ILU(0) passes multiply by the pivots' reciprocals, or divide where one overflows, also after new values between replays.  z =
+# y_0 M^{-1} v by the two colours' substitutions; where v is zero the scale of the row cancels.  Bound: eight roundings of
+# products and sums beside 1e-310 (units of 2^-1074, some 4e-13 of the pivot), and FP64's own.
+@pytest.mark.parametrize("n", [64, 513, 1025])
+def test_ilu_pivot_without_a_reciprocal(Solver, n):
+    A = workloads.convdiff(n, (5.0,))
+    val, k = A.val / abs(A.val).max(), 33
+    v = np.random.default_rng(n).standard_normal(n)
+    v[k] = 0.0
+    v /= np.linalg.norm(v)
+    M = A.to_scipy().tocsr()
+    M.data = val.copy()
+    odd, even = np.arange(1, n, 2), np.arange(0, n, 2)
+    d = M.diagonal()
+    L, U = M[odd][:, even] @ np.diag(1.0 / d[even]), M[even][:, odd].toarray()
+    want = np.empty(n)
+    want[odd] = (v[odd] - L @ v[even]) / (d[odd] - np.einsum("ij,ji->i", L, U))
+    want[even] = (v[even] - U @ want[odd]) / d[even]
+    small = val.copy()
+    small[A.row_ptr[k]:A.row_ptr[k + 1]] *= 1e-310
+    sv = Solver(n, A.row_ptr, A.col, val, sketch_seed=1, precond=1, max_outer=200)
+    for values in (val, small, val):
+        sv.update_values(dev_vec(values))
+        z, kk, _, _, y = sv.inner_cycle(dev_vec(v), m=1, s=32, k=1)
+        z, y = z.cpu().numpy(), float(y.cpu()[0])
+        assert kk == 1 and y != 0.0
+        assert np.max(np.abs(z / y - want)) <= 1e-12 + 1e-14 * np.max(np.abs(want))
+        x, info = sv.solve(dev_vec(v), m=30, s=60, k=2, tol=1e-8)
+        M.data = values.copy()
+        assert info["status"] == 0 and np.linalg.norm(v - M @ x.cpu().numpy()) <= 1.01e-8
+    sv.close()

@@ -1171,7 +1171,9 @@ int run_cycle(sfgmres_ctx* h, const Plan& P, int j, const double* v, const doubl
     return 0;
 }
 
-// Everything a captured outer step depends on: the plan's pointers and sizes and the cycle options.
+// Everything a captured outer step depends on: the plan's pointers and sizes, the version of the list blocks (which is never
+// used twice, so lists, orders or copies built anew never pass for freed ones, whatever addresses they got) and the
+// cycle options.
 std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
     std::vector<uint64_t> k;
     auto u = [&](const void* p) { k.push_back((uint64_t)(uintptr_t)p); };
@@ -1189,10 +1191,11 @@ std::vector<uint64_t> plan_key(const sfgmres_ctx* h, const Plan& P) {
                           (const void*)P.ffom_hist, (const void*)P.ires_hist, (const void*)P.rho_hist,
                           (const void*)P.k_hist, (const void*)P.reason_hist,
                           (const void*)P.ost, (const void*)P.st, (const void*)h->qst, (const void*)P.gsync,
-                          (const void*)P.xin, (const void*)P.ilu.lu, (const void*)P.so_off, (const void*)P.so_col,
-                          (const void*)P.so_val, (const void*)P.so_val32})
+                          (const void*)P.xin, (const void*)P.ilu.lu, (const void*)P.so_off, (const void*)P.so_len,
+                          (const void*)P.so_col, (const void*)P.so_val, (const void*)P.so_val32,
+                          (const void*)P.so_base})
         u(p);
-    for (int64_t v : std::initializer_list<int64_t>{(int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.staged, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
+    for (int64_t v : std::initializer_list<int64_t>{(int64_t)h->geo_ver, (int64_t)P.nnz, (int64_t)P.vec, (int64_t)P.staged, (int64_t)P.N, (int64_t)P.P, (int64_t)P.nblk, (int64_t)P.Bn,
                       (int64_t)P.s, (int64_t)P.zeta, (int64_t)P.kind, (int64_t)P.sk_headroom, (int64_t)P.prec,
                       (int64_t)P.m, (int64_t)P.t, (int64_t)P.qr.cluster, (int64_t)P.qr.staged, (int64_t)P.jmax, (int64_t)h->c3,
                       (int64_t)h->profile, (int64_t)P.gwait_extra, (int64_t)P.outer_variant,

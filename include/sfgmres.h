@@ -66,8 +66,9 @@ extern "C" {
                                         sfgmres_stats), default 0 */
 #define SFGMRES_OPT_SPMV_VECTOR 8    /* lanes per CSR row in the SpMV (2,4,8,16,32), or 0 (default) = chosen by the
                                         library: one thread per row when no row has more than 16 entries, else the
-                                        length-binned SpMV (each row block's rows ordered by length: short rows one
-                                        thread each, 17..64 entries 8 lanes, longer rows a warp).  Reading it
+                                        length-binned SpMV (each row block's rows ordered by length: one thread each,
+                                        up to 512 entries, from a sorted copy of them as far as they fill slices of 32
+                                        rows; the others 8 lanes, or a warp beyond 64 entries).  Reading it
                                         returns the shape in use: 1, 2..32, or 0 for the length-binned SpMV. */
 #define SFGMRES_OPT_BLOCK_ROWS 9     /* rows per row block of the fused inner kernels: a multiple of 32 in
                                         [32, 8192], or 0 (default) = chosen by the library (one system: two blocks

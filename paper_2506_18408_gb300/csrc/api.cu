@@ -640,7 +640,7 @@ int ensure_bins(sfgmres_ctx* h, bool transpose) {
     if (!h->perm[t]) CK(cudaMalloc(&h->perm[t], std::max<size_t>(h->n, 1) * sizeof(uint16_t)));
     if (h->cls[t]) cudaFree(h->cls[t]);
     h->cls[t] = nullptr;
-    CK(cudaMalloc(&h->cls[t], 3 * (size_t)h->nl * sizeof(int)));
+    CK(cudaMalloc(&h->cls[t], 2 * (size_t)h->nl * sizeof(int)));
     launch_bin_rows(h->nl, transpose ? h->rpT : h->rp, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->st);
     CK(cudaGetLastError());
     h->bins_ver[t] = h->geo_ver;
@@ -682,11 +682,10 @@ int ensure_slices(sfgmres_ctx* h) {
 }
 
 // The length-binned SpMV's sorted copy of A (or A^T): the rows of the current bins that take a thread each, as slices of the
-// block's length order, with FP64 values and, for FP32 and BF16 inner cycles, FP32 ones.
-int ensure_sorted(sfgmres_ctx* h, bool transpose) {
+// block's length order, with FP64 values and, if f32 (FP32 and BF16 inner cycles), FP32 ones.
+int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {
     const int t = transpose ? 1 : 0;
     ListSet::Sorted& S = h->so[t];
-    const bool f32 = h->prec != kFP64;
     if (S.ver == h->vals_ver && (S.val32 || !f32)) return 0;
     int rc;
     if ((rc = ensure_slices(h))) return rc;
@@ -770,7 +769,7 @@ void plan_geometry(sfgmres_ctx* h, const Geo* g, bool transpose, Plan& P) {
     P.perm = (P.vec == 0) ? h->perm[transpose ? 1 : 0] : nullptr;
     P.cls = (P.vec == 0) ? h->cls[transpose ? 1 : 0] : nullptr;
     const ListSet::Sorted& O = h->so[transpose ? 1 : 0];
-    const bool so = P.vec == 0 && O.ver == h->vals_ver;
+    const bool so = P.vec == 0;  // built by ensure_sorted before every launch
     P.so_off = so ? O.off : nullptr;
     P.so_len = so ? O.len : nullptr;
     P.so_col = so ? O.col : nullptr;
@@ -950,7 +949,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     const int maxlen = transpose ? h->maxlenT : h->maxlen;
     const bool staged = vec == 1 && h->prec != kFP64 && stage_fits(h, g->nblk, maxlen);
     if (vec == 0 && (rc = ensure_bins(h, transpose))) return rc;
-    if (vec == 0 && (rc = ensure_sorted(h, transpose))) return rc;
+    if (vec == 0 && (rc = ensure_sorted(h, transpose, h->prec != kFP64))) return rc;
     if (vec == 1 && h->prec == kFP64 && (rc = ensure_sell(h, transpose))) return rc;
     const size_t vt = (h->prec == kFP64) ? 8 : (h->prec == kFP32 ? 4 : 2);
     const size_t at = (h->prec == kFP64) ? 8 : 4;
@@ -2490,7 +2489,8 @@ int sfgmres_spmv(sfgmres_t h, const double* xv, double* yv) {
     choose_lists(h, 1);
     int rc = get_geometry(h, 1, &g);
     if (rc) return rc;
-    if (h->vec == 0 && (rc = ensure_bins(h, false))) return rc;
+    // the copy that the solves' products are formed with, so that y does not depend on what ran before
+    if (h->vec == 0 && ((rc = ensure_bins(h, false)) || (rc = ensure_sorted(h, false, false)))) return rc;
     Plan P;
     plan_geometry(h, g, false, P);
     launch_spmv_f64(P, xv, yv);

@@ -73,8 +73,8 @@ struct Plan {
     const double* sl_val = nullptr;
     const int* sl_base = nullptr;
     const uint16_t* perm = nullptr;  // length-binned SpMV: per matrix row block, its rows in length order
-    const int* cls = nullptr;        // [3 * list blocks] rows of the order with <= 16 entries, with <= 64, in the copy
-    // the length-binned SpMV's sorted copy (null: the CSR arrays through perm): slices of 32 rows of the order
+    const int* cls = nullptr;        // [2 * list blocks] rows of the order with <= 64 entries, and rows in the copy
+    // the length-binned SpMV's sorted copy: slices of 32 rows of the order
     const int* so_off = nullptr;       // slice widths as prefix sums in units of 32 entries
     const uint16_t* so_len = nullptr;  // per-lane row lengths
     const int* so_col = nullptr;
@@ -177,11 +177,11 @@ __device__ __forceinline__ BlockInfo block_info(const Plan& p, int b) {
     return bi;
 }
 
-// What the length-binned SpMV knows of a block: the rows of its order with at most 16 and at most 64 entries, and the sorted
-// copy's slices with the number of rows they hold (off null: no copy).
+// What the length-binned SpMV knows of a block: the rows of its order with at most 64 entries, and the sorted copy's slices
+// with the number of rows they hold.
 template <typename MT>
 struct SortedRows {
-    int n16, n64, na;
+    int n64, na;
     const int* off;
     const uint16_t* len;
     const int* col;
@@ -190,17 +190,14 @@ struct SortedRows {
 template <typename MT>
 __device__ __forceinline__ SortedRows<MT> sorted_rows(const Plan& p, const BlockInfo& bi) {
     SortedRows<MT> s;
-    s.n16 = p.cls[3 * bi.list];
-    s.n64 = p.cls[3 * bi.list + 1];
-    s.na = p.cls[3 * bi.list + 2];
-    const MT* val;
-    if constexpr (sizeof(MT) == 8) val = p.so_val;
-    else val = p.so_val32;
-    const int base = val ? p.so_base[bi.list] : 0;
-    s.off = val ? p.so_off + base : nullptr;
+    s.n64 = p.cls[2 * bi.list];
+    s.na = p.cls[2 * bi.list + 1];
+    const int base = p.so_base[bi.list];
+    s.off = p.so_off + base;
     s.len = p.so_len + (int64_t)base * 32;
     s.col = p.so_col;
-    s.val = val;
+    if constexpr (sizeof(MT) == 8) s.val = p.so_val;
+    else s.val = p.so_val32;
     return s;
 }
 
@@ -286,8 +283,8 @@ void launch_gather_vals(int64_t nnz, const int* src, const double* val, double* 
 void launch_pattern_outer(int n, const int* rp, const int* col, const double* u, const double* v, double alpha,
                           double* out, cudaStream_t st);
 // Row order of every matrix row block (nl blocks, block L = rows lb_m0[L] .. + lb_len[L]) for the length-binned
-// SpMV: perm[m0 + i] = local offset of the i-th row by (length, position); cls[3L ..]: rows with at most 16 entries, with
-// at most 64, and rows the sorted copy takes.
+// SpMV: perm[m0 + i] = local offset of the i-th row by (length, position); cls[2L ..]: rows with at most 64 entries, and rows
+// the sorted copy takes.
 constexpr int kSortedMax = 512;  // longest row of the sorted copy
 void launch_bin_rows(int nl, const int* rp, const int* lb_m0, const int* lb_len, uint16_t* perm, int* cls,
                      cudaStream_t st);

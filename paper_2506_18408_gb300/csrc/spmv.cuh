@@ -329,15 +329,14 @@ __device__ __forceinline__ void sorted_chunk(const int* __restrict__ cp, const M
 }
 
 // Length-binned SpMV of one block for matrices with irregular rows: out[k] for the block's local rows k, matrix rows
-// m0 + k.  The block's rows come in a precomputed order pm[0 .. len) (local offsets), by length.  With the sorted copy its
-// first so.na rows take one thread each, 32 rows of (nearly) one length per warp from a slice that the warp reads
+// m0 + k.  The block's rows come in a precomputed order pm[0 .. len) (local offsets), by length.  The first so.na, those of the
+// sorted copy, take one thread each, 32 rows of (nearly) one length per warp from a slice that the warp reads
 // coalesced: every FP64 instruction does 32 rows' products and no sum needs a shuffle tree (with 8 lanes or a warp per row
 // the trees and half-empty passes doubled the FP64 instructions of a 2M-row Zipf matrix, on a GPU whose FP64 pipe takes 17
 // cycles per warp and instruction).  Warps take the slices longest first, in alternating direction, so that their loads
 // even out.  2M rows, FP64: 270 -> 235 us per launch; whole steps 1M rows 227 -> 164 us, 1.5M FP32 213 -> 179 us.
-// The rows that the copy leaves (too long for the block, or slices that would be half empty), and without a copy the rows beyond
-// 16 entries, take 8 lanes (17..64 entries) or a warp from the CSR arrays.  Every row's sum runs over its entries in a
-// fixed order.
+// The rows that the copy leaves (too long for the block, or slices that would be half empty) take 8 lanes (up to 64 entries) or a
+// warp from the CSR arrays.  Every row's sum runs over its entries in a fixed order.
 template <typename MT, typename XT, typename AT>
 __device__ __forceinline__ void spmv_rows_binned(const int* __restrict__ rp, const int* __restrict__ col,
                                                  const MT* __restrict__ val, const XT* __restrict__ x, int m0, int len,
@@ -346,60 +345,34 @@ __device__ __forceinline__ void spmv_rows_binned(const int* __restrict__ rp, con
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint16_t* pm = perm + m0;
     const int* rpm = rp + m0;
-    int done;  // rows of the order that took a thread each
-    if (so.off) {
-        done = so.na;
-        const int ns = (so.na + 31) / 32;
-        for (int t0 = 0, flip = 0; t0 < ns; t0 += nwarps, flip ^= 1) {
-            const int t = t0 + (flip ? nwarps - 1 - warp : warp);
-            if (t >= ns) continue;
-            const int s = ns - 1 - t, i = 32 * s + lane;
-            const int o = __ldg(so.off + s), w = __ldg(so.off + s + 1) - o, rl = so.len[(int64_t)s * 32 + lane];
-            const int k = (i < so.na) ? pm[i] : -1;
-            const int* cp = so.col + (int64_t)o * 32 + lane;
-            const MT* vp = so.val + (int64_t)o * 32 + lane;
-            constexpr int CH = 8;
-            AT sum = AT(0);
-            int pk = 0;
-            for (; pk + CH < w; pk += CH) sorted_chunk<CH>(cp, vp, x, rl, pk, sum);
-            switch (w - pk) {
-                case 1: sorted_chunk<1>(cp, vp, x, rl, pk, sum); break;
-                case 2: sorted_chunk<2>(cp, vp, x, rl, pk, sum); break;
-                case 3: sorted_chunk<3>(cp, vp, x, rl, pk, sum); break;
-                case 4: sorted_chunk<4>(cp, vp, x, rl, pk, sum); break;
-                case 5: sorted_chunk<5>(cp, vp, x, rl, pk, sum); break;
-                case 6: sorted_chunk<6>(cp, vp, x, rl, pk, sum); break;
-                case 7: sorted_chunk<7>(cp, vp, x, rl, pk, sum); break;
-                case 8: sorted_chunk<8>(cp, vp, x, rl, pk, sum); break;
-                default: break;
-            }
-            if (k >= 0) out[k] = sum;
+    const int ns = (so.na + 31) / 32;
+    for (int t0 = 0, flip = 0; t0 < ns; t0 += nwarps, flip ^= 1) {
+        const int t = t0 + (flip ? nwarps - 1 - warp : warp);
+        if (t >= ns) continue;
+        const int s = ns - 1 - t, i = 32 * s + lane;
+        const int o = __ldg(so.off + s), w = __ldg(so.off + s + 1) - o, rl = so.len[(int64_t)s * 32 + lane];
+        const int k = (i < so.na) ? pm[i] : -1;
+        const int* cp = so.col + (int64_t)o * 32 + lane;
+        const MT* vp = so.val + (int64_t)o * 32 + lane;
+        constexpr int CH = 8;
+        AT sum = AT(0);
+        int pk = 0;
+        for (; pk + CH < w; pk += CH) sorted_chunk<CH>(cp, vp, x, rl, pk, sum);
+        switch (w - pk) {
+            case 1: sorted_chunk<1>(cp, vp, x, rl, pk, sum); break;
+            case 2: sorted_chunk<2>(cp, vp, x, rl, pk, sum); break;
+            case 3: sorted_chunk<3>(cp, vp, x, rl, pk, sum); break;
+            case 4: sorted_chunk<4>(cp, vp, x, rl, pk, sum); break;
+            case 5: sorted_chunk<5>(cp, vp, x, rl, pk, sum); break;
+            case 6: sorted_chunk<6>(cp, vp, x, rl, pk, sum); break;
+            case 7: sorted_chunk<7>(cp, vp, x, rl, pk, sum); break;
+            case 8: sorted_chunk<8>(cp, vp, x, rl, pk, sum); break;
+            default: break;
         }
-    } else {
-        done = so.n16;
-        for (int i0 = warp * 32; i0 < so.n16; i0 += nwarps * 32) {  // warp-uniform loop over the short rows
-            const int i = i0 + lane;
-            int k = -1, a = 0, rl = 0;
-            if (i < so.n16) {
-                k = pm[i];
-                a = __ldg(rpm + k);
-                rl = __ldg(rpm + k + 1) - a;
-            }
-            const int maxlen = (int)__reduce_max_sync(0xffffffffu, (unsigned)rl);
-            AT sum = AT(0);
-            for (int pk = 0; pk < maxlen; pk += 4) {
-                switch (min(maxlen - pk, 4)) {
-                    case 1: row_chunk<1>(col, val, x, a, rl, pk, sum); break;
-                    case 2: row_chunk<2>(col, val, x, a, rl, pk, sum); break;
-                    case 3: row_chunk<3>(col, val, x, a, rl, pk, sum); break;
-                    default: row_chunk<4>(col, val, x, a, rl, pk, sum); break;
-                }
-            }
-            if (k >= 0) out[k] = sum;
-        }
+        if (k >= 0) out[k] = sum;
     }
-    const int mid = max(done, so.n64);
-    spmv_sorted_vector<8, 2, 2, MT, XT, AT>(rpm, col, val, x, pm, done, mid, out);
+    const int mid = max(so.na, so.n64);
+    spmv_sorted_vector<8, 2, 2, MT, XT, AT>(rpm, col, val, x, pm, so.na, mid, out);
     spmv_sorted_vector<32, 2, 4, MT, XT, AT>(rpm, col, val, x, pm, mid, len, out);
 }
 

@@ -138,8 +138,7 @@ __global__ void __launch_bounds__(256) k_bin_rows(const int* __restrict__ rp, co
             cur[b] = run;
             run += cnt[b];
         }
-        cls[3 * L] = cur[17];
-        cls[3 * L + 1] = cur[65];
+        cls[2 * L] = cur[65];
     }
     const unsigned lt = (1u << lane) - 1u;
     for (int base = 0; base < len; base += blockDim.x) {
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(256) k_bin_rows(const int* __restrict__ rp, co
             const int sum = (int)__reduce_add_sync(0xffffffffu, l), w = (int)__reduce_max_sync(0xffffffffu, l);
             if (w <= 16 || (w <= kSortedMax && w <= most && 32 * w <= 2 * sum)) break;
         }
-        if (lane == 0) cls[3 * L + 2] = min(len, 32 * (q + 1));
+        if (lane == 0) cls[2 * L + 1] = min(len, 32 * (q + 1));
     }
 }
 
@@ -184,13 +183,13 @@ void launch_bin_rows(int nl, const int* rp, const int* lb_m0, const int* lb_len,
 
 // ---- the length-binned SpMV's sorted copy (SELL-32 over each row block's length order) ----
 // Slice base[L] + q holds rows 32q .. 32q+31 of block L's order (local rows perm[m0 + 32q + lane]), those below the block's
-// boundary cls[3L + 2]; it is as wide as its longest row and stored like the SELL-32 copy below.
+// boundary cls[2L + 1]; it is as wide as its longest row and stored like the SELL-32 copy below.
 
 // One CTA per row block: row lengths and slice widths (0 beyond the boundary).
 __global__ void k_sorted_len(const int* __restrict__ rp, const int* __restrict__ lb_m0, const int* __restrict__ lb_len,
                              const uint16_t* __restrict__ perm, const int* __restrict__ cls,
                              const int* __restrict__ base, uint16_t* __restrict__ len, int* __restrict__ wid) {
-    const int L = blockIdx.x, m0 = lb_m0[L], nr = lb_len[L], na = cls[3 * L + 2];
+    const int L = blockIdx.x, m0 = lb_m0[L], nr = lb_len[L], na = cls[2 * L + 1];
     const int lane = threadIdx.x & 31;
     for (int q = threadIdx.x >> 5; 32 * q < nr; q += blockDim.x >> 5) {
         const int i = 32 * q + lane;
@@ -213,7 +212,7 @@ __global__ void k_sorted_fill(const int* __restrict__ rp, const int* __restrict_
                               const uint16_t* __restrict__ perm, const int* __restrict__ cls,
                               const int* __restrict__ base, const int* __restrict__ off, int* __restrict__ scol,
                               MT* __restrict__ sval) {
-    const int L = blockIdx.x, m0 = lb_m0[L], na = cls[3 * L + 2];
+    const int L = blockIdx.x, m0 = lb_m0[L], na = cls[2 * L + 1];
     const int lane = threadIdx.x & 31;
     for (int q = threadIdx.x >> 5; 32 * q < na; q += blockDim.x >> 5) {
         const int i = 32 * q + lane;

@@ -328,6 +328,81 @@ __device__ __forceinline__ void sorted_chunk(const int* __restrict__ cp, const M
         if (pk + q < rl) sum += v[q] * xv[q];
 }
 
+// *out = the lane's row in a slice of w entries per row (out: a shared slot, null for lanes without a row).
+//
+// Up to 16 entries are one running sum.  A longer row's error would grow with its length (one running sum had 1.4 to 4.4
+// times the error of lanes' sums joined by a tree at 17 to 512 entries), so it is summed in chunks of at most eight of nearly one
+// size, each as two interleaved sums; the chunks' sums are added in groups, two of them up to 64 entries and of four chunks
+// beyond, and the groups into *out, the third and later ones with what that addition lost carried into the next group.  Against
+// the lanes' sums (8 up to 64 entries, else 32) that measures 1.02 to 1.05 of the error at 17 to 32 entries, 1.00 to 0.95 up to
+// 64, 1.03 at 65, 0.98 at 96, 0.83 at 256 and 0.71 at 512 (a dominant entry anywhere in the row, normal values; FP32 and FP64
+// alike).  The total stays in shared memory and a chunk's columns are loaded with the one before: eight gathers in flight
+// leave a thread of the FP64 kernels' 56 registers no room for a second set of sums.
+// Cycles of 60 steps on Zipf rows with one running sum and so, ms: FP64 2M rows 18.0 and 17.9, 1M 10.05 and 10.20, 700,000 9.84 and 9.79;
+// FP32 2M 14.4 and 14.7, 1M 7.87 and 7.75.  (Eight running sums per row: 18.8, 10.5 and 10.0 with eight loads in flight, which spill,
+// 17.2, 10.7 and 11.0 with four.)
+template <typename MT, typename XT, typename AT>
+__device__ __forceinline__ void sorted_row(const int* __restrict__ cp, const MT* __restrict__ vp,
+                                           const XT* __restrict__ x, int rl, int w, AT* out) {
+    int pk = 0;
+    AT sum = AT(0);
+    if (w <= 16) {
+        for (; pk + 8 < w; pk += 8) sorted_chunk<8>(cp, vp, x, rl, pk, sum);
+        switch (w - pk) {
+            case 1: sorted_chunk<1>(cp, vp, x, rl, pk, sum); break;
+            case 2: sorted_chunk<2>(cp, vp, x, rl, pk, sum); break;
+            case 3: sorted_chunk<3>(cp, vp, x, rl, pk, sum); break;
+            case 4: sorted_chunk<4>(cp, vp, x, rl, pk, sum); break;
+            case 5: sorted_chunk<5>(cp, vp, x, rl, pk, sum); break;
+            case 6: sorted_chunk<6>(cp, vp, x, rl, pk, sum); break;
+            case 7: sorted_chunk<7>(cp, vp, x, rl, pk, sum); break;
+            case 8: sorted_chunk<8>(cp, vp, x, rl, pk, sum); break;
+            default: break;
+        }
+        if (out) *out = sum;
+        return;
+    }
+    const int chunks = (w + 7) / 8, step = (w + chunks - 1) / chunks, group = chunks <= 8 ? (chunks + 1) / 2 : 4;
+    int c[8], left = group;
+    bool first = true;
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (q < step) c[q] = __ldcs(cp + q * 32);
+    for (; pk < w; pk += step) {
+        const int cnt = min(step, w - pk), next = min(step, w - pk - step);
+        AT v[8], xv[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = (q < cnt) ? (AT)__ldcs(vp + (pk + q) * 32) : AT(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) xv[q] = (q < cnt && pk + q < rl) ? load_as(x + c[q], AT()) : AT(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < next) c[q] = __ldcs(cp + (pk + step + q) * 32);
+        AT s0 = AT(0), s1 = AT(0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < cnt && pk + q < rl) {
+                if (q & 1) s1 += v[q] * xv[q];
+                else s0 += v[q] * xv[q];
+            }
+        sum += s0 + s1;
+        if (--left == 0 && next > 0) {  // a group but the last
+            left = group;
+            if (first) {
+                if (out) *out = sum;
+                sum = AT(0);
+                first = false;
+            } else {
+                const AT t0 = out ? *out : AT(0), t = t0 + sum, d = t - t0;
+                const AT lost = (t0 - (t - d)) + (sum - d);
+                if (out) *out = t;
+                sum = isfinite(t) ? lost : AT(0);
+            }
+        }
+    }
+    if (out) *out += sum;
+}
+
 // Length-binned SpMV of one block for matrices with irregular rows: out[k] for the block's local rows k, matrix rows
 // m0 + k.  The block's rows come in a precomputed order pm[0 .. len) (local offsets), by length.  The first so.na, those of the
 // sorted copy, take one thread each, 32 rows of (nearly) one length per warp from a slice that the warp reads
@@ -354,22 +429,7 @@ __device__ __forceinline__ void spmv_rows_binned(const int* __restrict__ rp, con
         const int k = (i < so.na) ? pm[i] : -1;
         const int* cp = so.col + (int64_t)o * 32 + lane;
         const MT* vp = so.val + (int64_t)o * 32 + lane;
-        constexpr int CH = 8;
-        AT sum = AT(0);
-        int pk = 0;
-        for (; pk + CH < w; pk += CH) sorted_chunk<CH>(cp, vp, x, rl, pk, sum);
-        switch (w - pk) {
-            case 1: sorted_chunk<1>(cp, vp, x, rl, pk, sum); break;
-            case 2: sorted_chunk<2>(cp, vp, x, rl, pk, sum); break;
-            case 3: sorted_chunk<3>(cp, vp, x, rl, pk, sum); break;
-            case 4: sorted_chunk<4>(cp, vp, x, rl, pk, sum); break;
-            case 5: sorted_chunk<5>(cp, vp, x, rl, pk, sum); break;
-            case 6: sorted_chunk<6>(cp, vp, x, rl, pk, sum); break;
-            case 7: sorted_chunk<7>(cp, vp, x, rl, pk, sum); break;
-            case 8: sorted_chunk<8>(cp, vp, x, rl, pk, sum); break;
-            default: break;
-        }
-        if (k >= 0) out[k] = sum;
+        sorted_row<MT, XT, AT>(cp, vp, x, rl, w, k >= 0 ? out + k : nullptr);
     }
     const int mid = max(so.na, so.n64);
     spmv_sorted_vector<8, 2, 2, MT, XT, AT>(rpm, col, val, x, pm, so.na, mid, out);

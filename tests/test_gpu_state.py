@@ -53,3 +53,49 @@ def test_product_does_not_depend_on_earlier_calls(Solver, precision):
     sv.solve_batch(many, nrhs=7, transpose=True, **PAR)
     assert np.array_equal(sv.spmv(x).cpu().numpy(), want)
     sv.close()
+
+
+# Single solves, several numbers of right-hand sides (row blocks of as many sizes), y = A x and S v in turn: what each needs is
+# built once, so that later rounds launch only the solves' own kernels, and give the same bits.
+@pytest.mark.parametrize("kind", ["convdiff", "zipf"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_calls_in_turn_build_their_row_blocks_once(Solver, kind, precision):
+    A = workloads.convdiff(64, (30.0, 10.0)) if kind == "convdiff" else workloads.random_zipf(6000, seed=3)
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, precision=precision)
+    counts = (1, 2, 4, 8, 16)
+    b = {r: dev_vec(workloads.rhs(r * A.n, seed=r)) for r in counts}
+    rounds = []
+    for _ in range(4):
+        launches, out = [], []
+        for r in counts:
+            x, info = sv.solve(b[1], **PAR) if r == 1 else sv.solve_batch(b[r], nrhs=r, **PAR)
+            assert info["status"] == 0
+            launches.append(info["kernel_launches"])
+            out += [x.cpu().numpy(), sv.spmv(b[1]).cpu().numpy(), sv.sketch(b[1], 120).cpu().numpy()]
+        rounds.append((launches, out))
+    for launches, out in rounds[1:]:
+        assert all(q < p for q, p in zip(launches[1:], rounds[0][0][1:])) and launches == rounds[1][0]
+        assert all(np.array_equal(p, q) for p, q in zip(out, rounds[0][1]))
+    sv.close()
+
+
+# a captured outer step is not replayed on row blocks built anew: sizes set back and forth with cycles, products and sketches (which
+# capture nothing) between two solves, more sizes than a handle keeps
+@pytest.mark.parametrize("kind", ["convdiff", "zipf"])
+def test_replay_after_row_blocks_were_rebuilt(Solver, kind):
+    A = workloads.convdiff(64, (30.0, 10.0)) if kind == "convdiff" else workloads.random_zipf(6000, seed=3)
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, block_rows=512)
+    b = dev_vec(workloads.rhs(A.n, seed=0))
+    v = b / b.norm()
+    want = sv.solve(b, **PAR)[0].cpu().numpy()
+    for rows in range(544, 544 + 32 * 40, 32):
+        sv.set("block_rows", rows)
+        sv.inner_cycle(v, m=4, s=120, k=2)
+        sv.spmv(b)
+    sv.set("block_rows", 512)
+    assert np.array_equal(sv.solve(b, **PAR)[0].cpu().numpy(), want)
+    sv.autotune(m=30, s=120, k=2)
+    sv.set("block_rows", 512)
+    sv.set("spmv_vector", 0)
+    assert np.array_equal(sv.solve(b, **PAR)[0].cpu().numpy(), want)
+    sv.close()

@@ -178,6 +178,11 @@ struct sfgmres_ctx : ListSet {
             rho_hist, k_hist, reason_hist, ost, pflag, rhs;
     };
     std::vector<LevelWs> lvl;
+    struct QrPlaced {
+        bool staged, places;
+        size_t smem;
+    };
+    std::vector<QrPlaced> qr_placed;  // sketched-QR clusters beyond the portable size that the device was asked about
     DevBuf gsync;           // fused inner step: grid arrival counters [0], [2] and give-up flag [1] (u64)
 
     // pinned host mirrors of the per-problem device state
@@ -1008,7 +1013,15 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
     const size_t stage = staged ? stage_smem(maxlen) : 0;
     const bool beside = vec == 0 || t > 4 || !h->fuse_step;  // binned, or steps of two launches (launch_inner_step)
-    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), vec == 0);
+    const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), vec == 0,
+                                [&](const QrShape& q) {
+                                    const size_t smem = qr_smem(q, m, m - 1);
+                                    for (const auto& known : h->qr_placed)
+                                        if (known.staged == q.staged && known.smem == smem) return known.places;
+                                    if (h->qr_placed.size() >= 64) h->qr_placed.clear();
+                                    h->qr_placed.push_back({q.staged, qr_places(q, m), smem});
+                                    return h->qr_placed.back().places;
+                                });
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;
     if ((rc = ensure(h, h->R, Pn * M * M * 8))) return rc;
     if ((rc = ensure(h, h->d, Pn * M * 8))) return rc;

@@ -13,7 +13,6 @@ constexpr int kMaxZeta = 16;    // largest number of nonzeros per sketch column
 constexpr int kMaxS = 4096;     // largest sketch size
 constexpr int kMaxM = 1024;     // largest inner basis size
 constexpr int kBlockRowsMax = 8192;  // rows per row block (local sketch offsets need <= 15 bits)
-constexpr int kQrCluster = 16;       // most CTAs of the cluster that runs a sketched QR update
 constexpr int kQrSms = 8;            // SMs that the row-block rule for medium systems leaves to the sketched QR
 
 // ------------------------------------------------------------------------------------------------------------

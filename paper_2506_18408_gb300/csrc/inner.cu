@@ -512,41 +512,45 @@ void launch_inner_axpy(const Plan& p, int i, bool last) {
     ++g_launches;
 }
 
-// Dynamic shared memory of update i: the staged columns, the CTA's rows of p and e, the projections and their parts.
-static size_t qr_smem(const QrShape& q, int m, int i) {
-    return ((size_t)(q.staged ? (i * q.nrp + 1) & ~1 : 0) + 2 * (size_t)q.nrp + 3 * (size_t)m) * sizeof(double);
+// The kernel for a shape, with the attributes that its launches need.
+using QrKernel = void (*)(const Plan, int);
+static cudaError_t qr_kernel(const QrShape& q, int m, QrKernel* fn) {
+    *fn = q.staged ? k_inner_qr<true> : k_inner_qr<false>;
+    set_smem((const void*)*fn, qr_smem(q, m, m - 1));
+    return q.cluster > kQrPortable
+               ? cudaFuncSetAttribute((const void*)*fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
+               : cudaSuccess;
 }
 
-// Few CTAs where an update's FP64 work is small (its latency is then the exchanges, which grow with the CTAs), many where it
-// is large.  Whole solves, 2 / 4 / 8 / 16 CTAs: s = 80, m = 20 (2D 32^2) 2.40 / 2.51 / 2.54 / 2.49 ms; s = 120, m = 30 (2D
-// 64^2) 4.34 / 4.12 / 5.21 / 5.03 ms; s = 240, m = 60 (3D 32^3) 3.36 / 3.19 / 3.56 / 3.41 ms; s = 320, m = 80 (40^3) 4.96 / 4.47
-// / 4.06 / 3.90 ms; s = 1000, m = 200 (80^3) 44.3 / 28.9 / 20.9 / 15.9 ms; beside the length-binned SpMV, s = 120, m = 30
-// (30,000 Zipf rows) 19.6 / 20.8 / 20.8 / 20.9 ms.  Batches take what leaves the problems' clusters
-// side by side on the GPU.
-QrShape qr_shape(int P, int s, int m, size_t smem_left, bool binned) {
-    QrShape q;
-    const int most = P <= 4 ? kQrCluster : P <= 16 ? 8 : P <= 32 ? 4 : P <= 64 ? 2 : 1;
-    q.cluster = std::min(most, s * m <= (binned ? 5000 : 3000) ? 2 : s * m <= 20000 ? 4 : kQrCluster);
-    q.nrp = ((s + q.cluster - 1) / q.cluster) | 1;
-    q.slice = (q.nrp * m + 1) & ~1;
-    q.staged = true;
-    q.staged = qr_smem(q, m, m - 1) + 3072 <= smem_left;  // its static shared memory and the reserve
-    return q;
+bool qr_places(const QrShape& q, int m) {
+    QrKernel fn;
+    int clusters = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)q.cluster, 1, 1);
+    cfg.blockDim = dim3(kQrThreads, 1, 1);
+    cfg.dynamicSmemBytes = qr_smem(q, m, m - 1);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = q.cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (qr_kernel(q, m, &fn) == cudaSuccess && cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess)
+        return clusters > 0;
+    cudaGetLastError();
+    return false;
 }
 
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st) {
     const QrShape& q = p.qr;
-    void (*fn)(const Plan, int) = q.staged ? k_inner_qr<true> : k_inner_qr<false>;
-    const size_t sm = qr_smem(q, p.m, i);
-    set_smem((const void*)fn, qr_smem(q, p.m, p.m - 1));
-    if (q.cluster > 8) {
-        const cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
+    QrKernel fn;
+    const cudaError_t e = qr_kernel(q, p.m, &fn);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(q.cluster * p.P), 1, 1);
     cfg.blockDim = dim3(kQrThreads, 1, 1);
-    cfg.dynamicSmemBytes = sm;
+    cfg.dynamicSmemBytes = qr_smem(q, p.m, i);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;

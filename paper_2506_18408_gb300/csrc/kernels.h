@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "shapes.h"
 
 namespace sfg {
 
@@ -43,14 +44,6 @@ struct IluHost {
     double2* piv = nullptr;    // device [n]: dev.piv, written by the factorisation
     const int* src = nullptr;  // device [nnz]: position in A's CSR of every entry of P A P^T
     IluDev dev;
-};
-
-// Shape of the sketched-QR update.
-struct QrShape {
-    int cluster = 8;     // CTAs per problem (one cluster)
-    int nrp = 0;         // rows of Q per CTA, padded to an odd number
-    int slice = 0;       // doubles of one CTA's slice of Q (nrp * m, even)
-    bool staged = false; // the slice is kept in shared memory during an update
 };
 
 // Everything a kernel needs, as plain device pointers and sizes (owned by the solver handle).
@@ -249,9 +242,7 @@ void inner_axpy_f64(const Plan& p, int i, bool last);
 void inner_axpy_f32(const Plan& p, int i, bool last);
 void inner_axpy_bf16(const Plan& p, int i, bool last);
 void launch_inner_axpy(const Plan& p, int i, bool last);
-// For P problems, sketch size s and basis size m, given the shared memory a QR CTA may take; binned: the step's SpMV is the length-
-// binned one.  The cluster, on which the rounding of the sums depends, is the same for steps of one and of two launches.
-QrShape qr_shape(int P, int s, int m, size_t smem_left, bool binned);
+bool qr_places(const QrShape& q, int m);  // the current device can hold one cluster of this shape
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st
 void launch_inner_finish(const Plan& p, double* z);  // y = R^{-1} d, z = sum_l y_l b_l (FP64)
 void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r] = sigma_l * u_l[r] (FP64)

@@ -100,45 +100,48 @@ __device__ __forceinline__ void two_sum(double& a, double& lost, double b) {
 }
 
 // c[r] = scale * the sum of part[b*s + r] over b: a CTA per 32 sketch rows (a lane each), warp w sums the partials w, w + 16,
-// ... as four interleaved sums, and the warps' sums are joined by a tree, for short vectors with what its roundings lose.  The
-// partials of a vector of a few thousand entries are of 128 columns each; added one after another they cost up to 1.4 times the
-// error of sums that are exact over 1024 columns, by a plain tree 1.12 times at 2,000 entries and 1.0 from 10,000 on, so up
-// to kCarryPartials of them (16,384 entries) the tree carries its losses.  (Every addition with what it loses, six FP64
-// instructions on eight SMs: 48 -> 69 us at n = 1,000,003, s = 240; the whole tree: 50 us.)
-constexpr int kCarryPartials = 128;
+// ... and the warps' sums are added in order.
+//
+// CARRY, for vectors of up to 32,768 entries, whose partials are of 128 columns each: the warps' sums are joined by a tree that
+// carries what its roundings lose.  Added one after another such partials cost up to 1.4 times the error of sums that are exact
+// over 1024 columns (3,000 entries; 1.2 at 10,000, 1.0 at 30,000, less beyond, where chunks are longer).  Back to back, a call
+// of 2,000 entries takes 11.1 us against 10.7, of 32,000 16.4 against 14.3; longer ones are as before (n = 1,000,003, s = 240: 51.2,
+// and 71.8 with every addition carrying its loss).
+constexpr int64_t kCarryCols = 32768;
+
+template <bool CARRY>
 __global__ void __launch_bounds__(512) k_noalloc_reduce(int nblk, int s, double scale, const double* __restrict__ part,
                                                         double* __restrict__ c) {
-    __shared__ double sh[16][32], sl[16][32];
+    __shared__ double sh[16][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = blockIdx.x * 32 + lane;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    double a = 0.0;
     if (r < s) {
-        for (int b = warp; b < nblk; b += 128) {
-            double v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = (b + 16 * u < nblk) ? part[(int64_t)(b + 16 * u) * s + r] : 0.0;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) a[u & 3] += v[u];
-        }
+#pragma unroll 8
+        for (int b = warp; b < nblk; b += 16) a += part[(int64_t)b * s + r];
     }
-    const bool carry = nblk <= kCarryPartials;
-    double sum = (a[0] + a[2]) + (a[1] + a[3]), lost = 0.0;
-#pragma unroll
-    for (int h = 8; h > 0; h >>= 1) {  // a level reads [h, 2h) and the next writes below h: one barrier each
-        if (warp < 2 * h) {
-            sh[warp][lane] = sum;
-            if (carry) sl[warp][lane] = lost;
-        }
+    sh[warp][lane] = a;
+    if constexpr (!CARRY) {
         __syncthreads();
-        if (warp >= h) continue;
-        if (carry) {
-            two_sum(sum, lost, sh[warp + h][lane]);
-            lost += sl[warp + h][lane];
-        } else {
-            sum += sh[warp + h][lane];
+        if (warp == 0 && r < s) {
+            for (int w = 1; w < 16; ++w) a += sh[w][lane];
+            c[r] = scale * a;
         }
+    } else {
+        __shared__ double sl[16][32];
+        double lost = 0.0;
+#pragma unroll
+        for (int h = 8; h > 0; h >>= 1) {  // a level reads [h, 2h) and the next writes below h: one barrier each
+            __syncthreads();
+            if (warp >= h) continue;
+            const double t = sh[warp + h][lane];
+            if (h < 8) lost += sl[warp + h][lane];
+            two_sum(a, lost, t);
+            sh[warp][lane] = a;
+            sl[warp][lane] = lost;
+        }
+        if (warp == 0 && r < s) c[r] = scale * (isfinite(a) ? a + lost : a);
     }
-    if (warp == 0 && r < s) c[r] = scale * (isfinite(sum) ? sum + lost : sum);
 }
 
 // Dynamic shared memory of k_noalloc_partials for s sketch rows: a 64-bit sum and an FP64 partial per row.
@@ -157,8 +160,7 @@ static PartialsKernel partials_kernel(int zeta) {
 
 // Once per device, with that device current: look up the device address of the scratch array (cudaGetSymbolAddress;
 // in host code the array's name is only a host-side stand-in) and allow k_noalloc_partials the dynamic shared memory
-// of the largest sketch (4096 rows need 48 KiB, which with the kernel's static shared memory is above the default
-// limit).  Both results are cached per device.
+// of the largest sketch (4096 rows need 64 KiB, above the default limit).  Both results are cached per device.
 static cudaError_t device_setup(double** out) {
     static std::mutex mu;
     static double* cache[64] = {nullptr};
@@ -239,8 +241,8 @@ extern "C" int sfgmres_sketch_apply_noalloc(int64_t n, int32_t s, int32_t zeta, 
                          cudaGetErrorString(e));
         return SFGMRES_ERR_CUDA;
     }
-    e = launch(k_noalloc_reduce, (unsigned)((s + 31) / 32), 512, 0, st, (int)nblk, (int)s,
-               1.0 / std::sqrt((double)zeta), (const double*)part, c);
+    e = launch(n <= kCarryCols ? k_noalloc_reduce<true> : k_noalloc_reduce<false>, (unsigned)((s + 31) / 32), 512, 0, st,
+               (int)nblk, (int)s, 1.0 / std::sqrt((double)zeta), (const double*)part, c);
     if (e != cudaSuccess) {
         set_global_error(std::string("sfgmres_sketch_apply_noalloc: launch of the reduction kernel: ") +
                          cudaGetErrorString(e));

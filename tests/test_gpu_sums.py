@@ -74,7 +74,7 @@ def test_long_rows_round_no_more_than_lanes(Solver, precision, length):
 
 # The allocation-free sketch adds a vector's sums of 128 columns (short vectors) without the error of plain additions: no larger
 # an error than that of sums that are exact over 1024 columns, whose own conversions and additions are two or three roundings.
-@pytest.mark.parametrize("n,s,zeta", [(1500, 40, 4), (3000, 100, 4), (6000, 64, 1), (12_000, 100, 16)])
+@pytest.mark.parametrize("n,s,zeta", [(1500, 40, 4), (3000, 100, 4), (6000, 64, 1), (12_000, 100, 16), (32_000, 240, 8), (33_000, 240, 8)])
 def test_allocation_free_sketch_of_short_vectors(n, s, zeta):
     need_gpu()
     from oracle import sketch as osk

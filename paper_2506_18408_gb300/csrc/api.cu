@@ -1019,7 +1019,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
                                     for (const auto& known : h->qr_placed)
                                         if (known.staged == q.staged && known.smem == smem) return known.places;
                                     if (h->qr_placed.size() >= 64) h->qr_placed.clear();
-                                    h->qr_placed.push_back({q.staged, qr_places(q, m), smem});
+                                    h->qr_placed.push_back({q.staged, qr_places(q, s, m), smem});
                                     return h->qr_placed.back().places;
                                 });
     if ((rc = ensure(h, h->Q, Pn * qs.cluster * qs.slice * 8))) return rc;

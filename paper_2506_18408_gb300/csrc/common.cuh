@@ -324,8 +324,7 @@ inline int sketch_pieces(int s) {
 }
 
 // Sum of x[k * stride] * y[k] over 0 <= k < n as the sums over even and over odd k: half as many roundings on an entry's way as
-// in one running sum.  (The sketched QR's products: an 80^3 cycle at s = 1000, m = 200 takes 9.75 ms against 9.72 with one sum and
-// 9.95 with four, a 64^2 solve 4.50 against 4.48 and 4.62.)
+// in one running sum.
 __host__ __device__ __forceinline__ double dot2(const double* __restrict__ x, int stride,
                                                     const double* __restrict__ y, int n) {
     double c0 = 0.0, c1 = 0.0;

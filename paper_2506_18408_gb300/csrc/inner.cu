@@ -43,6 +43,8 @@ namespace sfg {
 //  * projection a = Q^T p: column l by thread wp of group gp (Gp groups of rows), the CTAs' parts exchanged through
 //    distributed shared memory and summed in rank order (the same values in every CTA, so every decision is the same);
 //  * subtraction p -= Q a: row r by thread ws of group gs (Gs groups of columns).
+// A thread's part of a product is one running sum, or with LONG (qr_long) the sums over even and odd terms: a chain twice
+// as long has 1.4 times the rounding error.
 // Group partials are added in group order: every sum has a fixed order.  Five cluster barriers per update: one per pass, one
 // for ||p||^2 and p^T e together (d_i = p^T e / r_ii), one for the updated residual norm, and a last one before any
 // CTA leaves.  Each CTA reads the stop state itself (written by earlier launches; the one field another stream may change
@@ -52,7 +54,6 @@ namespace sfg {
 // An update takes (clock64 of CTA 0) 11 us at s = 120, i = 15 on 4 CTAs, 15 us at s = 400, i = 50 on 16 and 27 us at s = 1000,
 // i = 100 on 16; the earlier form, which streamed column- and row-major copies of Q from L2 on 8 CTAs, took 58 us per update
 // of an 80^3 cycle at s = 1000, m = 200 (that cycle 13.4 -> 8.4 ms).
-constexpr int kQrThreads = 128;
 
 // Sum of v over groups of 16 lanes (every lane gets its group's sum).
 __device__ __forceinline__ double half_warp_sum(double v) {
@@ -81,7 +82,7 @@ __device__ __forceinline__ double qr_pair_sum(double x, double y, double (*red)[
     return v;
 }
 
-template <bool STAGED>
+template <bool STAGED, bool LONG>
 __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i) {
     cg::cluster_group cl = cg::this_cluster();
     cl.barrier_arrive();  // waited for before the first access to another CTA's shared memory: all CTAs have started
@@ -144,7 +145,14 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
     for (int pass = 0; pass < 2 && i > 0; ++pass) {
         double* ap = part + pass * m;
         for (int l = wp; l < i; l += Wp) {
-            const double v = dot2(Q + l * nrp + pr0, 1, p + pr0, pr1 - pr0);
+            const double* ql = Q + l * nrp;
+            double v = 0.0;
+            if constexpr (LONG) {
+                v = dot2(ql + pr0, 1, p + pr0, pr1 - pr0);
+            } else {
+#pragma unroll 8
+                for (int r = pr0; r < pr1; ++r) v = fma(ql[r], p[r], v);
+            }
             if (Gp == 1) ap[l] = v;
             else grp[gp * i + l] = v;
         }
@@ -177,8 +185,14 @@ __global__ void __launch_bounds__(kQrThreads, 9) k_inner_qr(const Plan P, int i)
         __syncthreads();
         for (int r0 = 0; r0 < nr; r0 += Wr) {
             const int r = r0 + ws;
+            double v = 0.0;
             if (r < nr) {
-                const double v = dot2(Q + sl0 * nrp + r, nrp, a + sl0, sl1 - sl0);
+                if constexpr (LONG) {
+                    v = dot2(Q + sl0 * nrp + r, nrp, a + sl0, sl1 - sl0);
+                } else {
+#pragma unroll 8
+                    for (int l = sl0; l < sl1; ++l) v = fma(Q[l * nrp + r], a[l], v);
+                }
                 if (Gs == 1) p[r] -= v;
                 else grp[gs * Wr + ws] = v;
             }
@@ -514,15 +528,17 @@ void launch_inner_axpy(const Plan& p, int i, bool last) {
 
 // The kernel for a shape, with the attributes that its launches need.
 using QrKernel = void (*)(const Plan, int);
-static cudaError_t qr_kernel(const QrShape& q, int m, QrKernel* fn) {
-    *fn = q.staged ? k_inner_qr<true> : k_inner_qr<false>;
+static cudaError_t qr_kernel(const QrShape& q, int s, int m, int i, QrKernel* fn) {
+    const bool lg = qr_long(s, q.cluster, i);
+    if (q.staged) *fn = lg ? k_inner_qr<true, true> : k_inner_qr<true, false>;
+    else *fn = lg ? k_inner_qr<false, true> : k_inner_qr<false, false>;
     set_smem((const void*)*fn, qr_smem(q, m, m - 1));
     return q.cluster > kQrPortable
                ? cudaFuncSetAttribute((const void*)*fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
                : cudaSuccess;
 }
 
-bool qr_places(const QrShape& q, int m) {
+bool qr_places(const QrShape& q, int s, int m) {
     QrKernel fn;
     int clusters = 0;
     cudaLaunchConfig_t cfg = {};
@@ -536,7 +552,7 @@ bool qr_places(const QrShape& q, int m) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (qr_kernel(q, m, &fn) == cudaSuccess && cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess)
+    if (qr_kernel(q, s, m, m - 1, &fn) == cudaSuccess && cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess)
         return clusters > 0;
     cudaGetLastError();
     return false;
@@ -545,7 +561,7 @@ bool qr_places(const QrShape& q, int m) {
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st) {
     const QrShape& q = p.qr;
     QrKernel fn;
-    const cudaError_t e = qr_kernel(q, p.m, &fn);
+    const cudaError_t e = qr_kernel(q, p.s, p.m, i, &fn);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(q.cluster * p.P), 1, 1);

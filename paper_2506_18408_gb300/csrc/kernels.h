@@ -242,7 +242,7 @@ void inner_axpy_f64(const Plan& p, int i, bool last);
 void inner_axpy_f32(const Plan& p, int i, bool last);
 void inner_axpy_bf16(const Plan& p, int i, bool last);
 void launch_inner_axpy(const Plan& p, int i, bool last);
-bool qr_places(const QrShape& q, int m);  // the current device can hold one cluster of this shape
+bool qr_places(const QrShape& q, int s, int m);  // the current device can hold one cluster of this shape
 cudaError_t launch_inner_qr(const Plan& p, int i, cudaStream_t st);  // on stream st
 void launch_inner_finish(const Plan& p, double* z);  // y = R^{-1} d, z = sum_l y_l b_l (FP64)
 void launch_export_basis(const Plan& p, double* out, int count);  // out[l*N + r] = sigma_l * u_l[r] (FP64)

@@ -7,6 +7,7 @@
 namespace sfg {
 
 constexpr int kQrCluster = 16;   // most CTAs of the cluster that runs a sketched QR update
+constexpr int kQrThreads = 128;  // threads of such a CTA
 constexpr int kQrPortable = 8;   // the largest cluster that every device of the architecture places
 
 // Shape of the sketched-QR update.
@@ -20,6 +21,17 @@ struct QrShape {
 // Dynamic shared memory of update i: the staged columns, the CTA's rows of p and e, the projections and their parts.
 inline size_t qr_smem(const QrShape& q, int m, int i) {
     return ((size_t)(q.staged ? (i * q.nrp + 1) & ~1 : 0) + 2 * (size_t)q.nrp + 3 * (size_t)m) * sizeof(double);
+}
+
+// Whether a thread's part of one of update i's products (k_inner_qr: rows of a group, columns of a group) passes 16 terms.  Two
+// sums where the parts are short cost a 64^2 solve (8 terms) 1.5 %; where they are long, 0.5 % of an 80^3 cycle at s = 1000, m = 200, and
+// four sums 2.5 %.
+inline bool qr_long(int s, int cluster, int i) {
+    const int nr = (s + cluster - 1) / cluster;
+    int gp = 1, wr = 32;
+    while (gp < 8 && 2 * gp * i <= kQrThreads && 4 * gp <= nr) gp *= 2;
+    while (wr < nr && wr < kQrThreads) wr *= 2;
+    return (nr + gp - 1) / gp > 16 || (i * wr + kQrThreads - 1) / kQrThreads > 16;
 }
 
 // The shape for P problems, sketch size s and basis size m, given the shared memory a QR CTA may take; binned: the step's SpMV

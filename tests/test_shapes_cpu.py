@@ -30,6 +30,10 @@ int main() {
     line(1, 120, 30, big, 0, 0);
     line(16, 1000, 200, big, 0, 0);
     line(4, 400, 100, big, 8, 8);
+    for (int i : {0, 8, 16, 30}) std::printf("%d ", qr_long(120, 4, i));
+    for (int i : {1, 16, 32, 33, 59}) std::printf("%d ", qr_long(240, 4, i));
+    for (int i : {1, 16, 17, 99}) std::printf("%d ", qr_long(1000, 16, i));
+    std::printf("\n");
 }
 """
 
@@ -42,8 +46,11 @@ def test_clusters_fall_back_to_what_the_device_places(tmp_path):
     src.write_text(PROGRAM)
     r = subprocess.run([gxx, "-std=c++17", "-I", CSRC, "-o", str(exe), str(src)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
-    got = [tuple(map(int, ln.split())) for ln in
-           subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.splitlines()]
+    *got, parts = [tuple(map(int, ln.split())) for ln in
+                   subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.splitlines()]
+    # 64^2 (30 rows: at most 8 a group, 30 columns in four groups); 60 rows in 8, 4 or 2 groups, 59 columns in two; 63 rows in
+    # 8 groups up to 8 columns' worth of threads, then 4 (16 rows) and 2 (32 rows)
+    assert parts == (0, 0, 0, 0) + (0, 0, 0, 1, 1) + (0, 0, 0, 1)
     kind = [(c, st, asked) for c, st, _, _, asked, _ in got]
     assert kind == [(16, 1, 1),   # held as wanted
                     (16, 0, 2),   # not with its slice in shared memory: the same cluster, so the same sums, from L2

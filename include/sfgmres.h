@@ -75,7 +75,7 @@ extern "C" {
                                         per SM, of all SMs but 8 for medium systems, or at most 128 blocks for small
                                         ones, which leaves SMs to the sketched-QR update running beside; many
                                         right-hand sides of one system: 5120; several systems: 4096).  Reading it
-                                        returns the size in use. */
+                                        returns the size in use (the latest call's). */
 #define SFGMRES_OPT_GRAPH 10         /* 1 (default): each outer step (one inner cycle for every problem and the outer
                                         FGMRES update) is captured once into a CUDA graph and replayed; the graphs
                                         are kept while the solve's parameters and workspaces stay the same.  0: the

@@ -5,7 +5,8 @@ lambda = A^{-T} g solves the adjoint system, dL/db = lambda and dL/dA_ij = -lamb
 only.  Both the forward solves and the adjoint solves run in the CUDA library (sfgmres_solve, sfgmres_solve_transpose
 with the same sketch and parameters), and the pattern gradient is accumulated by sfgmres_pattern_outer.  Several
 right-hand sides (rows of b) are solved together as one batch (sfgmres_solve_batch, nrhs = rows of b): every row is
-still its own FGMRES problem with its own stop rules, and gets the result a separate solve would give.
+still its own FGMRES problem with its own stop rules, and gets the result a separate solve would give to rounding (the
+row blocks, and with them the order of block sums, follow the number of rows).
 """
 from __future__ import annotations
 

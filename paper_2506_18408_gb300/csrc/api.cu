@@ -394,9 +394,12 @@ void choose_lists(sfgmres_ctx* h, int nrhs) {
 // Shared memory that a sketched-QR CTA may take (6 to 8 KB per step CTA for its static shared memory and the reserve).  A
 // stencil's steps of one launch that fill the SMs do best with the QR staged, waiting for an SM that their CTAs leave, and not
 // beside two of them (128^3 solve FP64 46.8 ms against 54.0, FP32 42.0 against 54.7, 80^3 cycle at s = 1000 9.5 against 10.5).
-// The longer steps of the length-binned SpMV, and steps of two launches, would pay for that wait with a second wave of the
-// next SpMV on those SMs (2M Zipf rows, FP64: 494 us per step against 299; 1.5M, FP32: 318 against 179): there the QR
-// has to fit beside two CTAs, within the carveout that they chose, the smallest that holds them.
+// The longer steps of the length-binned SpMV would pay for that wait with a second wave of the next SpMV on those SMs (2M Zipf
+// rows, FP64: 494 us per step against 299; 1.5M, FP32: 318 against 179): there, and where the caller asks for two launches, the
+// QR has to fit beside two CTAs, within the carveout that they chose, the smallest that holds them.  A stencil's launches of several
+// waves (one system above 2.5M rows, batches, many right-hand sides) take either form within 1 or 2 %, and wait: cycles of
+// 100 steps at 140^3 / 160^3 / 180^3 FP64 15.0 / 19.9 / 29.0 ms and beside 14.8 / 19.7 / 28.8, FP32 9.6 / 13.1 / 19.0 and 9.7 / 13.0 / 19.1; 24 2D
+// systems x 4 FP32 109.3 and 110.2 ms, 64^3 x 16 forward and backward 131.4 and 134.6.
 size_t qr_smem_left(int nblk, int sms, size_t step_smem, bool beside) {
     constexpr size_t KB = 1024;
     if (nblk <= sms || !beside) {
@@ -1012,7 +1015,7 @@ int prepare(sfgmres_ctx* h, int nrhs, int m, int s, int t, int jmax, Plan* p, Ge
     if ((rc = ensure(h, h->cpart, nb * S * at))) return rc;
     if ((rc = ensure(h, h->C, Pn * M * S * 8))) return rc;
     const size_t stage = staged ? stage_smem(maxlen) : 0;
-    const bool beside = vec == 0 || t > 4 || !h->fuse_step;  // binned, or steps of two launches (launch_inner_step)
+    const bool beside = vec == 0 || t > 4 || !h->fuse_step;  // binned, or two launches by the caller's parameters
     const QrShape qs = qr_shape(g->P, s, m, qr_smem_left(g->nblk, h->sms, ((size_t)h->Bn + 1) * at + stage, beside), vec == 0,
                                 [&](const QrShape& q) {
                                     const size_t smem = qr_smem(q, m, m - 1);

@@ -408,7 +408,8 @@ void launch_final_x(const Plan& p, int J, const double* x0, double* x) {
     g_launches += 2;
 }
 
-// y = A x; staged entries: each block in pieces of kPlainRows rows (one CTA each, grid y), so that an SM holds four CTAs.
+// y = A x; staged entries: each block in pieces of kPlainRows rows (one CTA each, grid y), which come and go on the two CTAs of 64
+// registers a thread that an SM holds, so that their waits and ends do not fall together.
 constexpr int kPlainRows = 2048;
 template <int V, int U>
 __global__ void __launch_bounds__(512, 2)

@@ -409,7 +409,8 @@ __device__ __forceinline__ void sorted_row(const int* __restrict__ cp, const MT*
 // coalesced: every FP64 instruction does 32 rows' products and no sum needs a shuffle tree (with 8 lanes or a warp per row
 // the trees and half-empty passes doubled the FP64 instructions of a 2M-row Zipf matrix, on a GPU whose FP64 pipe takes 17
 // cycles per warp and instruction).  Warps take the slices longest first, in alternating direction, so that their loads
-// even out.  2M rows, FP64: 270 -> 235 us per launch; whole steps 1M rows 227 -> 164 us, 1.5M FP32 213 -> 179 us.
+// even out.  2M rows, FP64, one running sum per row: 270 -> 235 us per launch; whole steps 1M rows 227 -> 164 us, 1.5M FP32 213 ->
+// 179 us (sorted_row has what its order of sums costs beside that).
 // The rows that the copy leaves (too long for the block, or slices that would be half empty) take 8 lanes (up to 64 entries) or a
 // warp from the CSR arrays.  Every row's sum runs over its entries in a fixed order.
 template <typename MT, typename XT, typename AT>

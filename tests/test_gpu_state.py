@@ -99,3 +99,22 @@ def test_replay_after_row_blocks_were_rebuilt(Solver, kind):
     sv.set("spmv_vector", 0)
     assert np.array_equal(sv.solve(b, **PAR)[0].cpu().numpy(), want)
     sv.close()
+
+
+# Blocks of several waves, where every step is two launches: the QR staged in shared memory (it waits for an SM) and, beside the
+# steps the caller asks to split, read from L2 form the same sums, in cycles and solves.
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_blocks_of_several_waves(Solver, precision):
+    A = workloads.convdiff(150, (30.0, 10.0))
+    b = dev_vec(workloads.rhs(A.n, seed=4))
+    sv = Solver(A.n, A.row_ptr, A.col, A.val, sketch_seed=1, precision=precision, block_rows=32)
+    got = []
+    for fused in (1, 0):
+        sv.set("fused_step", fused)
+        z = sv.inner_cycle(b / b.norm(), m=100, s=400, k=2)[0].cpu().numpy()
+        x, info = sv.solve(b, m=100, s=400, k=2, tol=1e-8)
+        r = A.to_scipy() @ x.cpu().numpy() - b.cpu().numpy()
+        assert info["status"] == 0 and np.linalg.norm(r) <= 1.01e-8 * float(b.norm())
+        got.append((z, x.cpu().numpy()))
+    assert all(np.array_equal(p, q) for p, q in zip(*got))
+    sv.close()

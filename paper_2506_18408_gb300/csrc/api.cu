@@ -236,24 +236,31 @@ void drop_lists(ListSet& L) {
     L = ListSet();
 }
 
+// Device memory for the handle; the list blocks that are only kept for later calls make room where it would not fit.
+template <typename T>
+cudaError_t dev_alloc(sfgmres_ctx* h, T** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && !h->kept.empty()) {
+        for (ListSet& L : h->kept) drop_lists(L);
+        h->kept.clear();
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+    }
+    return e;
+}
+
 int ensure(sfgmres_ctx* h, DevBuf& b, size_t bytes) {
     bytes = std::max<size_t>(bytes, 16);
     if (b.bytes >= bytes) return 0;
     if (b.p) cudaFree(b.p);
     b.p = nullptr;
     b.bytes = 0;
-    cudaError_t e = cudaMalloc(&b.p, bytes);
-    if (e != cudaSuccess && !h->kept.empty()) {  // the list blocks that are only kept for later calls make room
-        cudaGetLastError();
-        for (ListSet& L : h->kept) drop_lists(L);
-        h->kept.clear();
-        e = cudaMalloc(&b.p, bytes);
-    }
-    if (e != cudaSuccess) {
-        b.p = nullptr;
-        cudaGetLastError();
+    if (dev_alloc(h, &b.p, bytes) != cudaSuccess)
         return fail(h, SFGMRES_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
-    }
     b.bytes = bytes;
     return 0;
 }
@@ -531,11 +538,11 @@ int build_sketch(sfgmres_ctx* h, int s) {
     int* counts = nullptr;
     int* units = nullptr;
     const int64_t tq = (int64_t)maxn * zeta;
-    CK(cudaMalloc(&rows, tq * sizeof(int)));
-    CK(cudaMalloc(&neg, tq));
-    CK(cudaMalloc(&counts, ncnt * sizeof(int)));
-    CK(cudaMalloc(&units, nseg * sizeof(int)));
-    CK(cudaMalloc(&h->seg, nseg * sizeof(int)));
+    CK(dev_alloc(h, &rows, tq * sizeof(int)));
+    CK(dev_alloc(h, &neg, tq));
+    CK(dev_alloc(h, &counts, ncnt * sizeof(int)));
+    CK(dev_alloc(h, &units, nseg * sizeof(int)));
+    CK(dev_alloc(h, &h->seg, nseg * sizeof(int)));
     CK(cudaMemsetAsync(counts, 0, ncnt * sizeof(int), h->st));
     for (int q = 0; q < h->nsys; ++q) {
         launch_sketch_pattern(h->sys_n[q], s, zeta, h->kind, h->seed, rows, neg, h->st);
@@ -549,7 +556,7 @@ int build_sketch(sfgmres_ctx* h, int s) {
     const int64_t total = (int64_t)hs[nseg - 1] * 8;  // entries
     if (hs[nseg - 1] < 0 || total >= ((int64_t)1 << 34))
         return fail(h, SFGMRES_ERR_INVALID_ARG, "sketch too large for 32-bit gather lists");
-    CK(cudaMalloc(&h->ent, std::max<int64_t>(total, 8) * sizeof(uint16_t)));
+    CK(dev_alloc(h, &h->ent, std::max<int64_t>(total, 8) * sizeof(uint16_t)));
     h->n_ent = total;
     launch_fill_u16(total, (uint16_t)h->Bn, h->ent, h->st);  // padding points at the zero slot
     for (int q = 0; q < h->nsys; ++q) {
@@ -640,7 +647,7 @@ int get_geometry(sfgmres_ctx* h, int nrhs, Geo** out) {
 int ensure_f32(sfgmres_ctx* h, bool transpose) {
     float*& v32 = transpose ? h->val32T : h->val32;
     if (v32) return 0;
-    CK(cudaMalloc(&v32, (h->nnz + kEntryPad) * sizeof(float)));
+    CK(dev_alloc(h, &v32, (h->nnz + kEntryPad) * sizeof(float)));
     k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, transpose ? h->valT : h->val, v32);
     CK(cudaGetLastError());
     return 0;
@@ -654,12 +661,12 @@ int ensure_transpose(sfgmres_ctx* h) {
     const int64_t nz = h->nnz + kEntryPad;
     int* counts = nullptr;
     int* mx = nullptr;
-    CK(cudaMalloc(&h->rpT, ((size_t)h->n + 1) * sizeof(int)));
-    CK(cudaMalloc(&h->colT, nz * sizeof(int)));
-    CK(cudaMalloc(&h->srcT, nz * sizeof(int)));
-    CK(cudaMalloc(&h->valT, nz * sizeof(double)));
-    CK(cudaMalloc(&counts, (size_t)h->n * sizeof(int)));
-    CK(cudaMalloc(&mx, sizeof(int)));
+    CK(dev_alloc(h, &h->rpT, ((size_t)h->n + 1) * sizeof(int)));
+    CK(dev_alloc(h, &h->colT, nz * sizeof(int)));
+    CK(dev_alloc(h, &h->srcT, nz * sizeof(int)));
+    CK(dev_alloc(h, &h->valT, nz * sizeof(double)));
+    CK(dev_alloc(h, &counts, (size_t)h->n * sizeof(int)));
+    CK(dev_alloc(h, &mx, sizeof(int)));
     CK(cudaMemsetAsync(counts, 0, (size_t)h->n * sizeof(int), h->st));
     CK(cudaMemsetAsync(mx, 0, sizeof(int), h->st));
     launch_transpose(h->n, h->nnz, h->rp, h->col, counts, h->rpT, h->colT, h->srcT, mx, h->st);
@@ -688,14 +695,14 @@ int ensure_bins(sfgmres_ctx* h, bool transpose) {
                 hb[h->nl + L] = std::min(Bq, nq - k * Bq);
             }
         }
-        CK(cudaMalloc(&h->lb, hb.size() * sizeof(int)));
+        CK(dev_alloc(h, &h->lb, hb.size() * sizeof(int)));
         CK(cudaMemcpy(h->lb, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice));
         h->lb_ver = h->geo_ver;
     }
-    if (!h->perm[t]) CK(cudaMalloc(&h->perm[t], std::max<size_t>(h->n, 1) * sizeof(uint16_t)));
+    if (!h->perm[t]) CK(dev_alloc(h, &h->perm[t], std::max<size_t>(h->n, 1) * sizeof(uint16_t)));
     if (h->cls[t]) cudaFree(h->cls[t]);
     h->cls[t] = nullptr;
-    CK(cudaMalloc(&h->cls[t], 2 * (size_t)h->nl * sizeof(int)));
+    CK(dev_alloc(h, &h->cls[t], 2 * (size_t)h->nl * sizeof(int)));
     launch_bin_rows(h->nl, transpose ? h->rpT : h->rp, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->st);
     CK(cudaGetLastError());
     h->bins_ver[t] = h->geo_ver;
@@ -715,7 +722,7 @@ int ensure_slices(sfgmres_ctx* h) {
         if (ns > INT32_MAX - 1) return fail(h, SFGMRES_ERR_INVALID_ARG, "too many rows for slices of 32");
         t[h->nsys] = (int)ns;
         for (int q = 0; q <= h->nsys; ++q) t[h->nsys + 1 + q] = h->sys_moff[q];
-        CK(cudaMalloc(&h->sl_sys, t.size() * sizeof(int)));
+        CK(dev_alloc(h, &h->sl_sys, t.size() * sizeof(int)));
         CK(cudaMemcpy(h->sl_sys, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice));
         h->sl_ns = (int)ns;
     }
@@ -729,7 +736,7 @@ int ensure_slices(sfgmres_ctx* h) {
         }
         if (h->sl_base) cudaFree(h->sl_base);
         h->sl_base = nullptr;
-        CK(cudaMalloc(&h->sl_base, hb.size() * sizeof(int)));
+        CK(dev_alloc(h, &h->sl_base, hb.size() * sizeof(int)));
         CK(cudaMemcpy(h->sl_base, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice));
         h->sl_base_ver = h->geo_ver;
     }
@@ -752,9 +759,9 @@ int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {
     if (fresh) {
         drop_sorted(S);  // what a failed build left
         int* wid = nullptr;
-        CK(cudaMalloc(&wid, std::max<size_t>((size_t)ns, 1) * sizeof(int)));
-        CK(cudaMalloc(&S.off, ((size_t)ns + 1) * sizeof(int)));
-        CK(cudaMalloc(&S.len, std::max<size_t>((size_t)ns, 1) * 32 * sizeof(uint16_t)));
+        CK(dev_alloc(h, &wid, std::max<size_t>((size_t)ns, 1) * sizeof(int)));
+        CK(dev_alloc(h, &S.off, ((size_t)ns + 1) * sizeof(int)));
+        CK(dev_alloc(h, &S.len, std::max<size_t>((size_t)ns, 1) * 32 * sizeof(uint16_t)));
         launch_sorted_build(h->nl, ns, rp, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->sl_base, S.len, wid, S.off,
                             h->st);
         int tot = 0;
@@ -763,10 +770,10 @@ int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {
         cudaFree(wid);
         CK(cudaGetLastError());
         S.total = std::max<int64_t>((int64_t)tot * 32, 1);
-        CK(cudaMalloc(&S.col, S.total * sizeof(int)));
-        CK(cudaMalloc(&S.val, S.total * sizeof(double)));
+        CK(dev_alloc(h, &S.col, S.total * sizeof(int)));
+        CK(dev_alloc(h, &S.val, S.total * sizeof(double)));
     }
-    if (f32 && !S.val32) CK(cudaMalloc(&S.val32, S.total * sizeof(float)));
+    if (f32 && !S.val32) CK(dev_alloc(h, &S.val32, S.total * sizeof(float)));
     launch_sorted_fill(h->nl, rp, col, val, h->lb, h->lb + h->nl, h->perm[t], h->cls[t], h->sl_base, S.off,
                        fresh ? S.col : nullptr, S.val, S.val32, h->st);
     CK(cudaGetLastError());
@@ -789,9 +796,9 @@ int ensure_sell(sfgmres_ctx* h, bool transpose) {
     const int* moff = h->sl_sys + h->nsys + 1;
     if (!S.off) {
         int* wid = nullptr;
-        CK(cudaMalloc(&S.off, ((size_t)ns + 1) * sizeof(int)));
-        CK(cudaMalloc(&S.len, std::max<size_t>((size_t)ns * 32, 1)));
-        CK(cudaMalloc(&wid, std::max<size_t>((size_t)ns, 1) * sizeof(int)));
+        CK(dev_alloc(h, &S.off, ((size_t)ns + 1) * sizeof(int)));
+        CK(dev_alloc(h, &S.len, std::max<size_t>((size_t)ns * 32, 1)));
+        CK(dev_alloc(h, &wid, std::max<size_t>((size_t)ns, 1) * sizeof(int)));
         launch_sell_build(ns, sl0, h->nsys, moff, rp, S.len, wid, S.off, h->st);
         int tot = 0;
         CK(cudaMemcpyAsync(&tot, S.off + ns, sizeof(int), cudaMemcpyDeviceToHost, h->st));
@@ -799,8 +806,8 @@ int ensure_sell(sfgmres_ctx* h, bool transpose) {
         cudaFree(wid);
         CK(cudaGetLastError());
         S.total = (int64_t)tot * 32;
-        CK(cudaMalloc(&S.col, std::max<int64_t>(S.total, 1) * sizeof(int)));
-        CK(cudaMalloc(&S.val, std::max<int64_t>(S.total, 1) * sizeof(double)));
+        CK(dev_alloc(h, &S.col, std::max<int64_t>(S.total, 1) * sizeof(int)));
+        CK(dev_alloc(h, &S.val, std::max<int64_t>(S.total, 1) * sizeof(double)));
         launch_sell_fill(ns, sl0, h->nsys, moff, rp, col, val, S.off, S.len, S.col, S.val, h->st);
         CK(cudaGetLastError());
     }
@@ -2525,7 +2532,7 @@ int sfgmres_sketch_pattern(sfgmres_t h, int32_t s, int32_t* rows, int8_t* signs)
     CK(cudaSetDevice(h->dev));
     const int zeta = (h->kind == 1) ? 1 : h->zeta;
     int8_t* neg = nullptr;
-    CK(cudaMalloc(&neg, (size_t)h->n * zeta));
+    CK(dev_alloc(h, &neg, (size_t)h->n * zeta));
     launch_sketch_pattern(h->n, s, zeta, h->kind, h->seed, rows, neg, h->st);
     const int64_t cnt = (int64_t)h->n * zeta;
     k_neg_to_sign<<<grid_for(cnt), 256, 0, h->st>>>(cnt, neg, signs);

@@ -657,16 +657,28 @@ int ensure_f32(sfgmres_ctx* h, bool transpose) {
 // transpose of the block-diagonal matrix is block-diagonal with the same blocks, so the row-block geometry and the
 // sketch lists serve both.
 int ensure_transpose(sfgmres_ctx* h) {
-    if (h->rpT) return 0;
+    if (h->valT) return 0;  // allocated last: set only when the rest is there
     const int64_t nz = h->nnz + kEntryPad;
-    int* counts = nullptr;
-    int* mx = nullptr;
-    CK(dev_alloc(h, &h->rpT, ((size_t)h->n + 1) * sizeof(int)));
-    CK(dev_alloc(h, &h->colT, nz * sizeof(int)));
-    CK(dev_alloc(h, &h->srcT, nz * sizeof(int)));
-    CK(dev_alloc(h, &h->valT, nz * sizeof(double)));
-    CK(dev_alloc(h, &counts, (size_t)h->n * sizeof(int)));
-    CK(dev_alloc(h, &mx, sizeof(int)));
+    for (int** q : {&h->rpT, &h->colT, &h->srcT}) {  // what a failed build left
+        if (*q) cudaFree(*q);
+        *q = nullptr;
+    }
+    DevBuf tmp;  // [n] counts, then the longest row
+    int rc = ensure(h, tmp, ((size_t)h->n + 1) * sizeof(int));
+    if (rc) return rc;
+    auto members = [&]() -> int {
+        CK(dev_alloc(h, &h->rpT, ((size_t)h->n + 1) * sizeof(int)));
+        CK(dev_alloc(h, &h->colT, nz * sizeof(int)));
+        CK(dev_alloc(h, &h->srcT, nz * sizeof(int)));
+        CK(dev_alloc(h, &h->valT, nz * sizeof(double)));
+        return 0;
+    };
+    if ((rc = members())) {
+        release(tmp);
+        return rc;
+    }
+    int* counts = (int*)tmp.p;
+    int* mx = counts + h->n;
     CK(cudaMemsetAsync(counts, 0, (size_t)h->n * sizeof(int), h->st));
     CK(cudaMemsetAsync(mx, 0, sizeof(int), h->st));
     launch_transpose(h->n, h->nnz, h->rp, h->col, counts, h->rpT, h->colT, h->srcT, mx, h->st);
@@ -674,8 +686,7 @@ int ensure_transpose(sfgmres_ctx* h) {
     CK(cudaMemcpyAsync(&h->maxlenT, mx, sizeof(int), cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));
     CK(cudaGetLastError());
-    cudaFree(counts);
-    cudaFree(mx);
+    release(tmp);
     h->vecT = choose_vec(h->nnz, h->n, h->maxlenT);
     return 0;
 }
@@ -794,7 +805,10 @@ int ensure_sell(sfgmres_ctx* h, bool transpose) {
     const int ns = h->sl_ns;
     const int* sl0 = h->sl_sys;
     const int* moff = h->sl_sys + h->nsys + 1;
-    if (!S.off) {
+    if (!S.val) {  // allocated last: set only when the rest is there
+        for (void* q : {(void*)S.off, (void*)S.len, (void*)S.col})  // what a failed build left
+            if (q) cudaFree(q);
+        S = sfgmres_ctx::Sell();
         int* wid = nullptr;
         CK(dev_alloc(h, &S.off, ((size_t)ns + 1) * sizeof(int)));
         CK(dev_alloc(h, &S.len, std::max<size_t>((size_t)ns * 32, 1)));
@@ -834,7 +848,7 @@ void plan_geometry(sfgmres_ctx* h, const Geo* g, bool transpose, Plan& P) {
     P.so_val32 = so ? O.val32 : nullptr;
     P.so_base = so ? h->sl_base : nullptr;
     const sfgmres_ctx::Sell& S = h->sell[transpose ? 1 : 0];
-    const bool sl = (P.vec == 1) && h->prec == kFP64 && S.off && h->sl_base_ver == h->geo_ver;
+    const bool sl = (P.vec == 1) && h->prec == kFP64 && S.val && h->sl_base_ver == h->geo_ver;
     P.sl_off = sl ? S.off : nullptr;
     P.sl_len = sl ? S.len : nullptr;
     P.sl_col = sl ? S.col : nullptr;
@@ -2042,7 +2056,7 @@ int sfgmres_update_values(sfgmres_t h, const double* vals) {
                        is_device_ptr(vals) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
     ++h->vals_ver;  // the ILU(0) factors (if any) are recomputed at their next use
     if (h->val32) k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, h->val, h->val32);
-    if (h->rpT) {
+    if (h->valT) {
         launch_gather_vals(h->nnz, h->srcT, h->val, h->valT, h->st);
         if (h->val32T) k_to_f32<<<grid_for(h->nnz), 256, 0, h->st>>>(h->nnz, h->valT, h->val32T);
     }
@@ -2055,7 +2069,7 @@ int sfgmres_update_values(sfgmres_t h, const double* vals) {
     }
     for (int t = 0; t < 2; ++t) {  // the SELL-32 copies' values
         sfgmres_ctx::Sell& S = h->sell[t];
-        if (!S.off) continue;
+        if (!S.val) continue;
         launch_sell_fill(h->sl_ns, h->sl_sys, h->nsys, h->sl_sys + h->nsys + 1, t ? h->rpT : h->rp, nullptr,
                          t ? h->valT : h->val, S.off, S.len, nullptr, S.val, h->st);
     }

@@ -25,3 +25,13 @@ def test_plan_key_holds_every_pointer_of_the_plan():
 
 def test_plan_key_holds_the_version_of_the_list_blocks():
     assert "h->geo_ver" in _body("api.cu", "std::vector<uint64_t> plan_key(", "\n}\n")
+
+
+def test_copies_are_marked_as_built_by_their_last_allocation():
+    """A build that runs out of memory half way is taken up again by the next call, not read through null pointers."""
+    body = _body("api.cu", "int ensure_transpose(sfgmres_ctx* h) {", "\n}\n")
+    assert re.search(r"if \(h->(\w+)\) return 0;", body).group(1) == re.findall(r"dev_alloc\(h, &h->(\w+),", body)[-1]
+    body = _body("api.cu", "int ensure_sell(sfgmres_ctx* h, bool transpose) {", "\n}\n")
+    assert re.search(r"if \(!S\.(\w+)\) \{", body).group(1) == re.findall(r"dev_alloc\(h, &S\.(\w+),", body)[-1]
+    body = _body("api.cu", "int ensure_sorted(sfgmres_ctx* h, bool transpose, bool f32) {", "\n}\n")
+    assert body.rindex("S.ver = h->vals_ver;") > body.rindex("dev_alloc(")
